@@ -12,6 +12,7 @@
 #include <cuda_runtime.h>
 #include <math.h>
 
+#include "solve_scalars.cuh"
 #include "svt_internal.h"
 
 namespace svt {
@@ -22,18 +23,6 @@ __device__ __forceinline__ void set_status(int *status, svt_status s)
 {
     if (status)
         atomicCAS(status, 0, (int)s);
-}
-
-// alpha = 2^e with e = round(log2 ||A||_F) (1 for a zero matrix): dividing by it is exact.
-__device__ __forceinline__ double pow2_alpha(double nrm2)
-{
-    if (!(nrm2 > 0.0) || !isfinite(nrm2))
-        return 1.0;
-    int e;
-    double f = frexp(sqrt(nrm2), &e);  // sqrt = f 2^e, f in [0.5, 1)
-    if (f < 0.70710678118654752)
-        e -= 1;
-    return ldexp(1.0, e);
 }
 
 // ---- ingest: column (or row) norms and the split into scaled copies

@@ -16,6 +16,7 @@
 
 #include <nvtx3/nvToolsExt.h>
 
+#include "small_solve.h"
 #include "svt_internal.h"
 
 namespace svt {
@@ -151,7 +152,13 @@ struct Plan {
     int force_bn = 0;               // 0: tile width per launch; 128 / 256: fixed (grouped batches);
                                     // -1: per-launch widths from bn_choice (autotuned)
     std::vector<int> bn_choice;     // tile width of each product launch (autotuned plans)
+    // One-launch solve of a one-tile matrix (kSmallPlan): no product table, no workspace.
+    bool small = false;
+    SmallSolve small_args;          // all but the call's pointers, strides and tau
 };
+
+// force_bn code of the plans that run as one small_solve launch.
+constexpr int kSmallPlan = 1;
 
 // Autotuned tile widths of one (shape, options): one entry per product launch.
 struct TuneKey {

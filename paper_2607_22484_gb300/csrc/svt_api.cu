@@ -288,6 +288,25 @@ Layout make_layout(int64_t m, int64_t n, const Resolved &r)
 namespace svt {
 namespace {
 
+// Leading S-chain steps that run in the FP32-class tier: all of them in the FP32 tier; in
+// the BF16 tier the first hp_steps (auto: the steps whose design interval starts below 0.1,
+// while the shifted Gram's small eigenvalues are still below BF16 resolution relative to the
+// largest). lo: the lower end of each step's design interval.
+int hp_steps_of(const Resolved &o, const std::vector<double> &lo)
+{
+    if (o.prec == SVT_FP32)
+        return o.iters;
+    if (o.prec != SVT_BF16)
+        return 0;
+    if (o.hp_steps >= 0)
+        return std::min(o.hp_steps, o.iters);
+    int hp = 0;
+    for (int t = 0; t < o.iters; ++t)
+        if (lo[t] < 0.1)
+            hp = t + 1;
+    return hp;
+}
+
 // ---------------------------------------------------------- plan builder
 
 struct Builder {
@@ -502,22 +521,7 @@ struct Builder {
         const bool pairs = o.prec == SVT_FP32;
         const bool skipP = o.mode == SVT_MODE_RANK_R;
         const int M = (int)L.M, N = (int)L.N;
-        // Leading S-chain steps run in the FP32-class tier: all of them in the FP32
-        // tier; in the BF16 tier the first hp_steps (auto: the steps whose design
-        // interval starts below 0.1, while the shifted Gram's small eigenvalues are
-        // still below BF16 resolution relative to the largest).
-        int hpS = 0;
-        if (pairs) {
-            hpS = o.iters;
-        } else if (o.prec == SVT_BF16) {
-            if (o.hp_steps >= 0) {
-                hpS = std::min(o.hp_steps, o.iters);
-            } else {
-                for (int t = 0; t < o.iters; ++t)
-                    if (P.lo[t] < 0.1)
-                        hpS = t + 1;
-            }
-        }
+        const int hpS = hp_steps_of(o, P.lo);
         // S after t steps is a pair iff step t (its consumer) runs FP32-class.
         auto s_pair = [&](int t) { return pairs || t < hpS; };
         P.hp_steps_s = hpS;
@@ -823,6 +827,22 @@ __global__ void prep_kernel(const float *__restrict__ A, int64_t lda, int wide, 
 
 } // namespace
 
+// Event pair around one product launch (svt_ctx_profile).
+static svt_status profile_events(svt_ctx *ctx, cudaEvent_t *e0, cudaEvent_t *e1)
+{
+    if (ctx->prof_next + 2 > ctx->prof_pool.size()) {
+        for (int k = 0; k < 64; ++k) {
+            cudaEvent_t ev;
+            if (cudaEventCreate(&ev) != cudaSuccess)
+                return SVT_ERR_CUDA;
+            ctx->prof_pool.push_back(ev);
+        }
+    }
+    *e0 = ctx->prof_pool[ctx->prof_next++];
+    *e1 = ctx->prof_pool[ctx->prof_next++];
+    return SVT_OK;
+}
+
 svt_status run_ops(svt_ctx *ctx, Plan &P, const CallArgs &a, cudaStream_t s, size_t first,
                    size_t last, int sms)
 {
@@ -861,16 +881,8 @@ svt_status run_ops(svt_ctx *ctx, Plan &P, const CallArgs &a, cudaStream_t s, siz
             l.call_inline.d_status = a.d_status;
             cudaEvent_t e0 = nullptr, e1 = nullptr;
             if (prof) {
-                if (ctx->prof_next + 2 > ctx->prof_pool.size()) {
-                    for (int k = 0; k < 64; ++k) {
-                        cudaEvent_t ev;
-                        if (cudaEventCreate(&ev) != cudaSuccess)
-                            return SVT_ERR_CUDA;
-                        ctx->prof_pool.push_back(ev);
-                    }
-                }
-                e0 = ctx->prof_pool[ctx->prof_next++];
-                e1 = ctx->prof_pool[ctx->prof_next++];
+                if (profile_events(ctx, &e0, &e1) != SVT_OK)
+                    return SVT_ERR_CUDA;
                 cudaEventRecord(e0, s);
             }
             err = tc_gemm_launch_fused(l, P.fused_bn, P.fused_tiles, grid_sms, s, P.uses_strips);
@@ -932,16 +944,8 @@ svt_status run_ops(svt_ctx *ctx, Plan &P, const CallArgs &a, cudaStream_t s, siz
                 }
             cudaEvent_t e0 = nullptr, e1 = nullptr;
             if (prof) {
-                if (ctx->prof_next + 2 > ctx->prof_pool.size()) {
-                    for (int k = 0; k < 64; ++k) {
-                        cudaEvent_t ev;
-                        if (cudaEventCreate(&ev) != cudaSuccess)
-                            return SVT_ERR_CUDA;
-                        ctx->prof_pool.push_back(ev);
-                    }
-                }
-                e0 = ctx->prof_pool[ctx->prof_next++];
-                e1 = ctx->prof_pool[ctx->prof_next++];
+                if (profile_events(ctx, &e0, &e1) != SVT_OK)
+                    return SVT_ERR_CUDA;
                 cudaEventRecord(e0, s);
             }
             err = tc_gemm_launch(l, op.bn, grid_sms, s);
@@ -1010,8 +1014,38 @@ svt_status upload_fused_table(svt_ctx *ctx, Plan &P, cudaStream_t s)
                : SVT_ERR_CUDA;
 }
 
+// A one-tile solve: one launch, nothing in the workspace.
+static svt_status run_small(svt_ctx *ctx, Plan &P, const CallArgs &a, cudaStream_t s)
+{
+    SmallSolve q = P.small_args;
+    q.A = a.A;
+    q.lda = a.lda;
+    q.Y = a.Y;
+    q.ldy = a.ldy;
+    q.tau = a.tau;
+    q.d_status = a.d_status;
+    const bool prof = ctx->profile && !a.in_graph;
+    cudaEvent_t e0 = nullptr, e1 = nullptr;
+    if (prof) {
+        if (profile_events(ctx, &e0, &e1) != SVT_OK)
+            return SVT_ERR_CUDA;
+        cudaEventRecord(e0, s);
+    }
+    if (small_solve_launch(q, s) != cudaSuccess)
+        return SVT_ERR_CUDA;
+    if (prof) {
+        cudaEventRecord(e1, s);
+        ctx->prof_pending.push_back({e0, e1, P.fused_flops, P.fused_tensor_flops});
+    }
+    if (!a.in_graph)
+        ctx->launches += 1;
+    return SVT_OK;
+}
+
 svt_status run_plan(svt_ctx *ctx, Plan &P, const CallArgs &a, cudaStream_t s, int sms)
 {
+    if (P.small)
+        return run_small(ctx, P, a, s);
     return run_ops(ctx, P, a, s, 0, P.ops.size(), sms);
 }
 
@@ -1267,6 +1301,29 @@ svt_status get_plan(svt_ctx *ctx, int64_t m, int64_t n, const Resolved &r, size_
     if (schedule_coeffs(r.schedule, r.iters, r.ell0, r.delta, plan->coef.data(),
                         plan->lo.data()) != 0)
         return SVT_ERR_INVALID;
+    if (force_bn == kSmallPlan) {
+        plan->small = true;
+        SmallSolve &q = plan->small_args;
+        std::memset(&q, 0, sizeof(q));
+        q.m = (int)m;
+        q.n = (int)n;
+        q.pairs = r.prec == SVT_FP32;
+        q.rank_r = r.mode == SVT_MODE_RANK_R;
+        q.iters = r.iters;
+        q.hp_steps = hp_steps_of(r, plan->lo);
+        q.norm_fro = r.norm == SVT_NORM_FRO;
+        q.cubic = r.schedule == SVT_SCHED_NS3;
+        for (int i = 0; i < 3 * r.iters; ++i)
+            q.coef[i] = (float)plan->coef[i];
+        for (int i = 0; i < 3; ++i)
+            q.first[i] = plan->coef[i];
+        small_solve_flops(q, &plan->fused_flops, &plan->fused_tensor_flops);
+        *out = plan.get();
+        if (keep)
+            *keep = plan;
+        ctx->plans[k] = std::move(plan);
+        return SVT_OK;
+    }
     Builder b{ctx, plan.get(), ctx->ws + ws_base, 256};
     if (!b.build())
         return SVT_ERR_CUDA;
@@ -1279,10 +1336,25 @@ svt_status get_plan(svt_ctx *ctx, int64_t m, int64_t n, const Resolved &r, size_
     return SVT_OK;
 }
 
+// Whether a solve runs as one small_solve launch: both sides within one tile, the default
+// pipeline on tensor cores (fused, polished, no e4m3 steps), no tile mode asked for and no
+// shortened dependency wait (that launch waits on no other tile). One tile is its limit: three
+// regions of 128 x 128 hi/lo pairs fill a CTA's shared memory. At 128 x 128 it takes 131 us
+// (BF16 tier, 20 steps) where the general launches take about 440, and the gap only widens
+// below, so there is no lower bound.
+static bool use_small(const svt_ctx *ctx, int64_t m, int64_t n, const Resolved &r)
+{
+    return std::max(m, n) <= kSmallDim && r.prec != SVT_FP64 && r.fuse && r.polish && !r.tile &&
+           r.iters <= kSmallIters && !r.fp8_p && !r.fp8_s && !ctx->dbg_wait_ns;
+}
+
 svt_status plan_for_solve(svt_ctx *ctx, int64_t m, int64_t n, const Resolved &r, Plan **out,
                           std::shared_ptr<Plan> *keep)
 {
-    const int fbn = r.tile ? r.tile : (ctx->tuning.count(tune_key(m, n, r)) ? -1 : 0);
+    const int fbn = r.tile ? r.tile
+                           : (use_small(ctx, m, n, r)
+                                  ? kSmallPlan
+                                  : (ctx->tuning.count(tune_key(m, n, r)) ? -1 : 0));
     return get_plan(ctx, m, n, r, 0, ctx->ws_bytes, out, fbn, keep);
 }
 
