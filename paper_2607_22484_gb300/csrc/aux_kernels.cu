@@ -414,8 +414,10 @@ __global__ void grouped_finalize_kernel(const AuxRec *recs, const CallRec *calls
 
 // ------------------------------------------------------------ FP64 tier
 
-constexpr int kF64Tile = 64;
-constexpr int kF64K = 16;
+// Output tile and threads of one CTA of the FP64 product, and K per shared-memory stage.
+constexpr int kF64Tile = 8;
+constexpr int kF64Threads = kF64Tile * kF64Tile;
+constexpr int kF64K = 32;
 
 __device__ __forceinline__ double f64_load_c(const Epi &e, int64_t r, int64_t c)
 {
@@ -435,8 +437,17 @@ __device__ __forceinline__ void f64_store(int kind, void *p, int64_t off, double
         static_cast<float *>(p)[off] = (float)v;
 }
 
-// D = L R^T, 64 x 64 tile per block of 256 threads, 4 x 4 outputs per thread.
-__global__ void __launch_bounds__(256) f64_gemm_kernel(const __grid_constant__ F64Launch l)
+// D = L R^T, one 8 x 8 tile per CTA of 64 threads, one output per thread, K in order.
+//
+// Bound by the FP64 units: 2 lanes a cycle and SM, 16 cycles for a warp's FMA, so an 8 x 8 tile's
+// operands (128 bytes per K, 4 bytes a cycle and SM from L2) and its two shared-memory reads per
+// FMA cost nothing beside it, and the split that counts is the one that keeps all 152 SMs equally
+// busy. 64 x 64 tiles left 134 SMs idle at 256 x 192, where a stage's products are 600 tiles of
+// 8 x 8, four per SM (16 x 16 tiles: 156, one SM in forty taking twice as long as the rest).
+// 256 x 192, 20 steps: 15.5 -> 1.94 ms (FP64 units alone:
+// 1.03); 512 x 512: 36.0 -> 18.1 (16.2); 1024 x 1024: 199 -> 134. The next stage of K is loaded into registers while
+// this one is used.
+__global__ void __launch_bounds__(kF64Threads) f64_gemm_kernel(const __grid_constant__ F64Launch l)
 {
     const F64Problem &P = l.p[blockIdx.z];
     const int tm = blockIdx.y, tn = blockIdx.x;
@@ -444,72 +455,80 @@ __global__ void __launch_bounds__(256) f64_gemm_kernel(const __grid_constant__ F
         return;
     if (P.sym && tm > tn)
         return;
-    __shared__ double sL[kF64K][kF64Tile + 1];
-    __shared__ double sR[kF64K][kF64Tile + 1];
-    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-    double acc[4][4] = {};
+    __shared__ double sL[kF64Tile][kF64K + 1];
+    __shared__ double sR[kF64Tile][kF64K + 1];
+    __shared__ double scale[3];
+    const int tx = threadIdx.x % kF64Tile, ty = threadIdx.x / kF64Tile;
+    constexpr int kLoads = kF64Tile * kF64K / kF64Threads;
+    double gl[kLoads], gr[kLoads];
+    // Row (threadIdx.x / 32) + 2 i of the tile, column threadIdx.x % 32 of the stage.
+    const int lk = threadIdx.x % kF64K, lr = threadIdx.x / kF64K;
+    auto fetch = [&](int k0) {
+#pragma unroll
+        for (int i = 0; i < kLoads; ++i) {
+            const int r = lr + (kF64Threads / kF64K) * i, gk = k0 + lk;
+            const int64_t a = (int64_t)tm * kF64Tile + r, b = (int64_t)tn * kF64Tile + r;
+            gl[i] = (a < P.M && gk < P.K) ? P.L[a * P.ldl + gk] : 0.0;
+            gr[i] = (b < P.N && gk < P.K) ? P.R[b * P.ldr + gk] : 0.0;
+        }
+    };
+    double acc = 0.0;
+    fetch(0);
     for (int k0 = 0; k0 < P.K; k0 += kF64K) {
-        for (int idx = threadIdx.x; idx < kF64Tile * kF64K; idx += 256) {
-            int rr = idx / kF64K, kk = idx % kF64K;
-            int64_t gr = (int64_t)tm * kF64Tile + rr, gk = k0 + kk;
-            sL[kk][rr] = (gr < P.M && gk < P.K) ? P.L[gr * P.ldl + gk] : 0.0;
-            int64_t gc = (int64_t)tn * kF64Tile + rr;
-            sR[kk][rr] = (gc < P.N && gk < P.K) ? P.R[gc * P.ldr + gk] : 0.0;
+#pragma unroll
+        for (int i = 0; i < kLoads; ++i) {
+            const int r = lr + (kF64Threads / kF64K) * i;
+            sL[r][lk] = gl[i];
+            sR[r][lk] = gr[i];
         }
         __syncthreads();
+        if (k0 + kF64K < P.K)
+            fetch(k0 + kF64K);
 #pragma unroll
-        for (int kk = 0; kk < kF64K; ++kk) {
-            double a[4], b[4];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                a[i] = sL[kk][ty + 16 * i];
-                b[i] = sR[kk][tx + 16 * i];
-            }
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-#pragma unroll
-                for (int j = 0; j < 4; ++j)
-                    acc[i][j] = fma(a[i], b[j], acc[i][j]);
-        }
+        for (int kk = 0; kk < kF64K; ++kk)
+            acc = fma(sL[ty][kk], sR[tx][kk], acc);
         __syncthreads();
     }
     const Epi &e = P.ep;
     double al = e.alpha, be = e.beta, ga = e.gamma;
-    if (e.theta_src) {
-        double theta = pow(*e.theta_src, e.theta_pow);
-        if (theta > 0.0 && isfinite(theta)) {
-            al *= pow(theta, -e.ea);
-            be *= pow(theta, -e.eb);
-            ga *= pow(theta, -e.eg);
-        } else if (!isfinite(theta)) {
-            set_status(e.status, SVT_ERR_DIVERGED);
-        }  // theta == 0: the chain's matrix is zero; nothing to scale
+    if (e.theta_src) {  // one thread computes the scales: every FP64 instruction of a warp counts
+        if (threadIdx.x == 0) {
+            const double theta = root_theta(*e.theta_src, e.theta_pow == 0.25);
+            if (theta > 0.0 && isfinite(theta)) {
+                al /= int_pow(theta, (int)e.ea);
+                be /= int_pow(theta, (int)e.eb);
+                ga /= int_pow(theta, (int)e.eg);
+            } else if (!isfinite(theta)) {
+                set_status(e.status, SVT_ERR_DIVERGED);
+            }  // theta == 0: the chain's matrix is zero; nothing to scale
+            scale[0] = al;
+            scale[1] = be;
+            scale[2] = ga;
+        }
+        __syncthreads();
+        al = scale[0];
+        be = scale[1];
+        ga = scale[2];
     }
     double nrm = 0.0;
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            int64_t r = (int64_t)tm * kF64Tile + ty + 16 * i;
-            int64_t c = (int64_t)tn * kF64Tile + tx + 16 * j;
-            if (r >= P.M || c >= P.N || (P.sym && r > c))
-                continue;
-            double x = al * acc[i][j];
-            if (e.c_kind != C_NONE)
-                x += be * f64_load_c(e, r, c);
-            if (r == c) {
-                x += ga;
-                if (e.diag)
-                    x = e.diag[r] * e.dss[0] - e.dss[1];
-            }
-            if (e.norm_acc)
-                nrm += (P.sym && r != c) ? 2.0 * x * x : x * x;
-            f64_store(e.o_kind, e.o0, e.o_trans ? c * e.ldo + r : r * e.ldo + c, x);
-            if (P.sym && r != c)
-                f64_store(e.o_kind, e.o0, c * e.ldo + r, x);
-            if (e.t_kind != O_NONE)
-                f64_store(e.t_kind, e.t0, c * e.ldt + r, x);
+    const int64_t r = (int64_t)tm * kF64Tile + ty, c = (int64_t)tn * kF64Tile + tx;
+    if (r < P.M && c < P.N && !(P.sym && r > c)) {
+        double x = al * acc;
+        if (e.c_kind != C_NONE)
+            x += be * f64_load_c(e, r, c);
+        if (r == c) {
+            x += ga;
+            if (e.diag)
+                x = e.diag[r] * e.dss[0] - e.dss[1];
         }
+        if (e.norm_acc)
+            nrm = (P.sym && r != c) ? 2.0 * x * x : x * x;
+        f64_store(e.o_kind, e.o0, e.o_trans ? c * e.ldo + r : r * e.ldo + c, x);
+        if (P.sym && r != c)
+            f64_store(e.o_kind, e.o0, c * e.ldo + r, x);
+        if (e.t_kind != O_NONE)
+            f64_store(e.t_kind, e.t0, c * e.ldt + r, x);
+    }
     if (e.norm_acc) {
         for (int o = 16; o > 0; o >>= 1)
             nrm += __shfl_xor_sync(0xffffffffu, nrm, o);
@@ -608,7 +627,7 @@ cudaError_t f64_gemm_launch(const F64Launch &l, cudaStream_t s)
     }
     if (tm == 0 || tn == 0)
         return cudaSuccess;
-    f64_gemm_kernel<<<dim3(tn, tm, l.nprob), 256, 0, s>>>(l);
+    f64_gemm_kernel<<<dim3(tn, tm, l.nprob), kF64Threads, 0, s>>>(l);
     return cudaGetLastError();
 }
 
