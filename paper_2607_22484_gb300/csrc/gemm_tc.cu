@@ -11,11 +11,14 @@
 // c (X^T X)^2) of both polar chains, the polish step and the final combine
 // 1/2 (A - tau P)(I + S) of Proposition 1.
 //
-// Structure (persistent, one CTA per SM, 320 threads):
+// Structure (persistent, one CTA per SM, 384 threads):
 //   warp 0    : TMA producer (one thread), STAGES-deep shared-memory ring.
 //   warp 1    : tensor-memory allocator and MMA issuer (one thread).
 //   warps 2-9 : epilogue; warp w reads TMEM lanes 32 (w % 4) .. 32 (w % 4) + 31, and
 //               the two warps of a lane quadrant take alternate 32-column chunks.
+//   warp 10   : tile scheduler of fused launches (one thread): takes, decodes and waits for
+//               the next tile's dependencies while the producer loads the current one.
+//   warp 11   : publisher of fused launches (one thread): releases finished tiles.
 // Two accumulator buffers of BN FP32 columns each let the epilogue of one tile
 // overlap the MMAs of the next.
 //
@@ -39,14 +42,18 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "solve_scalars.cuh"
 #include "tc_ptx.cuh"
 
 namespace svt {
 
 namespace {
 
-constexpr int kThreads = 320;  // 2 producer/MMA warps + 8 epilogue warps
+// Warp roles: producer, MMA issuer, 8 epilogue warps, tile scheduler, publisher.
 constexpr int kEpiWarps = 8;
+constexpr int kSchedWarp = 2 + kEpiWarps;
+constexpr int kPubWarp = kSchedWarp + 1;
+constexpr int kThreads = 32 * (kPubWarp + 1);
 
 // Limit of the waits on other tiles' results (the launch's debug setting, else 2 s).
 __device__ __forceinline__ uint64_t dep_limit(const TcLaunch &L)
@@ -166,15 +173,22 @@ struct EpiScales {
     float alpha, beta, gamma;
 };
 
-__device__ __forceinline__ EpiScales epi_scales(const Epi &e, double alpha)
+// The FP32 scales of a problem's epilogue. Problems scaled by a norm take theta =
+// norm^theta_pow (1/2 or 1/4) from the finished sum; their FP64 roots and products run in one
+// thread per tile (FP64 is 2 lanes a cycle and SM: the eight epilogue warps computing pow each
+// held the first Z products of a solve for 23,500 cycles).
+__device__ __forceinline__ EpiScales epi_scales(const TcProblem &P, const CallRec *calls)
 {
-    EpiScales s{(float)alpha, (float)e.beta, (float)e.gamma};
+    const Epi &e = P.ep;
+    EpiScales s{e.falpha, e.fbeta, e.fgamma};
+    if (P.patch & PT_ALPHA_NEG_TAU)
+        s.alpha = -calls[P.call_idx].tau;
     if (e.theta_src) {
-        double theta = pow(*e.theta_src, e.theta_pow);
+        const double theta = root_theta(*e.theta_src, e.theta_pow == 0.25);
         if (theta > 0.0 && isfinite(theta)) {
-            s.alpha = (float)(alpha * pow(theta, -e.ea));
-            s.beta = (float)(e.beta * pow(theta, -e.eb));
-            s.gamma = (float)(e.gamma * pow(theta, -e.eg));
+            s.alpha = (float)(e.alpha / int_pow(theta, (int)e.ea));
+            s.beta = (float)(e.beta / int_pow(theta, (int)e.eb));
+            s.gamma = (float)(e.gamma / int_pow(theta, (int)e.eg));
         } else if (!isfinite(theta) && e.status) {
             atomicCAS(e.status, 0, (int)SVT_ERR_DIVERGED);
         }  // theta == 0: the chain's matrix is zero; nothing to scale
@@ -203,7 +217,6 @@ struct EpiHot {
     void *f0;          // e4m3 copy (FP8 experiment), null: none
     int64_t ldf;
     float fscale;
-    int strip_base, tiles_m;  // fused solves: the problem's strip counters
 };
 
 // Raw C values of one lane's 32-column row segment: BF16 hi in q[0..3] (lo of a
@@ -752,7 +765,8 @@ __device__ __forceinline__ void epilogue_finish_spec(const EpiHot &h, int64_t r0
 
 // Load the epilogue fields of problem P (with the per-call fields of a grouped or
 // fused launch) into registers.
-__device__ __forceinline__ void load_hot(EpiHot &h, const TcProblem &P, const CallRec *calls)
+__device__ __forceinline__ void load_hot(EpiHot &h, const TcProblem &P, const CallRec *calls,
+                                         const EpiScales &sc)
 {
     const Epi &e = P.ep;
     h.c0 = e.c0;
@@ -775,15 +789,12 @@ __device__ __forceinline__ void load_hot(EpiHot &h, const TcProblem &P, const Ca
     h.ttma = P.t_tma;
     h.c_kind = e.c_kind;
     h.c_trans = e.c_trans;
-    h.strip_base = P.strip_base;  // read only by strip launches
-    h.tiles_m = P.tiles_m;
     h.o_kind = e.o_kind;
     h.o_trans = e.o_trans;
     h.t_kind = e.t_kind;
     h.f0 = e.f0;
     h.ldf = e.ldf;
     h.fscale = e.fscale;
-    double alpha = e.alpha;
     if (P.patch) {  // grouped / fused launch: per-call fields
         const CallRec &cr = calls[P.call_idx];
         if (P.patch & PT_C_IS_A) {
@@ -795,10 +806,7 @@ __device__ __forceinline__ void load_hot(EpiHot &h, const TcProblem &P, const Ca
             h.ldo = cr.ldy;
             h.otma = 0;
         }
-        if (P.patch & PT_ALPHA_NEG_TAU)
-            alpha = -(double)cr.tau;
     }
-    const EpiScales sc = epi_scales(e, alpha);
     h.alpha = sc.alpha;
     h.beta = sc.beta;
     h.gamma = sc.gamma;
@@ -806,7 +814,17 @@ __device__ __forceinline__ void load_hot(EpiHot &h, const TcProblem &P, const Ca
 
 // --------------------------------------------------------------- kernel
 
-constexpr int kRingTiles = 4;  // fused launches: tile ids in flight between the roles
+constexpr int kRingTiles = 4;  // fused launches: tiles in flight between the roles
+
+// A tile handed from the scheduler to the other roles (and to the peer CTA of a pair): its
+// operands' dependencies are met, its epilogue's scales computed.
+struct RingTile {
+    int tile;  // index in the launch (-1: no more tiles)
+    int prob;  // -1: nothing to compute
+    int tm, tn;
+    float alpha, beta, gamma;
+    int pad;
+};
 
 template <int BN, int STAGES, bool CHAIN, bool PAIR, int NSTG, bool STRIPS>
 __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_constant__ TcLaunch L)
@@ -831,13 +849,16 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(drain + 1);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_slot + 1);
     int *skip_flag = reinterpret_cast<int *>(tmem_slot + 2);
-    // Fused launches: a ring of tile ids from the producer to the MMA and epilogue roles.
+    // Fused launches: the ring of tiles from the scheduler to the other roles; pdone[i]: the
+    // epilogue warps' parts of the tile in entry i are in global memory; ptaken: the producer
+    // has read its latest entry.
     uint64_t *rfull = reinterpret_cast<uint64_t *>(
         (reinterpret_cast<uintptr_t>(tmem_slot + 3) + 7) & ~static_cast<uintptr_t>(7));
     uint64_t *rempty = rfull + kRingTiles;
-    // Ring entry i: tring[4 i .. 4 i + 3] = tile index (-1: no more tiles), problem
-    // (-1: nothing to compute), tile row, tile column -- decoded once by the producer.
-    volatile int *tring = reinterpret_cast<volatile int *>(rempty + kRingTiles);
+    uint64_t *pdone = rempty + kRingTiles;
+    uint64_t *ptaken = pdone + kRingTiles;
+    volatile RingTile *ring = reinterpret_cast<volatile RingTile *>(
+        (reinterpret_cast<uintptr_t>(ptaken + 1) + 15) & ~static_cast<uintptr_t>(15));
     const CallRec *calls = L.calls ? L.calls : &L.call_inline;
 
     const int warp = threadIdx.x >> 5;
@@ -860,10 +881,12 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
         mbar_init(drain, 1);
         for (int i = 0; i < kRingTiles; ++i) {
             mbar_init(&rfull[i], 1);
-            // Consumers of a ring entry: the MMA issuer and the epilogue warps; for
-            // pairs also the peer's producer and epilogue warps.
-            mbar_init(&rempty[i], PAIR ? 2 * (1 + kEpiWarps) : 1 + kEpiWarps);
+            // Consumers of a ring entry: producer, MMA issuer, epilogue warps and publisher;
+            // for pairs also the peer's (which issues no MMAs).
+            mbar_init(&rempty[i], PAIR ? 2 * (2 + kEpiWarps) + 1 : 3 + kEpiWarps);
+            mbar_init(&pdone[i], kEpiWarps);
         }
+        mbar_init(ptaken, 1);
         *abort_flag = 0;
         // A solve whose earlier launch already timed out does no further work.
         *skip_flag = (status0 && *reinterpret_cast<volatile int *>(status0) == (int)SVT_ERR_TIMEOUT);
@@ -889,7 +912,149 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
     const int t_first = PAIR ? (int)(blockIdx.x >> 1) : (int)blockIdx.x;
     const int t_step = PAIR ? (int)(gridDim.x >> 1) : (int)gridDim.x;
 
-    if (warp == 0 && lane == 0) {
+    // Take over ring entry ri: wait for it, read it, and release it at once (`keep`: the
+    // caller releases it later).
+    auto ring_release = [&](int ri) {
+        if (PAIR && !leader)
+            mbar_arrive_remote(peer_addr(&rempty[ri], 0));
+        else
+            mbar_arrive(&rempty[ri]);
+    };
+    if (warp == kSchedWarp && lane == 0) {
+        // ------------------------------------------------ tile scheduler (fused launches)
+        // Takes tiles in table order, one ahead of the one the producer is loading, so that the
+        // counter's round trip, the decoding, the tensor maps' and problem fields' fetches and
+        // the dependency wait of a tile run beside the copies of the tile before it (in the
+        // producer they cost 2200 cycles between tiles). With the publisher: 256-matrix batch
+        // 10.03 -> 8.68 ms, single solves 1 to 2 % faster.
+        if (CHAIN && (!PAIR || leader)) {
+            int ri = 0, hint = 0;
+            uint32_t rphase = 0, taken = 0;
+            int dep_prob = -1;  // problem whose whole dependencies have been waited for
+            bool src_done[2] = {false, false};
+            for (bool first = true;; first = false) {
+                if (!first) {
+                    if (!mbar_wait(ptaken, taken, abort_flag, status0, kWaitTimeoutNs))
+                        break;
+                    taken ^= 1u;
+                }
+                if (!wait_bar<PAIR>(&rempty[ri], rphase ^ 1u, abort_flag, status0, kWaitTimeoutNs))
+                    break;
+                const int next = L.tile_lo + atomicAdd(L.tile_counter, 1);
+                int t = next < total ? next : -1;
+                TileCoord tc{-1, 0, 0, false};
+                if (t >= 0)
+                    tc = decode_tile<BN, TILE_ROWS, STRIPS>(L, t, hint);
+                EpiScales sc{1.f, 0.f, 0.f};
+                bool ok = true;
+                if (tc.valid) {
+                    const TcProblem &P = prob_at(L, tc.prob);
+                    // The fields that the other roles read, into L1, and the tensor maps of the
+                    // first segment into the descriptor cache.
+                    const char *pb = reinterpret_cast<const char *>(&P.o_tma);
+                    const int nlines =
+                        (int)((sizeof(TcProblem) - offsetof(TcProblem, o_tma) + 127) / 128) + 1;
+                    for (int k = 0; k < nlines; ++k)
+                        asm volatile("prefetch.L1 [%0];" ::"l"(pb + 128 * k));
+                    prefetch_tensormap(&P.mapL[P.segL[0]]);
+                    prefetch_tensormap(&P.mapR[P.segR[0]]);
+                    // Operands are results of earlier problems: wait until they are complete
+                    // (whole problems), or until the strips this tile reads are (L: the strip
+                    // of this tile's row, R: of its column).
+                    if (!STRIPS || tc.prob != dep_prob) {  // strips: once per problem, counts only grow
+                        for (int d = 0; d < 2 && ok; ++d)
+                            if (P.dep[d] >= 0)
+                                ok = wait_counter(&L.done[P.dep[d]], P.dep_target[d], abort_flag,
+                                                  status0, dep_limit(L));
+                    }
+                    if (STRIPS) {
+                        if (tc.prob != dep_prob) {
+                            dep_prob = tc.prob;
+                            src_done[0] = !P.sdep_mode[0];
+                            src_done[1] = !P.sdep_mode[1];
+                        }
+                        for (int q = 0; q < 2 && ok; ++q)
+                            if (!src_done[q])
+                                ok = wait_strip(L, P, q, q ? tc.tn : tc.tm, src_done[q], abort_flag,
+                                                status0);
+                        if (P.ep.theta_src)  // the norm its scales come from is complete
+                            for (int d = 0; d < P.nwdep && ok; ++d)
+                                ok = wait_counter(&L.done[P.wdep[d]], P.wdep_target[d], abort_flag,
+                                                  status0, dep_limit(L));
+                    }
+                    if (ok) {
+                        sc = epi_scales(P, calls);
+                        fence_async_global();  // the TMA reads of the tile come after the acquire
+                    }
+                }
+                if (!ok) {  // the wait gave up: end the ring, also for the peer CTA
+                    t = -1;
+                    tc.valid = false;
+                }
+                const int ent[7] = {t, tc.valid ? tc.prob : -1, tc.tm, tc.tn, __float_as_int(sc.alpha),
+                                    __float_as_int(sc.beta), __float_as_int(sc.gamma)};
+                volatile int *w = reinterpret_cast<volatile int *>(&ring[ri]);
+#pragma unroll
+                for (int k = 0; k < 7; ++k)
+                    w[k] = ent[k];
+                if (PAIR) {
+                    const uint32_t pw = peer_addr((const void *)&ring[ri], 1);
+#pragma unroll
+                    for (int k = 0; k < 7; ++k)
+                        st_remote_u32(pw + 4 * k, ent[k]);
+                    mbar_arrive_remote(peer_addr(&rfull[ri], 1));
+                }
+                mbar_arrive(&rfull[ri]);
+                if (++ri == kRingTiles) {
+                    ri = 0;
+                    rphase ^= 1u;
+                }
+                if (t < 0)
+                    break;
+            }
+        }
+    } else if (warp == kPubWarp && lane == 0) {
+        // ------------------------------------------------ publisher (fused launches)
+        // Releases a tile's results to the tiles that read them: once every epilogue warp's
+        // stores are complete, one GPU-scope fence (cumulative over what the warps released to
+        // this thread) and the increment of the problem's counter. The fence takes 1700 to 2200
+        // cycles, which the epilogue warps, each fencing for itself, spent between tiles.
+        if (CHAIN) {
+            int ri = 0;
+            uint32_t rphase = 0, par = 0;  // bit i: parity of pdone[i]'s next use
+            for (;;) {
+                if (!wait_bar<PAIR>(&rfull[ri], rphase, abort_flag, status0, kWaitTimeoutNs))
+                    break;
+                const int t = ring[ri].tile, prob = ring[ri].prob, tm = ring[ri].tm, tn = ring[ri].tn;
+                if (prob >= 0) {
+                    const TcProblem &P = prob_at(L, prob);
+                    const int pid = P.pid;
+                    if (!mbar_wait(&pdone[ri], (par >> ri) & 1u, abort_flag, status0, kWaitTimeoutNs))
+                        break;
+                    par ^= 1u << ri;
+                    fence_async_global();
+                    asm volatile("fence.acq_rel.gpu;" ::: "memory");
+                    red_add_relaxed(&L.done[pid], kEpiWarps);
+                    if (STRIPS && P.strip_base >= 0) {  // the strips this tile completes a part of
+                        int *sp = L.strips + P.strip_base;
+                        red_add_relaxed(sp + tm, kEpiWarps);
+                        if (!P.sym)
+                            red_add_relaxed(sp + P.tiles_m + tn, kEpiWarps);
+                        else if (tn != tm)
+                            red_add_relaxed(sp + tn, kEpiWarps);
+                    }
+                }
+                // Released only now: entry ri, and with it pdone[ri], comes round again after this.
+                ring_release(ri);
+                if (++ri == kRingTiles) {
+                    ri = 0;
+                    rphase ^= 1u;
+                }
+                if (t < 0)
+                    break;
+            }
+        }
+    } else if (warp == 0 && lane == 0) {
         // ------------------------------------------------ TMA producer
         int stage = 0;
         uint32_t phase = 0;
@@ -898,44 +1063,19 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
         int ri = 0;
         uint32_t rphase = 0;
         int hint = 0;
-        int dep_prob = -1;       // problem whose whole dependencies have been waited for
-        bool src_done[2] = {false, false};
-        int smode[2] = {0, 0};   // that problem's strip dependencies of L and R
         for (int t = t_first; ok; t += t_step) {
             TileCoord tc;
             if (CHAIN) {
-                if (!PAIR || leader) {
-                    // Take the next tile in table order, decode it and hand it to the
-                    // other roles (and to the peer CTA of a pair).
-                    if (!wait_bar<PAIR>(&rempty[ri], rphase ^ 1u, abort_flag, status0, kWaitTimeoutNs))
-                        break;
-                    t = L.tile_lo + atomicAdd(L.tile_counter, 1);
-                    t = (t < total) ? t : -1;
-                    tc = TileCoord{-1, 0, 0, false};
-                    if (t >= 0)
-                        tc = decode_tile<BN, TILE_ROWS, STRIPS>(L, t, hint);
-                    const int ent[4] = {t, tc.valid ? tc.prob : -1, tc.tm, tc.tn};
-#pragma unroll
-                    for (int k = 0; k < 4; ++k)
-                        tring[4 * ri + k] = ent[k];
-                    if (PAIR) {
-#pragma unroll
-                        for (int k = 0; k < 4; ++k)
-                            st_remote_u32(peer_addr((const void *)&tring[4 * ri + k], 1), ent[k]);
-                        mbar_arrive_remote(peer_addr(&rfull[ri], 1));
-                    }
-                    mbar_arrive(&rfull[ri]);
-                } else {
-                    // Peer CTA: the leader's tile.
-                    if (!mbar_wait_cluster(&rfull[ri], rphase, abort_flag, status0, kWaitTimeoutNs))
-                        break;
-                    t = tring[4 * ri];
-                    tc.prob = tring[4 * ri + 1];
-                    tc.tm = tring[4 * ri + 2];
-                    tc.tn = tring[4 * ri + 3];
-                    tc.valid = tc.prob >= 0;
-                    mbar_arrive_remote(peer_addr(&rempty[ri], 0));
-                }
+                if (!wait_bar<PAIR>(&rfull[ri], rphase, abort_flag, status0, kWaitTimeoutNs))
+                    break;
+                t = ring[ri].tile;
+                tc.prob = ring[ri].prob;
+                tc.tm = ring[ri].tm;
+                tc.tn = ring[ri].tn;
+                tc.valid = tc.prob >= 0;
+                ring_release(ri);
+                if (!PAIR || leader)
+                    mbar_arrive(ptaken);
                 if (++ri == kRingTiles) {
                     ri = 0;
                     rphase ^= 1u;
@@ -950,50 +1090,13 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
             if (!tc.valid)
                 continue;
             const TcProblem &P = prob_at(L, tc.prob);
-            {
-                // The epilogue reads this problem's fields after o_tma (and the Epi) when
-                // it reaches the tile, a few tiles later: bring their lines into L1 now.
-                const char *pb = reinterpret_cast<const char *>(&P.o_tma);
-                const int nlines =
-                    (int)((sizeof(TcProblem) - offsetof(TcProblem, o_tma) + 127) / 128) + 1;
-                for (int k = 0; k < nlines; ++k)
-                    asm volatile("prefetch.L1 [%0];" ::"l"(pb + 128 * k));
-            }
             // A k-block is one 128-byte swizzle row: 64 BF16 or 128 e4m3 elements.
             const int kshift = P.fp8 ? 7 : 6;
             const int kblocks = (P.K + (1 << kshift) - 1) >> kshift;
             const int row0 = (PAIR ? 2 * tc.tm + (int)rank : tc.tm) * kBM;
             const int col0 = tc.tn * BN + (int)rank * B_ROWS;
-            if (CHAIN) {
-                // Operands are results of earlier problems: wait until they are complete
-                // (whole problems), or until the strips this tile reads are (L: the
-                // strip of this tile's row, R: of its column).
-                if (STRIPS) {
-                    if (tc.prob != dep_prob) {  // once per problem: counts only grow
-                        for (int d = 0; d < 2 && ok; ++d)
-                            if (P.dep[d] >= 0)
-                                ok = wait_counter(&L.done[P.dep[d]], P.dep_target[d], abort_flag,
-                                                  status0, dep_limit(L));
-                        dep_prob = tc.prob;
-                        smode[0] = P.sdep_mode[0];
-                        smode[1] = P.sdep_mode[1];
-                        src_done[0] = !smode[0];
-                        src_done[1] = !smode[1];
-                    }
-                    for (int q = 0; q < 2 && ok; ++q)
-                        if (!src_done[q])
-                            ok = wait_strip(L, P, q, q ? tc.tn : tc.tm, src_done[q], abort_flag,
-                                            status0);
-                } else {
-                    for (int d = 0; d < 2 && ok; ++d)
-                        if (P.dep[d] >= 0)
-                            ok = wait_counter(&L.done[P.dep[d]], P.dep_target[d], abort_flag,
-                                              status0, dep_limit(L));
-                }
-                fence_async_global();  // the TMA reads below come after the acquire
-                if (!ok)
-                    break;
-            }
+            if (CHAIN)
+                fence_async_global();  // the TMA reads below come after the scheduler's acquire
             for (int sg = 0; sg < P.nseg && ok; ++sg) {
                 const CUtensorMap *mL = &P.mapL[P.segL[sg]];
                 const CUtensorMap *mR = &P.mapR[P.segR[sg]];
@@ -1049,12 +1152,12 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
             if (CHAIN) {
                 if (!mbar_wait(&rfull[ri], rphase, abort_flag, status0, kWaitTimeoutNs))
                     break;
-                t = tring[4 * ri];
-                tc.prob = tring[4 * ri + 1];
-                tc.tm = tring[4 * ri + 2];
-                tc.tn = tring[4 * ri + 3];
+                t = ring[ri].tile;
+                tc.prob = ring[ri].prob;
+                tc.tm = ring[ri].tm;
+                tc.tn = ring[ri].tn;
                 tc.valid = tc.prob >= 0;
-                mbar_arrive(&rempty[ri]);
+                ring_release(ri);
                 if (++ri == kRingTiles) {
                     ri = 0;
                     rphase ^= 1u;
@@ -1136,7 +1239,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
             mma_commit(drain);
         volatile int no_abort = 0;
         mbar_wait(drain, 0, &no_abort, nullptr, kWaitTimeoutNs / 4);
-    } else if (warp >= 2) {
+    } else if (warp >= 2 && warp < kSchedWarp) {
         // ------------------------------------------------ epilogue
         const int quad = warp & 3;  // TMEM lane quadrant this warp may access
         const int half = (warp - 2) >> 2;  // two warps per quadrant split the column chunks
@@ -1151,21 +1254,21 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
         int hint = 0;
         for (int t = t_first;; t += t_step) {
             TileCoord tc;
+            EpiScales sc;
+            int entry = 0;  // the tile's ring entry
             if (CHAIN) {
                 if (!wait_bar<PAIR>(&rfull[ri], rphase, abort_flag, status0, kWaitTimeoutNs))
                     break;
-                t = tring[4 * ri];
-                tc.prob = tring[4 * ri + 1];
-                tc.tm = tring[4 * ri + 2];
-                tc.tn = tring[4 * ri + 3];
+                t = ring[ri].tile;
+                tc.prob = ring[ri].prob;
+                tc.tm = ring[ri].tm;
+                tc.tn = ring[ri].tn;
                 tc.valid = tc.prob >= 0;
+                sc = EpiScales{ring[ri].alpha, ring[ri].beta, ring[ri].gamma};
+                entry = ri;
                 __syncwarp();
-                if (lane == 0) {
-                    if (PAIR && !leader)
-                        mbar_arrive_remote(peer_addr(&rempty[ri], 0));
-                    else
-                        mbar_arrive(&rempty[ri]);
-                }
+                if (lane == 0)
+                    ring_release(ri);
                 if (++ri == kRingTiles) {
                     ri = 0;
                     rphase ^= 1u;
@@ -1180,8 +1283,8 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
             if (!tc.valid)
                 continue;
             const TcProblem &P = prob_at(L, tc.prob);
-            if (CHAIN && !STRIPS && (P.ep.c_kind != C_NONE || P.ep.theta_src)) {
-                // C or the norm bound is an earlier result: make it visible to these loads.
+            if (CHAIN && !STRIPS && P.ep.c_kind != C_NONE) {
+                // C is an earlier result: make it visible to these loads.
                 for (int d = 0; d < 2; ++d)
                     if (P.dep[d] >= 0 && lane == 0)
                         wait_counter(&L.done[P.dep[d]], P.dep_target[d], abort_flag, status0,
@@ -1189,11 +1292,11 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
                 __syncwarp();
             }
             if (STRIPS) {
-                // C or the norm bound is an earlier result: make it visible to these loads;
-                // earlier readers of the buffers this tile overwrites must be done.
+                // C is an earlier result: make it visible to these loads; earlier readers of the
+                // buffers this tile overwrites must be done.
                 if (lane == 0) {
                     if (tc.prob != last_prob) {  // once per problem: counts only grow
-                        if (P.ep.c_kind != C_NONE || P.ep.theta_src)
+                        if (P.ep.c_kind != C_NONE)
                             for (int d = 0; d < 2; ++d)
                                 if (P.dep[d] >= 0)
                                     wait_counter(&L.done[P.dep[d]], P.dep_target[d], abort_flag,
@@ -1211,7 +1314,9 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
             if (PAIR)
                 tc.tm = 2 * tc.tm + (int)rank;  // this CTA's 128-row half of the tile
             EpiHot h;  // per tile: its registers are free outside the tile's loops
-            load_hot(h, P, calls);
+            if (!CHAIN)
+                sc = epi_scales(P, calls);
+            load_hot(h, P, calls, sc);
             const int spec = epi_spec(h);
             last_prob = tc.prob;
             const int64_t warp_row0 = (int64_t)tc.tm * kBM + quad * 32;
@@ -1305,27 +1410,15 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
                 tphase ^= 1u;
             }
             if (CHAIN) {
-                // Publish: this warp's part of the tile is in global memory. The lanes'
-                // plain stores (diagonal blocks of symmetric products, ragged edges) are
-                // ordered before lane 0's accesses by __syncwarp; lane 0's GPU-scope fence
-                // is cumulative over them and over its TMA stores (waited for and fenced
-                // into the generic proxy), and its counter increment releases them all to
-                // the tiles that acquire the counter.
+                // This warp's part of the tile is in global memory: tell the publisher. The
+                // lanes' plain stores (diagonal blocks of symmetric products, ragged edges) are
+                // ordered before lane 0's arrival by __syncwarp, its TMA stores by their
+                // completion.
                 __syncwarp();
                 if (lane == 0) {
                     bulk_wait_all0();
                     fence_async_global();
-                    __threadfence();
-                    atomicAdd(&L.done[P.pid], 1);
-                    if (STRIPS && h.strip_base >= 0) {  // the strips this tile completes a part of
-                        int *sp = L.strips + h.strip_base;
-                        const int sr = PAIR ? (tc.tm >> 1) : tc.tm;  // tile (pair) row
-                        atomicAdd(sp + sr, 1);
-                        if (!h.sym)
-                            atomicAdd(sp + h.tiles_m + tc.tn, 1);
-                        else if (tc.tn != sr)
-                            atomicAdd(sp + tc.tn, 1);
-                    }
+                    mbar_arrive(&pdone[entry]);
                 }
                 __syncwarp();
             }

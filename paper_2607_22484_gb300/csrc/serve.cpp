@@ -431,7 +431,7 @@ svt_status issue_window(svt_ctx *ctx, ServeState *s, int sms)
                         attach_store_maps(tp);
                     }
                     if (pr.flags & PT_ALPHA_NEG_TAU)
-                        tp.ep.alpha = -(double)r->m.tau;
+                        tp.ep.falpha = -r->m.tau;
                 }
             tp.patch = 0;
             starts[g].push_back(tiles[g]);

@@ -241,50 +241,6 @@ __device__ __forceinline__ void tmem_ld_frag(uint32_t taddr, float *v)
         v[i] = __uint_as_float(r[i]);
 }
 
-__device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
-
-__device__ __forceinline__ void ldmatrix4(uint32_t (&w)[4], uint32_t addr)
-{
-    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
-                 : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3])
-                 : "r"(addr)
-                 : "memory");
-}
-
-template <bool TRANS>
-__device__ __forceinline__ void stmatrix4(uint32_t addr, const uint32_t (&w)[4])
-{
-    if (TRANS)
-        asm volatile("stmatrix.sync.aligned.m8n8.x4.trans.shared.b16 [%0], {%1, %2, %3, %4};" ::"r"(addr),
-                     "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3])
-                     : "memory");
-    else
-        asm volatile("stmatrix.sync.aligned.m8n8.x4.shared.b16 [%0], {%1, %2, %3, %4};" ::"r"(addr),
-                     "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3])
-                     : "memory");
-}
-
-__device__ __forceinline__ uint32_t movmatrix_trans(uint32_t w)
-{
-    uint32_t t;
-    asm volatile("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;" : "=r"(t) : "r"(w));
-    return t;
-}
-
-// The 8 x 8 diagonal block with its lower triangle taken from the upper one.
-__device__ __forceinline__ uint32_t mirror_diag(uint32_t w, int lane)
-{
-    const uint32_t t = movmatrix_trans(w);
-    const int row = lane >> 2, col = 2 * (lane & 3);
-    const uint32_t lo = col >= row ? w : t, hi = col + 1 >= row ? w : t;
-    return (lo & 0xffffu) | (hi & 0xffff0000u);
-}
-
-__device__ __forceinline__ float2 bf16x2(uint32_t w)
-{
-    return __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&w));
-}
-
 // A thread's shared-memory offsets for its warp's first chunk (rows 32 (warp % 4), columns
 // 16 (warp / 4)), the same for every product. stmatrix and ldmatrix move the four 8 x 8 blocks
 // g (rows + 8 g) of one column group k (columns + 8 k); lane l gives the address of row l % 8 of

@@ -117,7 +117,10 @@ bool encode_store_map(CUtensorMap *map, const void *ptr, int64_t rows, int64_t c
 
 void attach_store_maps(TcProblem &p)
 {
-    const Epi &e = p.ep;
+    Epi &e = p.ep;
+    e.falpha = (float)e.alpha;
+    e.fbeta = (float)e.beta;
+    e.fgamma = (float)e.gamma;
     p.o_tma = 0;
     p.t_tma = 0;
     // Output: tile-oriented M x N, or transposed N x M when o_trans.
@@ -940,7 +943,7 @@ svt_status run_ops(svt_ctx *ctx, Plan &P, const CallArgs &a, cudaStream_t s, siz
                         e.ldo = a.ldy;
                     }
                     if (pr.flags & PT_ALPHA_NEG_TAU)
-                        e.alpha = -(double)a.tau;
+                        e.falpha = -a.tau;
                 }
             cudaEvent_t e0 = nullptr, e1 = nullptr;
             if (prof) {

@@ -54,6 +54,7 @@ enum Scal : int {
 
 struct Epi {
     double alpha, beta, gamma;       // v = alpha D + beta C + gamma [r == c]
+    float falpha, fbeta, fgamma;     // the same in FP32, as the tensor-core epilogue scales
     double ea, eb, eg;               // exponents: alpha *= theta^-ea, ...
     const double *theta_src;         // theta = (*theta_src)^theta_pow; null: theta = 1
     double theta_pow;

@@ -2,6 +2,7 @@
 // shared-memory and instruction descriptors, MMA issue, tensor-memory allocation and reads.
 #pragma once
 
+#include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -215,6 +216,16 @@ __device__ __forceinline__ int ld_acquire_gpu(const int *p)
     return v;
 }
 
+__device__ __forceinline__ void red_add_relaxed(int *p, int v)
+{
+    asm volatile("red.relaxed.gpu.global.add.s32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
+
+__device__ __forceinline__ void prefetch_tensormap(const CUtensorMap *map)
+{
+    asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(map)) : "memory");
+}
+
 // Bounded wait until *counter >= target (another CTA's completion count).
 __device__ bool wait_counter(const int *counter, int target, volatile int *abort_flag, int *status,
                              uint64_t limit_ns)
@@ -397,6 +408,70 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float *v)
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
     for (int i = 0; i < 32; ++i)
+        v[i] = __uint_as_float(r[i]);
+}
+
+// ---- matrix fragments: of an 8 x 8 block, thread t holds row t / 4 and columns 2 (t % 4), + 1
+// (a BF16 pair), which is what ldmatrix and stmatrix move and what the .16x256b tensor-memory
+// load delivers.
+
+__device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+
+__device__ __forceinline__ void ldmatrix4(uint32_t (&w)[4], uint32_t addr)
+{
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3])
+                 : "r"(addr)
+                 : "memory");
+}
+
+template <bool TRANS>
+__device__ __forceinline__ void stmatrix4(uint32_t addr, const uint32_t (&w)[4])
+{
+    if (TRANS)
+        asm volatile("stmatrix.sync.aligned.m8n8.x4.trans.shared.b16 [%0], {%1, %2, %3, %4};" ::"r"(addr),
+                     "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3])
+                     : "memory");
+    else
+        asm volatile("stmatrix.sync.aligned.m8n8.x4.shared.b16 [%0], {%1, %2, %3, %4};" ::"r"(addr),
+                     "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3])
+                     : "memory");
+}
+
+__device__ __forceinline__ uint32_t movmatrix_trans(uint32_t w)
+{
+    uint32_t t;
+    asm volatile("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;" : "=r"(t) : "r"(w));
+    return t;
+}
+
+// The 8 x 8 diagonal block with its lower triangle taken from the upper one.
+__device__ __forceinline__ uint32_t mirror_diag(uint32_t w, int lane)
+{
+    const uint32_t t = movmatrix_trans(w);
+    const int row = lane >> 2, col = 2 * (lane & 3);
+    const uint32_t lo = col >= row ? w : t, hi = col + 1 >= row ? w : t;
+    return (lo & 0xffffu) | (hi & 0xffff0000u);
+}
+
+__device__ __forceinline__ float2 bf16x2(uint32_t w)
+{
+    return __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&w));
+}
+
+// 16 tensor-memory lanes x 32 columns: v[4 k], v[4 k + 1] row t / 4, columns 8 k + 2 (t % 4), + 1;
+// v[4 k + 2], v[4 k + 3] row t / 4 + 8.
+__device__ __forceinline__ void tmem_ld_frag32(uint32_t taddr, float *v)
+{
+    uint32_t r[16];
+    asm volatile("tcgen05.ld.sync.aligned.16x256b.x4.b32 "
+                 "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]),
+                   "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]),
+                   "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+                 : "r"(taddr));
+#pragma unroll
+    for (int i = 0; i < 16; ++i)
         v[i] = __uint_as_float(r[i]);
 }
 
