@@ -233,8 +233,9 @@ svt_status svt_batch_workspace_bytes(const svt_matrix *mats, int count, size_t *
  * (A and Y stay caller-owned device memory and must stay valid until the ticket
  * completes) into the admission queue and returns a ticket. A scheduler thread
  * admits queued requests while their workspaces fit in the context's workspace
- * and a slot is free, advances all admitted requests one stage window at a time
- * with one grouped launch per window, and retires finished requests. Requests of
+ * and a slot is free, advances all admitted requests one window (a few stages, about
+ * a millisecond) at a time with one launch per window, and retires finished requests.
+ * Requests of
  * at least 8 Mi elements take the large lane instead, one at a time: a fused solve
  * issued as consecutive launches of a few milliseconds each, on every SM while no
  * smaller request is waiting or running and on all but 32 SMs otherwise.

@@ -19,9 +19,9 @@
 //   * admits queued requests in arrival order while a slot is free and their
 //     workspace fits in a free range of the context's workspace (first fit),
 //   * issues one window on its stream: grouped ingest of the newly admitted,
-//     ONE grouped product launch per tile width that carries the next stage of
-//     every active request (both polar chains of each), and grouped finalize of
-//     requests at their last op.
+//     ONE fused product launch per tile width that carries the next stages of
+//     every active request (both polar chains of each), about a millisecond of
+//     work, and grouped finalize of requests that reach their last op.
 // A request therefore joins the very next window after memory frees up, and
 // its stages share launches with whatever else is running.
 #include <cuda_runtime.h>
@@ -125,9 +125,18 @@ struct Request {
 
 // Device tables of one serving window live in a ring of slots at the end of the
 // workspace; each slot is staged from its own pinned host buffer.
-constexpr int kRing = 8;
-constexpr size_t kRingSlotBytes = 128 << 10;
+constexpr int kRing = 2;
+constexpr size_t kRingSlotBytes = 512 << 10;
 constexpr size_t kRingBytes = kRing * kRingSlotBytes;
+
+// A window carries consecutive product stages of every active request in one fused launch,
+// whose tiles wait on device-side counters for their own request's earlier stages only, until
+// its tensor flops reach kWindowWork (about a millisecond on the whole GPU; scaled by the SMs
+// the window may use) or its tables fill a ring slot. One stage per window left the SMs idle at
+// every stage's end: a burst of 24 requests of 256 to 2048 took 10.7 ms with 64 windows of
+// 80 us a request, 8.4 ms with these.
+constexpr double kWindowWork = 4e11;
+constexpr int kSingleOps = 8;  // ops per window of a request that the grouped kernels do not cover
 
 // Grouped batch: the stage-merged launch sequence of `count` same-option solves.
 struct BatchPlan {
@@ -315,8 +324,8 @@ bool admissible(const svt_ctx *ctx, const Request *r, double now)
     return ctx->dbg_admit_delay_us <= 0 || now >= r->t_submit + 1e-3 * (double)ctx->dbg_admit_delay_us;
 }
 
-// One serving window: grouped ingest of newly admitted requests, one grouped
-// product launch per tile width holding the next product stage of every active
+// One serving window: grouped ingest of newly admitted requests, one fused
+// product launch per tile width holding the next product stages of every active
 // request, grouped finalize of requests that reached their last op.
 svt_status issue_window(svt_ctx *ctx, ServeState *s, int sms)
 {
@@ -404,43 +413,81 @@ svt_status issue_window(svt_ctx *ctx, ServeState *s, int sms)
         blk_s += grouped_split_blocks(r->plan->m, r->plan->n);
         r->pc += 3;
     }
-    // Product stage of every grouped request (including the ones just ingested).
+    // Product stages of every grouped request (including the ones just ingested), stage by
+    // stage, each problem depending on the previous one of its request's chain in this window
+    // (the combine on both chains; earlier windows precede on the stream).
     std::vector<TcProblem> probs[2];
-    std::vector<int> starts[2];
+    std::vector<int> starts[2], valid[2];
     int tiles[2] = {0, 0};
-    for (Request *r : s->active) {
-        if (r->state != 1 || !r->grouped)
-            continue;
-        Plan &P = *r->plan;
-        const Op &op = P.ops[r->pc];
-        if (op.kind != OP_TC)
-            continue;
-        const int g = (op.bn == 256) ? 1 : 0;
-        const TcLaunch &l = P.tc[op.idx];
-        for (int q = 0; q < l.nprob; ++q) {
-            TcProblem tp = l.p[q];
-            for (const PatchRec &pr : P.patches)
-                if (pr.kind == OP_TC && pr.launch == op.idx && pr.prob == q) {
-                    if (pr.flags & PT_C_IS_A) {
-                        tp.ep.c0 = r->m.A;
-                        tp.ep.ldc = r->m.lda;
+    std::map<const Request *, std::array<int, 2>> lastp;
+    const double work_cap = kWindowWork * sms / ctx->num_sms;
+    double work = 0.0;
+    // Bytes of everything but the problem tables, at most (aux and call records of the ingested
+    // and the finished, starts and counters of both widths).
+    const size_t other = (2 * kSlots) * (sizeof(AuxRec) + sizeof(CallRec)) + 16 * kAlign;
+    auto table_bytes = [&](size_t extra) {
+        return (probs[0].size() + probs[1].size() + extra) * (sizeof(TcProblem) + 2 * sizeof(int)) + other;
+    };
+    bool more = true;
+    for (int stage = 0; more && (stage == 0 || work < work_cap); ++stage) {
+        more = false;
+        for (Request *r : s->active) {
+            if (r->state != 1 || !r->grouped)
+                continue;
+            Plan &P = *r->plan;
+            const Op &op = P.ops[r->pc];
+            if (op.kind != OP_TC)
+                continue;
+            const TcLaunch &l = P.tc[op.idx];
+            if (stage > 0 && table_bytes((size_t)l.nprob) > kRingSlotBytes) {
+                more = false;
+                work = work_cap;
+                break;
+            }
+            more = true;
+            work += P.tc_tensor_flops[op.idx];
+            const int g = (op.bn == 256) ? 1 : 0;
+            size_t chain_at = 0;  // first entry of this launch in tc_chain
+            for (int k = 0; k < op.idx; ++k)
+                chain_at += (size_t)P.tc[k].nprob;
+            auto last = lastp.emplace(r, std::array<int, 2>{-1, -1}).first;
+            for (int q = 0; q < l.nprob; ++q) {
+                TcProblem tp = l.p[q];
+                for (const PatchRec &pr : P.patches)
+                    if (pr.kind == OP_TC && pr.launch == op.idx && pr.prob == q) {
+                        if (pr.flags & PT_C_IS_A) {
+                            tp.ep.c0 = r->m.A;
+                            tp.ep.ldc = r->m.lda;
+                        }
+                        if (pr.flags & PT_O_IS_Y) {
+                            tp.ep.o0 = r->m.Y;
+                            tp.ep.ldo = r->m.ldy;
+                            attach_store_maps(tp);
+                        }
+                        if (pr.flags & PT_ALPHA_NEG_TAU)
+                            tp.ep.falpha = -r->m.tau;
                     }
-                    if (pr.flags & PT_O_IS_Y) {
-                        tp.ep.o0 = r->m.Y;
-                        tp.ep.ldo = r->m.ldy;
-                        attach_store_maps(tp);
-                    }
-                    if (pr.flags & PT_ALPHA_NEG_TAU)
-                        tp.ep.falpha = -r->m.tau;
+                tp.patch = 0;
+                const int chain = P.tc_chain[chain_at + (size_t)q];
+                const int pid = (int)probs[g].size();
+                tp.pid = pid;
+                for (int d = 0; d < 2; ++d) {
+                    tp.dep[d] = chain < 2 ? (d == 0 ? last->second[chain] : -1) : last->second[d];
+                    tp.dep_target[d] = tp.dep[d] >= 0 ? kEpiWarpsPublic * valid[g][tp.dep[d]] : 0;
                 }
-            tp.patch = 0;
-            starts[g].push_back(tiles[g]);
-            tiles[g] += tc_num_tiles(tp, op.bn);
-            probs[g].push_back(tp);
+                if (chain < 2)
+                    last->second[chain] = pid;
+                else
+                    last->second = {pid, pid};
+                starts[g].push_back(tiles[g]);
+                tiles[g] += tc_num_tiles(tp, op.bn);
+                valid[g].push_back(tc_valid_ctas(tp, op.bn));
+                probs[g].push_back(tp);
+            }
+            r->pc += 1;
+            if (P.ops[r->pc].kind == OP_FINAL)
+                fin.push_back(r);
         }
-        r->pc += 1;
-        if (P.ops[r->pc].kind == OP_FINAL)
-            fin.push_back(r);
     }
     // Finalize records.
     std::vector<AuxRec> faux;
@@ -452,11 +499,12 @@ svt_status issue_window(svt_ctx *ctx, ServeState *s, int sms)
     // Stage the tables.
     size_t o_aux = take(sizeof(AuxRec) * aux.size()), o_calls = take(sizeof(CallRec) * calls.size());
     size_t o_faux = take(sizeof(AuxRec) * faux.size()), o_fcalls = take(sizeof(CallRec) * fcalls.size());
-    size_t o_p[2], o_s[2];
+    size_t o_p[2], o_s[2], o_n[2];
     for (int g = 0; g < 2; ++g) {
         starts[g].push_back(tiles[g]);
         o_p[g] = take(sizeof(TcProblem) * probs[g].size());
         o_s[g] = take(sizeof(int) * starts[g].size());
+        o_n[g] = take(sizeof(int) * (probs[g].size() + 1));  // completion counters, tile counter
     }
     if (used > kRingSlotBytes)
         return SVT_ERR_OOM;
@@ -467,6 +515,7 @@ svt_status issue_window(svt_ctx *ctx, ServeState *s, int sms)
     for (int g = 0; g < 2; ++g) {
         std::memcpy(h + o_p[g], probs[g].data(), sizeof(TcProblem) * probs[g].size());
         std::memcpy(h + o_s[g], starts[g].data(), sizeof(int) * starts[g].size());
+        std::memset(h + o_n[g], 0, sizeof(int) * (probs[g].size() + 1));
     }
     cudaStream_t st = s->win;
     if (used && cudaMemcpyAsync(d, h, used, cudaMemcpyHostToDevice, st) != cudaSuccess)
@@ -491,16 +540,16 @@ svt_status issue_window(svt_ctx *ctx, ServeState *s, int sms)
         L.gstart = reinterpret_cast<const int *>(d + o_s[g]);
         L.gcount = (int)probs[g].size();
         L.dep_wait_ns = ctx->dbg_wait_ns;
-        if (tc_gemm_launch_grouped(L, g ? 256 : 128, tiles[g], sms, st) != cudaSuccess)
+        L.done = reinterpret_cast<int *>(d + o_n[g]);
+        L.tile_counter = L.done + probs[g].size();
+        if (tc_gemm_launch_fused(L, g ? 256 : 128, tiles[g], sms, st) != cudaSuccess)
             return SVT_ERR_CUDA;
         ++launched;
     }
-    // Requests outside the grouped kinds advance one op with ordinary launches.
+    // Requests outside the grouped kinds advance a few ops with ordinary launches.
     for (Request *r : single) {
         CallArgs a{r->m.A, r->m.lda, r->m.tau, r->m.Y, r->m.ldy, r->m.d_status};
-        size_t last = r->pc + 1;
-        if (r->plan->ops[r->pc].kind == OP_MEMSET)
-            last = r->pc + 3;  // memset, reduce, split together
+        const size_t last = std::min(r->pc + kSingleOps, r->plan->ops.size());
         svt_status e;
         {
             std::lock_guard<std::mutex> g(ctx->mu);
