@@ -208,21 +208,27 @@ __device__ __forceinline__ bool aligned16(const void *p)
 struct EpiHot {
     const void *c0, *c1;
     void *o0, *o1, *t0, *t1;
-    const CUtensorMap *maps;  // mapO[0..1] then mapT[0..1] of the problem
+    const CUtensorMap *maps;  // mapO[0..1], mapT[0..1], mapU[0..1] of the problem
     double *norm_acc;
     const double *diag, *dss;
     int64_t ldc, ldo, ldt;
     float alpha, beta, gamma;
-    int M, N, sym, otma, ttma, c_kind, c_trans, o_kind, o_trans, t_kind;
+    int M, N, sym, otma, ttma, wide_tma, c_kind, c_trans, o_kind, o_trans, t_kind;
     void *f0;          // e4m3 copy (FP8 experiment), null: none
     int64_t ldf;
     float fscale;
 };
 
-// Raw C values of one lane's 32-column row segment: BF16 hi in q[0..3] (lo of a
-// pair in q[4..7]) or FP32 in q[0..7].
+// Raw C values of one lane: for the generic loop its 32-column row segment, BF16 hi in q[0..3]
+// (lo of a pair in q[4..7]) or FP32 in q[0..7]; for the specialised ones its fragment of the
+// 32 x 32 block, BF16 pairs of block (g, k) in word 4 k + g (lo of a pair 16 further on).
 struct CRaw {
     uint4 q[8];
+    __device__ __forceinline__ uint32_t &word(int i)
+    {
+        uint4 &x = q[i >> 2];
+        return (i & 3) == 0 ? x.x : ((i & 3) == 1 ? x.y : ((i & 3) == 2 ? x.z : x.w));
+    }
 };
 
 // Issue the loads of C(r, c0 .. c0 + 31) into registers. Returns false where the
@@ -641,17 +647,17 @@ __device__ __forceinline__ void epilogue_finish(const EpiHot &h, int64_t r0, int
 // (0 symmetric, 1 symmetric with C, 2 general with copy).
 template <int S>
 struct EpiSpec {
+    static constexpr int code = S;
     static constexpr bool generic = S < 0;
-    static constexpr int okind = S >= 3 ? O_PAIR : O_BF16;
+    static constexpr bool pair = S >= 3;
     static constexpr bool sym = S >= 0 && S % 3 != 2;
-    static constexpr int ckind = (S >= 0 && S % 3 == 1) ? (S >= 3 ? C_PAIR : C_BF16) : C_NONE;
-    static constexpr bool has_t = S >= 0 && S % 3 == 2;
+    static constexpr bool has_c = S >= 0 && S % 3 == 1;
 };
 
 __device__ __forceinline__ int epi_spec(const EpiHot &h)
 {
     if ((h.o_kind != O_BF16 && h.o_kind != O_PAIR) || !h.otma || h.o_trans || h.norm_acc || h.f0 ||
-        h.diag)
+        h.diag || !h.wide_tma)
         return -1;
     const bool pair = h.o_kind == O_PAIR;
     const int base = pair ? 3 : 0;
@@ -667,100 +673,141 @@ __device__ __forceinline__ int epi_spec(const EpiHot &h)
     return -1;
 }
 
-// c_load / c_apply for an untransposed C in BF16 (CK = C_BF16) or as a hi/lo pair.
-template <int CK>
-__device__ __forceinline__ bool c_load_spec(const EpiHot &h, int64_t r, int64_t c0, bool full_row,
-                                            CRaw &cr)
+// Issue the loads of this lane's fragment of C's 32 x 32 block at (r0, c0). Columns past the
+// matrix lie in the row padding of the workspace buffers (rows padded to 64 elements).
+template <bool PAIRED>
+__device__ __forceinline__ void c_load_frag(const EpiHot &h, int64_t r0, int64_t c0, int lane, CRaw &cr)
 {
-    if (!full_row)
-        return false;
-    const int64_t off = r * h.ldc + c0;
-    const __nv_bfloat16 *ph = static_cast<const __nv_bfloat16 *>(h.c0) + off;
-    const __nv_bfloat16 *pl = static_cast<const __nv_bfloat16 *>(h.c1) + off;
-    if (!aligned16(ph) || (CK == C_PAIR && !aligned16(pl)))
-        return false;
 #pragma unroll
-    for (int q = 0; q < 4; ++q)
-        cr.q[q] = __ldg(reinterpret_cast<const uint4 *>(ph) + q);
-    if (CK == C_PAIR) {
+    for (int g = 0; g < 4; ++g) {
+        const int64_t r = r0 + 8 * g + (lane >> 2);
+        const bool ok = r < h.M;
+        const int64_t off = r * h.ldc + c0 + 2 * (lane & 3);
+        const __nv_bfloat16 *ph = static_cast<const __nv_bfloat16 *>(h.c0) + off;
+        const __nv_bfloat16 *pl = static_cast<const __nv_bfloat16 *>(h.c1) + off;
 #pragma unroll
-        for (int q = 0; q < 4; ++q)
-            cr.q[4 + q] = __ldg(reinterpret_cast<const uint4 *>(pl) + q);
+        for (int k = 0; k < 4; ++k) {
+            cr.word(4 * k + g) = ok ? *reinterpret_cast<const uint32_t *>(ph + 8 * k) : 0u;
+            if (PAIRED)
+                cr.word(16 + 4 * k + g) = ok ? *reinterpret_cast<const uint32_t *>(pl + 8 * k) : 0u;
+        }
     }
-    return true;
 }
 
-template <int CK>
-__device__ __forceinline__ void c_apply_spec(const EpiHot &h, const CRaw &cr, bool vec, int64_t r,
-                                             int64_t c0, int ncol, bool row_ok, float *v)
+// How a specialised epilogue stages a 32 x 32 block for its TMA stores: as half of a 64-column
+// unit (BF16 only: one 64 x 32 box in place, one 32 x 64 box mirrored), by itself, or by itself
+// on the diagonal of a symmetric product (one box holding both triangles).
+constexpr int kStgSlots = 2;                  // 4 KiB staging slots of an epilogue warp
+constexpr int kStgBytes = kStgSlots * 4096;
+
+enum StageMode { STAGE_UNIT, STAGE_BLOCK, STAGE_DIAG };
+
+// Offsets in the warp's 8 KiB of staging. STAGE_UNIT: the 64-column rows (128-byte swizzle) at 0,
+// the mirrored rows at kStgMirror64. Else: in place at 0, mirrored at kStgMirror, the lo parts
+// kStgLo further on (64-byte swizzle).
+constexpr uint32_t kStgMirror = 2048, kStgLo = 4096, kStgMirror64 = 4096;
+
+// Stage one part (hi or lo) of a block: w[k][g] holds this lane's pair of 8 x 8 block (g, k).
+// Four blocks g of one k per stmatrix; the transposing form writes their mirror. half: which 32
+// columns of the unit.
+template <int MODE>
+__device__ __forceinline__ void stage_part(uint32_t (&w)[4][4], uint32_t stg, int half, int lane)
 {
-    if (!row_ok)
-        return;
-    const float beta = h.beta;
-    if (vec) {
+    const int g = lane >> 3, j = lane & 7;
 #pragma unroll
-        for (int half = 0; half < (CK == C_PAIR ? 2 : 1); ++half) {
+    for (int k = 0; k < 4; ++k) {
+        uint32_t da, ma;
+        if (MODE == STAGE_UNIT) {
+            const int row = 32 * half + 8 * k + j;
+            da = stg + lane * 128 + (((4 * half + k) ^ j) << 4);
+            ma = stg + kStgMirror64 + row * 64 + ((g ^ ((row >> 1) & 3)) << 4);
+        } else {
+            const int row = 8 * k + j;
+            da = stg + lane * 64 + ((k ^ ((lane >> 1) & 3)) << 4);
+            ma = stg + (MODE == STAGE_DIAG ? 0u : kStgMirror) + row * 64 + ((g ^ ((row >> 1) & 3)) << 4);
+        }
+        if (MODE == STAGE_DIAG) {
+            // The block's own lower triangle is not part of the result: its 8 x 8 blocks are
+            // the mirrors of those above the diagonal, and the ones on it mirror themselves.
+            w[k][k] = mirror_diag(w[k][k], lane);
+            const uint32_t dummy = stg + kStgMirror + 16 * j;
+            if (g > k)
+                da = dummy;
+            if (g >= k)
+                ma = dummy;
+        }
+        stmatrix4<false>(da, w[k]);
+        stmatrix4<true>(ma, w[k]);
+    }
+}
+
+// Value arithmetic and staging of one 32 x 32 block of a specialised product: v = alpha D +
+// beta C + gamma I from the accumulator at taddr, rounded to BF16 (and lo parts) in the staging.
+//
+// The accumulator is read as matrix fragments, so the staging takes 8 stmatrix a part where the
+// row-per-thread form took 4 16-byte and 32 two-byte stores and converted every value twice.
+template <int S, int MODE>
+__device__ __forceinline__ void spec_block(const EpiHot &h, CRaw &cr, uint32_t taddr, int64_t r0,
+                                           int64_t c0, uint32_t stg, int half, int lane)
+{
+    using Spec = EpiSpec<S>;
+    float v[2][16];
+    tmem_ld_frag32(taddr, v[0]);
+    tmem_ld_frag32(taddr + (16u << 16), v[1]);
+    tmem_ld_wait();
+    const bool edge = h.N - c0 < 32;
+    uint32_t w[4][4];
+    float x[4][4][2];
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const __nv_bfloat162 *b = reinterpret_cast<const __nv_bfloat162 *>(&cr.q[4 * half + q]);
+    for (int k = 0; k < 4; ++k)
 #pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    const float2 f = __bfloat1622float2(b[j]);
-                    v[q * 8 + 2 * j] += beta * f.x;
-                    v[q * 8 + 2 * j + 1] += beta * f.y;
+        for (int g = 0; g < 4; ++g) {
+            float a = __fmul_rn(v[g >> 1][4 * k + 2 * (g & 1)], h.alpha);
+            float b = __fmul_rn(v[g >> 1][4 * k + 2 * (g & 1) + 1], h.alpha);
+            if (Spec::has_c) {
+                float2 c = bf16x2(cr.word(4 * k + g));
+                if (Spec::pair) {
+                    const float2 l = bf16x2(cr.word(16 + 4 * k + g));
+                    if (edge) {  // a row that ends in this chunk adds the parts' sum
+                        c.x += l.x;
+                        c.y += l.y;
+                    }
+                    a = fmaf(h.beta, c.x, a);
+                    b = fmaf(h.beta, c.y, b);
+                    if (!edge) {
+                        a = fmaf(h.beta, l.x, a);
+                        b = fmaf(h.beta, l.y, b);
+                    }
+                } else {
+                    a = fmaf(h.beta, c.x, a);
+                    b = fmaf(h.beta, c.y, b);
                 }
             }
+            if (MODE == STAGE_DIAG && g == k) {
+                const int row = lane >> 2, col = 2 * (lane & 3);
+                if (row == col)
+                    a += h.gamma;
+                if (row == col + 1)
+                    b += h.gamma;
+            }
+            const __nv_bfloat162 h2 = __floats2bfloat162_rn(a, b);
+            w[k][g] = *reinterpret_cast<const uint32_t *>(&h2);
+            if (Spec::pair) {
+                x[k][g][0] = a - __low2float(h2);
+                x[k][g][1] = b - __high2float(h2);
+            }
         }
-        return;
+    stage_part<MODE>(w, stg, half, lane);
+    if (Spec::pair) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+#pragma unroll
+            for (int g = 0; g < 4; ++g) {
+                const __nv_bfloat162 l2 = __floats2bfloat162_rn(x[k][g][0], x[k][g][1]);
+                w[k][g] = *reinterpret_cast<const uint32_t *>(&l2);
+            }
+        stage_part<MODE>(w, stg + kStgLo, half, lane);
     }
-    const int64_t off = r * h.ldc + c0;
-    const __nv_bfloat16 *ph = static_cast<const __nv_bfloat16 *>(h.c0) + off;
-    const __nv_bfloat16 *pl = static_cast<const __nv_bfloat16 *>(h.c1) + off;
-#pragma unroll
-    for (int i = 0; i < 32; ++i)
-        if (i < ncol) {
-            float x = __bfloat162float(ph[i]);
-            if (CK == C_PAIR)
-                x += __bfloat162float(pl[i]);
-            v[i] += beta * x;
-        }
-}
-
-// epilogue_finish for the specialised kinds (output kind OK): the identity term on the
-// diagonal of a symmetric product, then TMA stores of the block, its mirror (symmetric,
-// off the diagonal) or its transposed copy; diagonal blocks of symmetric products are
-// stored whole from shared memory with their upper triangle mirrored, as in the generic
-// path.
-template <int NSTG, int OK, bool SYM, bool HAST>
-__device__ __forceinline__ void epilogue_finish_spec(const EpiHot &h, int64_t r0, int64_t c0,
-                                                     float *v, uint8_t *stg, int &slot, int lane)
-{
-    if (SYM) {
-        if (r0 == c0) {
-            const float g = h.gamma;
-#pragma unroll
-            for (int i = 0; i < 32; ++i)
-                if (i == lane)
-                    v[i] += g;
-            if (lane == 0)
-                bulk_wait_read0();
-            __syncwarp();
-            float *st = reinterpret_cast<float *>(stg);
-#pragma unroll
-            for (int i = 0; i < 32; ++i)
-                st[xs_idx(lane, i)] = v[i];
-            __syncwarp();
-            store_block(st, OK, h.o0, h.o1, h.ldo, r0, c0, h.M, h.N, false, true, lane);
-            __syncwarp();
-            return;
-        }
-        tma_store_block<NSTG>(v, OK, false, &h.maps[0], &h.maps[1], (int)r0, (int)c0, stg, slot, lane);
-        tma_store_block<NSTG>(v, OK, true, &h.maps[0], &h.maps[1], (int)r0, (int)c0, stg, slot, lane);
-        return;
-    }
-    tma_store_block<NSTG>(v, OK, false, &h.maps[0], &h.maps[1], (int)r0, (int)c0, stg, slot, lane);
-    if (HAST)
-        tma_store_block<NSTG>(v, OK, true, &h.maps[2], &h.maps[3], (int)r0, (int)c0, stg, slot, lane);
 }
 
 // Load the epilogue fields of problem P (with the per-call fields of a grouped or
@@ -787,6 +834,7 @@ __device__ __forceinline__ void load_hot(EpiHot &h, const TcProblem &P, const Ca
     h.sym = P.sym;
     h.otma = P.o_tma;
     h.ttma = P.t_tma;
+    h.wide_tma = P.u_tma;
     h.c_kind = e.c_kind;
     h.c_trans = e.c_trans;
     h.o_kind = e.o_kind;
@@ -816,17 +864,38 @@ __device__ __forceinline__ void load_hot(EpiHot &h, const TcProblem &P, const Ca
 
 constexpr int kRingTiles = 4;  // fused launches: tiles in flight between the roles
 
-// A tile handed from the scheduler to the other roles (and to the peer CTA of a pair): its
-// operands' dependencies are met, its epilogue's scales computed.
+// A tile handed from the scheduler to the other roles (and to the peer CTA of a pair), with its
+// epilogue's scales and what the producer and the MMA issuer would otherwise load from the
+// problem table between two tiles.
 struct RingTile {
     int tile;  // index in the launch (-1: no more tiles)
     int prob;  // -1: nothing to compute
     int tm, tn;
     float alpha, beta, gamma;
-    int pad;
+    int geom;  // see pack_geom
 };
 
-template <int BN, int STAGES, bool CHAIN, bool PAIR, int NSTG, bool STRIPS>
+// k-blocks of a segment in bits 0..15 (K < 2^21), segments in 16..17, their L and R parts in
+// 18..20 and 21..23, e4m3 operands in 24, "the operands' dependencies are met" in 25.
+constexpr int kGeomReady = 1 << 25;
+__device__ __forceinline__ int pack_geom(const TcProblem &P)
+{
+    // A k-block is one 128-byte swizzle row: 64 BF16 or 128 e4m3 elements.
+    const int kshift = P.fp8 ? 7 : 6;
+    int g = (P.K + (1 << kshift) - 1) >> kshift;
+    g |= P.nseg << 16 | (P.fp8 ? 1 << 24 : 0);
+#pragma unroll
+    for (int k = 0; k < 3; ++k)
+        g |= P.segL[k] << (18 + k) | P.segR[k] << (21 + k);
+    return g;
+}
+__device__ __forceinline__ int geom_kblocks(int g) { return g & 0xffff; }
+__device__ __forceinline__ int geom_segs(int g) { return (g >> 16) & 3; }
+__device__ __forceinline__ int geom_l(int g, int sg) { return (g >> (18 + sg)) & 1; }
+__device__ __forceinline__ int geom_r(int g, int sg) { return (g >> (21 + sg)) & 1; }
+__device__ __forceinline__ bool geom_fp8(int g) { return (g >> 24) & 1; }
+
+template <int BN, int STAGES, bool CHAIN, bool PAIR, bool STRIPS>
 __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_constant__ TcLaunch L)
 {
     static_assert(!STRIPS || CHAIN, "strip dependencies exist in fused launches only");
@@ -840,8 +909,8 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
     constexpr int TILE_ROWS = PAIR ? 2 * kBM : kBM;
     uint8_t *sA = smem;
     uint8_t *sB = smem + STAGES * A_BYTES;
-    uint8_t *stage_all = sB + STAGES * B_BYTES;  // kEpiWarps x NSTG x 4 KiB, 1024-aligned
-    uint64_t *full = reinterpret_cast<uint64_t *>(stage_all + kEpiWarps * NSTG * 4096);
+    uint8_t *stage_all = sB + STAGES * B_BYTES;  // 1024-aligned
+    uint64_t *full = reinterpret_cast<uint64_t *>(stage_all + kEpiWarps * kStgBytes);
     uint64_t *empty = full + STAGES;
     uint64_t *tfull = empty + STAGES;
     uint64_t *tempty = tfull + 2;
@@ -850,8 +919,8 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
     volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_slot + 1);
     int *skip_flag = reinterpret_cast<int *>(tmem_slot + 2);
     // Fused launches: the ring of tiles from the scheduler to the other roles; pdone[i]: the
-    // epilogue warps' parts of the tile in entry i are in global memory; ptaken: the producer
-    // has read its latest entry.
+    // epilogue warps' parts of the tile in entry i are in global memory; ptaken: the producer's
+    // latest tile can start.
     uint64_t *rfull = reinterpret_cast<uint64_t *>(
         (reinterpret_cast<uintptr_t>(tmem_slot + 3) + 7) & ~static_cast<uintptr_t>(7));
     uint64_t *rempty = rfull + kRingTiles;
@@ -946,6 +1015,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
                 if (t >= 0)
                     tc = decode_tile<BN, TILE_ROWS, STRIPS>(L, t, hint);
                 EpiScales sc{1.f, 0.f, 0.f};
+                int geom = 0;
                 bool ok = true;
                 if (tc.valid) {
                     const TcProblem &P = prob_at(L, tc.prob);
@@ -958,15 +1028,27 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
                         asm volatile("prefetch.L1 [%0];" ::"l"(pb + 128 * k));
                     prefetch_tensormap(&P.mapL[P.segL[0]]);
                     prefetch_tensormap(&P.mapR[P.segR[0]]);
-                    // Operands are results of earlier problems: wait until they are complete
-                    // (whole problems), or until the strips this tile reads are (L: the strip
-                    // of this tile's row, R: of its column).
+                    geom = pack_geom(P);
+                    // Operands are results of earlier problems. Strip launches wait here until
+                    // the strips this tile reads are complete (L: the strip of this tile's row,
+                    // R: of its column), and so do tiles whose scales come from a norm. Other
+                    // tiles are handed on; where their dependencies are not met yet the producer
+                    // waits itself, which leaves no hand-over between the last counter and the
+                    // first copy.
+                    const bool wait_here = STRIPS || P.ep.theta_src;
+                    bool ready = true;
                     if (!STRIPS || tc.prob != dep_prob) {  // strips: once per problem, counts only grow
                         for (int d = 0; d < 2 && ok; ++d)
-                            if (P.dep[d] >= 0)
-                                ok = wait_counter(&L.done[P.dep[d]], P.dep_target[d], abort_flag,
-                                                  status0, dep_limit(L));
+                            if (P.dep[d] >= 0) {
+                                if (wait_here)
+                                    ok = wait_counter(&L.done[P.dep[d]], P.dep_target[d], abort_flag,
+                                                      status0, dep_limit(L));
+                                else
+                                    ready = ready && ld_acquire_gpu(&L.done[P.dep[d]]) >= P.dep_target[d];
+                            }
                     }
+                    if (ready)
+                        geom |= kGeomReady;
                     if (STRIPS) {
                         if (tc.prob != dep_prob) {
                             dep_prob = tc.prob;
@@ -991,16 +1073,16 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
                     t = -1;
                     tc.valid = false;
                 }
-                const int ent[7] = {t, tc.valid ? tc.prob : -1, tc.tm, tc.tn, __float_as_int(sc.alpha),
-                                    __float_as_int(sc.beta), __float_as_int(sc.gamma)};
+                const int ent[8] = {t, tc.valid ? tc.prob : -1, tc.tm, tc.tn, __float_as_int(sc.alpha),
+                                    __float_as_int(sc.beta), __float_as_int(sc.gamma), geom};
                 volatile int *w = reinterpret_cast<volatile int *>(&ring[ri]);
 #pragma unroll
-                for (int k = 0; k < 7; ++k)
+                for (int k = 0; k < 8; ++k)
                     w[k] = ent[k];
                 if (PAIR) {
                     const uint32_t pw = peer_addr((const void *)&ring[ri], 1);
 #pragma unroll
-                    for (int k = 0; k < 7; ++k)
+                    for (int k = 0; k < 8; ++k)
                         st_remote_u32(pw + 4 * k, ent[k]);
                     mbar_arrive_remote(peer_addr(&rfull[ri], 1));
                 }
@@ -1065,6 +1147,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
         int hint = 0;
         for (int t = t_first; ok; t += t_step) {
             TileCoord tc;
+            int geom = 0;
             if (CHAIN) {
                 if (!wait_bar<PAIR>(&rfull[ri], rphase, abort_flag, status0, kWaitTimeoutNs))
                     break;
@@ -1073,15 +1156,18 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
                 tc.tm = ring[ri].tm;
                 tc.tn = ring[ri].tn;
                 tc.valid = tc.prob >= 0;
+                geom = ring[ri].geom;
                 ring_release(ri);
-                if (!PAIR || leader)
-                    mbar_arrive(ptaken);
                 if (++ri == kRingTiles) {
                     ri = 0;
                     rphase ^= 1u;
                 }
+                // The scheduler takes the next tile once this one can start: a CTA holding two
+                // tiles that wait would keep work from CTAs that are idle.
                 if (t < 0)
                     break;
+                if (!tc.valid && (!PAIR || leader))
+                    mbar_arrive(ptaken);
             } else {
                 if (t >= total)
                     break;
@@ -1090,16 +1176,26 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
             if (!tc.valid)
                 continue;
             const TcProblem &P = prob_at(L, tc.prob);
-            // A k-block is one 128-byte swizzle row: 64 BF16 or 128 e4m3 elements.
-            const int kshift = P.fp8 ? 7 : 6;
-            const int kblocks = (P.K + (1 << kshift) - 1) >> kshift;
+            if (!CHAIN)
+                geom = pack_geom(P);
+            const int kshift = geom_fp8(geom) ? 7 : 6, kblocks = geom_kblocks(geom);
             const int row0 = (PAIR ? 2 * tc.tm + (int)rank : tc.tm) * kBM;
             const int col0 = tc.tn * BN + (int)rank * B_ROWS;
-            if (CHAIN)
-                fence_async_global();  // the TMA reads below come after the scheduler's acquire
-            for (int sg = 0; sg < P.nseg && ok; ++sg) {
-                const CUtensorMap *mL = &P.mapL[P.segL[sg]];
-                const CUtensorMap *mR = &P.mapR[P.segR[sg]];
+            if (CHAIN) {
+                if (!(geom & kGeomReady))
+                    for (int d = 0; d < 2 && ok; ++d)
+                        if (P.dep[d] >= 0)
+                            ok = wait_counter(&L.done[P.dep[d]], P.dep_target[d], abort_flag, status0,
+                                              dep_limit(L));
+                if (!ok)
+                    break;
+                if (!PAIR || leader)
+                    mbar_arrive(ptaken);
+                fence_async_global();  // the TMA reads below come after the acquire
+            }
+            for (int sg = 0; sg < geom_segs(geom) && ok; ++sg) {
+                const CUtensorMap *mL = &P.mapL[geom_l(geom, sg)];
+                const CUtensorMap *mR = &P.mapR[geom_r(geom, sg)];
                 for (int kb = 0; kb < kblocks; ++kb) {
                     if (!wait_bar<PAIR>(&empty[stage], phase ^ 1u, abort_flag, status0, kWaitTimeoutNs)) {
                         ok = false;
@@ -1149,6 +1245,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
         int hint = 0;
         for (int t = t_first; ok; t += t_step) {
             TileCoord tc;
+            int geom = 0;
             if (CHAIN) {
                 if (!mbar_wait(&rfull[ri], rphase, abort_flag, status0, kWaitTimeoutNs))
                     break;
@@ -1157,6 +1254,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
                 tc.tm = ring[ri].tm;
                 tc.tn = ring[ri].tn;
                 tc.valid = tc.prob >= 0;
+                geom = ring[ri].geom;
                 ring_release(ri);
                 if (++ri == kRingTiles) {
                     ri = 0;
@@ -1168,10 +1266,11 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
                 if (t >= total)
                     break;
                 tc = decode_tile<BN, TILE_ROWS, STRIPS>(L, t, hint);
+                if (tc.valid)
+                    geom = pack_geom(prob_at(L, tc.prob));
             }
             if (!tc.valid)
                 continue;
-            const TcProblem &P = prob_at(L, tc.prob);
             if (!wait_bar<PAIR>(&tempty[buf], tphase ^ 1u, abort_flag, status0, kWaitTimeoutNs))
                 break;
             tc_fence_after();
@@ -1183,9 +1282,9 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
             auto k_loop = [&](auto f8_tag) -> bool {
                 constexpr bool F8 = decltype(f8_tag)::value;
                 constexpr uint32_t id = F8 ? idesc_e4m3(TILE_ROWS, BN) : idesc_bf16(TILE_ROWS, BN);
-                const int kblocks = F8 ? (P.K + 2 * kBK - 1) / (2 * kBK) : (P.K + kBK - 1) / kBK;
+                const int kblocks = geom_kblocks(geom), segs = geom_segs(geom);
                 uint32_t acc = 0;
-                for (int sg = 0; sg < P.nseg; ++sg) {
+                for (int sg = 0; sg < segs; ++sg) {
                     for (int kb = 0; kb < kblocks; ++kb) {
                         if (!mbar_wait(&full[stage], phase, abort_flag, status0, kWaitTimeoutNs))
                             return false;
@@ -1220,7 +1319,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
                 }
                 return true;
             };
-            ok = P.fp8 ? k_loop(BoolTag<true>{}) : k_loop(BoolTag<false>{});
+            ok = geom_fp8(geom) ? k_loop(BoolTag<true>{}) : k_loop(BoolTag<false>{});
             if (!ok)
                 break;
             if (PAIR)
@@ -1243,7 +1342,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
         // ------------------------------------------------ epilogue
         const int quad = warp & 3;  // TMEM lane quadrant this warp may access
         const int half = (warp - 2) >> 2;  // two warps per quadrant split the column chunks
-        uint8_t *stage_buf = stage_all + (warp - 2) * NSTG * 4096;
+        uint8_t *stage_buf = stage_all + (warp - 2) * kStgBytes;
         int slot = 0;  // next staging slot of this warp
         int buf = 0;
         uint32_t tphase = 0;
@@ -1322,64 +1421,113 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
             const int64_t warp_row0 = (int64_t)tc.tm * kBM + quad * 32;
             const int64_t row = warp_row0 + lane;
             const bool row_ok = row < h.M;
-            // This warp's 32-column chunks: every other one, skipping chunks right of
-            // N or wholly below the diagonal (warp-uniform).
+            // This warp's 32-column chunks: both of every other 64-column unit, skipping chunks
+            // right of N or wholly below the diagonal (warp-uniform).
             auto next_chunk = [&](int ch) {
-                for (; ch < BN / 32; ch += 2) {
+                for (; ch < BN / 32; ch += (ch & 1) ? 3 : 1) {
                     const int64_t c0 = (int64_t)tc.tn * BN + ch * 32;
                     if (c0 < h.N && warp_row0 < h.M && !(h.sym && warp_row0 > c0 + 31))
                         break;
                 }
                 return ch;
             };
+            auto after = [&](int ch) { return next_chunk(ch + ((ch & 1) ? 3 : 1)); };
             auto full_row = [&](int ch) {
                 return row_ok && (int64_t)h.N - ((int64_t)tc.tn * BN + ch * 32) >= 32;
             };
-            int ch = next_chunk(half);
+            int ch = next_chunk(2 * half);
             // The first chunk's C is loaded while the accumulator is still being computed.
             CRaw cr;
             bool cvec = false;
-            if (ch < BN / 32)
-                cvec = c_load(h, row, (int64_t)tc.tn * BN + ch * 32, full_row(ch), cr);
+            if (ch < BN / 32) {
+                if (spec == 1)
+                    c_load_frag<false>(h, warp_row0, (int64_t)tc.tn * BN + ch * 32, lane, cr);
+                else if (spec == 4)
+                    c_load_frag<true>(h, warp_row0, (int64_t)tc.tn * BN + ch * 32, lane, cr);
+                else if (spec < 0)
+                    cvec = c_load(h, row, (int64_t)tc.tn * BN + ch * 32, full_row(ch), cr);
+            }
             if (!wait_bar<PAIR>(&tfull[buf], tphase, abort_flag, status0, kWaitTimeoutNs))
                 break;
             tc_fence_after();
             double nrm = 0.0;
+            const uint32_t acc0 = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(buf * BN);
             // The chunk loop, one copy per product kind (epi_spec, chosen once per tile):
             // the specialised copies carry no tests of output, C, norm and copy kinds.
             auto chunk_loop = [&](auto spec_tag) {
                 using Spec = decltype(spec_tag);
 #pragma unroll 1
                 while (ch < BN / 32) {
-                    const int nx = next_chunk(ch + 2);
+                    const int nx = after(ch);
                     const int64_t c0 = (int64_t)tc.tn * BN + ch * 32;
-                    const int64_t rem = (int64_t)h.N - c0;
-                    float v[32];
-                    tmem_ld32(tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(buf * BN + ch * 32),
-                              v);
-#pragma unroll
-                    for (int i = 0; i < 32; ++i)
-                        v[i] *= h.alpha;
                     if constexpr (Spec::generic) {
+                        const int64_t rem = (int64_t)h.N - c0;
+                        float v[32];
+                        tmem_ld32(acc0 + (uint32_t)(ch * 32), v);
+#pragma unroll
+                        for (int i = 0; i < 32; ++i)
+                            v[i] *= h.alpha;
                         c_apply(h, cr, cvec, row, c0, rem < 32 ? (int)rem : 32, row_ok, v);
                         // The next chunk's C is in flight while this chunk is stored.
                         if (nx < BN / 32)
                             cvec = c_load(h, row, (int64_t)tc.tn * BN + nx * 32, full_row(nx), cr);
-                        epilogue_finish<NSTG>(h, warp_row0, c0, v, nrm, stage_buf, slot, lane);
+                        epilogue_finish<kStgSlots>(h, warp_row0, c0, v, nrm, stage_buf, slot, lane);
                     } else {
-                        if constexpr (Spec::ckind != C_NONE) {
-                            c_apply_spec<Spec::ckind>(h, cr, cvec, row, c0, rem < 32 ? (int)rem : 32,
-                                                      row_ok, v);
-                            if (nx < BN / 32)
-                                cvec = c_load_spec<Spec::ckind>(h, row, (int64_t)tc.tn * BN + nx * 32,
-                                                                full_row(nx), cr);
+                        constexpr int S = Spec::code;
+                        const uint32_t stg = smem_u32(stage_buf);
+                        const bool meets = Spec::sym && (c0 & ~(int64_t)63) < warp_row0 + 32;
+                        const bool unit = !Spec::pair && !meets;  // staged with its neighbour
+                        if (!unit || !(ch & 1)) {  // the staging's last stores have been read
+                            if (lane == 0)
+                                bulk_wait_read0();
+                            __syncwarp();
                         }
-                        epilogue_finish_spec<NSTG, Spec::okind, Spec::sym, Spec::has_t>(
-                            h, warp_row0, c0, v, stage_buf, slot, lane);
+                        const bool diag = Spec::sym && c0 == warp_row0;
+                        const uint32_t ta = acc0 + (uint32_t)(ch * 32);
+                        if (unit) {
+                            if constexpr (!Spec::pair)
+                                spec_block<S, STAGE_UNIT>(h, cr, ta, warp_row0, c0, stg, ch & 1, lane);
+                        } else if (diag) {
+                            if constexpr (Spec::sym)
+                                spec_block<S, STAGE_DIAG>(h, cr, ta, warp_row0, c0, stg, 0, lane);
+                        } else {
+                            spec_block<S, STAGE_BLOCK>(h, cr, ta, warp_row0, c0, stg, 0, lane);
+                        }
+                        // The next chunk's C is in flight while this chunk is stored.
+                        if (Spec::has_c && nx < BN / 32)
+                            c_load_frag<Spec::pair>(h, warp_row0, (int64_t)tc.tn * BN + nx * 32, lane, cr);
+                        if (!unit || (nx >> 1) != (ch >> 1)) {  // a block, or a unit's last chunk
+                            fence_async_smem();
+                            __syncwarp();
+                            if (lane == 0) {
+                                const int x = unit ? (int)(c0 & ~(int64_t)63) : (int)c0, y = (int)warp_row0;
+                                const CUtensorMap *m = h.maps;
+                                if (unit) {
+                                    tma_store_2d(&m[4], x, y, stage_buf);
+                                    tma_store_2d(&m[5], y, x, stage_buf + kStgMirror64);
+                                } else {
+                                    const CUtensorMap *mm = Spec::sym ? m : m + 2;
+                                    tma_store_2d(&m[0], x, y, stage_buf);
+                                    if (!diag)
+                                        tma_store_2d(&mm[0], y, x, stage_buf + kStgMirror);
+                                    if (Spec::pair) {
+                                        tma_store_2d(&m[1], x, y, stage_buf + kStgLo);
+                                        if (!diag)
+                                            tma_store_2d(&mm[1], y, x, stage_buf + kStgLo + kStgMirror);
+                                    }
+                                }
+                                bulk_commit();
+                            }
+                        }
                     }
                     ch = nx;
                 }
             };
+            if (!CHAIN) {  // the previous tile's stores have read the staging
+                if (lane == 0)
+                    bulk_wait_read0();
+                __syncwarp();
+            }
             switch (spec) {
             case 0: chunk_loop(EpiSpec<0>{}); break;
             case 1: chunk_loop(EpiSpec<1>{}); break;
@@ -1440,25 +1588,26 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
     }
 }
 
-static_assert(offsetof(TcProblem, mapT) == offsetof(TcProblem, mapO) + 2 * sizeof(CUtensorMap),
-              "the epilogue addresses mapO[0..1] and mapT[0..1] as one array");
+static_assert(offsetof(TcProblem, mapT) == offsetof(TcProblem, mapO) + 2 * sizeof(CUtensorMap) &&
+                  offsetof(TcProblem, mapU) == offsetof(TcProblem, mapT) + 2 * sizeof(CUtensorMap),
+              "the epilogue addresses mapO, mapT and mapU as one array");
 
-template <int BN, int STAGES, bool PAIR, int NSTG>
+template <int BN, int STAGES, bool PAIR>
 constexpr int smem_bytes()
 {
     return STAGES * (kBM + (PAIR ? BN / 2 : BN)) * kBK * 2 +
-           kEpiWarps * NSTG * 4096 /* epilogue staging */ + 1024 /* alignment slack */ +
+           kEpiWarps * kStgBytes /* epilogue staging */ + 1024 /* alignment slack */ +
            512 /* barriers, tile ring */;
 }
 
 // One launch of the product kernel over total_tiles tiles (tile-width code's
 // tiles: CTA pairs for kBnPair). Persistent: at most one CTA (pair) per SM (pair).
-template <int BN, int STAGES, bool CHAIN, bool PAIR, int NSTG, bool STRIPS = false>
+template <int BN, int STAGES, bool CHAIN, bool PAIR, bool STRIPS = false>
 cudaError_t launch_kernel(const TcLaunch &l, int total_tiles, int num_sms, cudaStream_t s)
 {
-    constexpr int smem = smem_bytes<BN, STAGES, PAIR, NSTG>();
+    constexpr int smem = smem_bytes<BN, STAGES, PAIR>();
     static_assert(smem <= 232448, "shared memory per CTA");
-    auto kern = tc_gemm_kernel<BN, STAGES, CHAIN, PAIR, NSTG, STRIPS>;
+    auto kern = tc_gemm_kernel<BN, STAGES, CHAIN, PAIR, STRIPS>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess)
         return e;
@@ -1503,23 +1652,15 @@ cudaError_t launch_width(const TcLaunch &l, int bn, int total_tiles, int num_sms
     // per epilogue warp, so that stores overlap; the wide tiles keep every byte for
     // pipeline stages.
     if (bn == 256)
-        return launch_kernel<256, 4, CHAIN, false, 1>(l, total_tiles, num_sms, s);
+        return launch_kernel<256, 3, CHAIN, false>(l, total_tiles, num_sms, s);
     if (bn == 128)
-        return launch_kernel<128, 5, CHAIN, false, 2>(l, total_tiles, num_sms, s);
+        return launch_kernel<128, 5, CHAIN, false>(l, total_tiles, num_sms, s);
     if (bn == kBnPair)
-        return launch_kernel<256, 6, CHAIN, true, 1>(l, total_tiles, num_sms, s);
+        return launch_kernel<256, 5, CHAIN, true>(l, total_tiles, num_sms, s);
     return cudaErrorInvalidValue;
 }
 
 } // namespace
-
-cudaError_t tc_gemm_launch_grouped(const TcLaunch &l, int bn, int total_tiles, int num_sms,
-                                   cudaStream_t s)
-{
-    TcLaunch g = l;
-    g.nprob = 0;
-    return launch_width<false>(g, bn, total_tiles, num_sms, s);
-}
 
 cudaError_t tc_gemm_launch_fused(const TcLaunch &l, int bn, int total_tiles, int num_sms,
                                  cudaStream_t s, bool strips)
@@ -1528,9 +1669,9 @@ cudaError_t tc_gemm_launch_fused(const TcLaunch &l, int bn, int total_tiles, int
     g.nprob = 0;
     if (strips) {  // square tiles only: per-strip dependencies
         if (bn == 128)
-            return launch_kernel<128, 5, true, false, 2, true>(g, total_tiles, num_sms, s);
+            return launch_kernel<128, 5, true, false, true>(g, total_tiles, num_sms, s);
         if (bn == kBnPair)
-            return launch_kernel<256, 6, true, true, 1, true>(g, total_tiles, num_sms, s);
+            return launch_kernel<256, 5, true, true, true>(g, total_tiles, num_sms, s);
         return cudaErrorInvalidValue;
     }
     return launch_width<true>(g, bn, total_tiles, num_sms, s);

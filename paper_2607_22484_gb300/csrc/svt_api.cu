@@ -96,7 +96,7 @@ bool encode_e4m3_map(CUtensorMap *map, const void *ptr, int64_t rows, int64_t co
 }
 
 bool encode_store_map(CUtensorMap *map, const void *ptr, int64_t rows, int64_t cols, int64_t ld,
-                      bool f32)
+                      bool f32, int box_cols, int box_rows)
 {
     std::call_once(g_encode_once, resolve_encode);
     const int64_t esz = f32 ? 4 : 2;
@@ -105,12 +105,12 @@ bool encode_store_map(CUtensorMap *map, const void *ptr, int64_t rows, int64_t c
         return false;
     cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
     cuuint64_t strides[1] = {(cuuint64_t)(ld * esz)};
-    cuuint32_t box[2] = {32, 32};
+    cuuint32_t box[2] = {(cuuint32_t)box_cols, (cuuint32_t)box_rows};
     cuuint32_t estr[2] = {1, 1};
     CUresult r = g_encode(map, f32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16,
                           2, const_cast<void *>(ptr), dims, strides, box, estr,
                           CU_TENSOR_MAP_INTERLEAVE_NONE,
-                          f32 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B,
+                          box_cols * esz == 128 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B,
                           CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     return r == CUDA_SUCCESS;
 }
@@ -139,6 +139,13 @@ void attach_store_maps(TcProblem &p)
             ok = encode_store_map(&p.mapT[1], e.t1, p.N, p.M, e.ldt, false);
         p.t_tma = ok ? 1 : 0;
     }
+    // 64-column units of a BF16 output: the mirror goes to the output itself (symmetric) or to
+    // the transposed copy.
+    p.u_tma = e.o_kind == O_PAIR ? 1 : 0;
+    if (e.o_kind == O_BF16 && p.o_tma && !e.o_trans && (p.sym || p.t_tma))
+        p.u_tma = encode_store_map(&p.mapU[0], e.o0, p.M, p.N, e.ldo, false, 64, 32) &&
+                  (p.sym ? encode_store_map(&p.mapU[1], e.o0, p.M, p.N, e.ldo, false, 32, 64)
+                         : encode_store_map(&p.mapU[1], e.t0, p.N, p.M, e.ldt, false, 32, 64));
 }
 
 

@@ -99,7 +99,11 @@ struct TcProblem {
     CUtensorMap mapR[2];             // R operands, box 64 x BN
     CUtensorMap mapO[2];             // output hi/lo (or FP32), box 32 x 32, for TMA stores
     CUtensorMap mapT[2];             // transposed copy hi/lo, box 32 x 32
+    CUtensorMap mapU[2];             // BF16 output's 64-column units: in place (box 64 x 32), and
+                                     // mirrored or as the transposed copy (box 32 x 64)
     int o_tma, t_tma;                // 1: store through mapO / mapT
+    int u_tma;                       // 1: mapU holds what a BF16 output's units need (or pairs,
+                                     // which have no units)
     int patch, call_idx;             // grouped launches: fields taken from calls[call_idx]
     // Fused (chained) launches: completion counter index of this problem, and the
     // problems whose results it reads with the counts that mean "complete".
@@ -172,10 +176,6 @@ int tc_num_tiles(const TcProblem &p, int bn);
 // launch: tiles with work, times the CTAs per tile.
 int tc_valid_ctas(const TcProblem &p, int bn);
 cudaError_t tc_gemm_launch(const TcLaunch &l, int bn, int num_sms, cudaStream_t s);
-// Grouped launch: l.gtab / l.gstart / l.gcount / l.calls point to device memory;
-// total_tiles (host copy of gstart[gcount]) sizes the grid.
-cudaError_t tc_gemm_launch_grouped(const TcLaunch &l, int bn, int total_tiles, int num_sms,
-                                   cudaStream_t s);
 // Fused launch: l.gtab / l.gstart / l.gcount hold every product of a solve in
 // dependency order; l.tile_counter and l.done point to zeroed device counters.
 // strips: the table carries per-strip dependencies (square tiles: bn 128 or kBnPair).
@@ -246,9 +246,10 @@ bool encode_bf16_map(CUtensorMap *map, const void *ptr, int64_t rows, int64_t co
 // e4m3 operand loads (FP8 experiment): box 128 (K) x box_rows, 128-byte swizzle.
 bool encode_e4m3_map(CUtensorMap *map, const void *ptr, int64_t rows, int64_t cols, int64_t ld,
                      int box_rows);
-// Epilogue stores: BF16 (64-byte swizzle) or FP32 (128-byte swizzle), box 32 x 32.
+// Epilogue stores, box box_cols x box_rows: BF16 or FP32, swizzled by the box's row bytes (64
+// or 128).
 bool encode_store_map(CUtensorMap *map, const void *ptr, int64_t rows, int64_t cols, int64_t ld,
-                      bool f32);
+                      bool f32, int box_cols = 32, int box_rows = 32);
 // Fill mapO / mapT of a problem from its epilogue's outputs where they qualify.
 void attach_store_maps(TcProblem &p);
 
