@@ -504,7 +504,7 @@ __device__ __forceinline__ void tma_store_block(const float *x, int kind, bool t
     uint8_t *stg0 = stg_base + slot * 4096, *stg1 = stg0 + 2048;
     if (++slot == NSTG)
         slot = 0;
-    if (lane == 0)
+    if (elect_one())
         bulk_wait_read<NSTG - 1>();  // the store that last used this slot has read it
     __syncwarp();
     if (kind == O_F32) {
@@ -551,7 +551,7 @@ __device__ __forceinline__ void tma_store_block(const float *x, int kind, bool t
     }
     fence_async_smem();
     __syncwarp();
-    if (lane == 0) {
+    if (elect_one()) {
         const int sx = trans ? r0 : c0, sy = trans ? c0 : r0;
         tma_store_2d(m0, sx, sy, stg0);
         if (kind == O_PAIR)
@@ -615,7 +615,7 @@ __device__ __forceinline__ void epilogue_finish(const EpiHot &h, int64_t r0, int
     if (!need_plain)
         return;
     // Coalesced plain-store path: stage with a swizzled pitch, then whole row segments.
-    if (lane == 0)
+    if (elect_one())
         bulk_wait_read0();
     __syncwarp();
     float *st = reinterpret_cast<float *>(stg);
@@ -697,6 +697,8 @@ __device__ __forceinline__ void c_load_frag(const EpiHot &h, int64_t r0, int64_t
 // How a specialised epilogue stages a 32 x 32 block for its TMA stores: as half of a 64-column
 // unit (BF16 only: one 64 x 32 box in place, one 32 x 64 box mirrored), by itself, or by itself
 // on the diagonal of a symmetric product (one box holding both triangles).
+// A warp's TMA stores and the waits for them run in one elected lane (the same for a given mask:
+// bulk groups belong to the thread that commits them).
 constexpr int kStgSlots = 2;                  // 4 KiB staging slots of an epilogue warp
 constexpr int kStgBytes = kStgSlots * 4096;
 
@@ -1136,7 +1138,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
                     break;
             }
         }
-    } else if (warp == 0 && lane == 0) {
+    } else if (warp == 0) {
         // ------------------------------------------------ TMA producer
         int stage = 0;
         uint32_t phase = 0;
@@ -1149,7 +1151,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
             TileCoord tc;
             int geom = 0;
             if (CHAIN) {
-                if (!wait_bar<PAIR>(&rfull[ri], rphase, abort_flag, status0, kWaitTimeoutNs))
+                if (!wait_warp<PAIR>(&rfull[ri], rphase, abort_flag, status0, kWaitTimeoutNs))
                     break;
                 t = ring[ri].tile;
                 tc.prob = ring[ri].prob;
@@ -1157,7 +1159,9 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
                 tc.tn = ring[ri].tn;
                 tc.valid = tc.prob >= 0;
                 geom = ring[ri].geom;
-                ring_release(ri);
+                __syncwarp();
+                if (elect_one())
+                    ring_release(ri);
                 if (++ri == kRingTiles) {
                     ri = 0;
                     rphase ^= 1u;
@@ -1166,7 +1170,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
                 // tiles that wait would keep work from CTAs that are idle.
                 if (t < 0)
                     break;
-                if (!tc.valid && (!PAIR || leader))
+                if (!tc.valid && (!PAIR || leader) && elect_one())
                     mbar_arrive(ptaken);
             } else {
                 if (t >= total)
@@ -1182,14 +1186,17 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
             const int row0 = (PAIR ? 2 * tc.tm + (int)rank : tc.tm) * kBM;
             const int col0 = tc.tn * BN + (int)rank * B_ROWS;
             if (CHAIN) {
-                if (!(geom & kGeomReady))
-                    for (int d = 0; d < 2 && ok; ++d)
-                        if (P.dep[d] >= 0)
-                            ok = wait_counter(&L.done[P.dep[d]], P.dep_target[d], abort_flag, status0,
-                                              dep_limit(L));
+                if (!(geom & kGeomReady)) {
+                    if (lane == 0)
+                        for (int d = 0; d < 2 && ok; ++d)
+                            if (P.dep[d] >= 0)
+                                ok = wait_counter(&L.done[P.dep[d]], P.dep_target[d], abort_flag,
+                                                  status0, dep_limit(L));
+                    ok = __shfl_sync(0xffffffffu, (int)ok, 0);
+                }
                 if (!ok)
                     break;
-                if (!PAIR || leader)
+                if ((!PAIR || leader) && elect_one())
                     mbar_arrive(ptaken);
                 fence_async_global();  // the TMA reads below come after the acquire
             }
@@ -1197,11 +1204,13 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
                 const CUtensorMap *mL = &P.mapL[geom_l(geom, sg)];
                 const CUtensorMap *mR = &P.mapR[geom_r(geom, sg)];
                 for (int kb = 0; kb < kblocks; ++kb) {
-                    if (!wait_bar<PAIR>(&empty[stage], phase ^ 1u, abort_flag, status0, kWaitTimeoutNs)) {
+                    if (!wait_warp<PAIR>(&empty[stage], phase ^ 1u, abort_flag, status0, kWaitTimeoutNs)) {
                         ok = false;
                         break;
                     }
-                    if (PAIR) {
+                    if (!elect_one()) {
+                        // the elected lane issues the copies
+                    } else if (PAIR) {
                         // Both CTAs' bytes complete on the leader's barrier.
                         const uint32_t fb = peer_addr(&full[stage], 0);
                         if (leader)
@@ -1233,8 +1242,12 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
                     mbar_wait_cluster(&empty[s], (issued_parity >> s) & 1u, &no_abort, nullptr,
                                       kWaitTimeoutNs / 4);
             }
-    } else if (warp == 1 && lane == 0 && (!PAIR || leader)) {
+    } else if (warp == 1 && (!PAIR || leader)) {
         // ------------------------------------------------ MMA issuer
+        // The whole warp runs the loop and one elected lane issues: its operands then live in
+        // uniform registers. A loop that only lane 0 ran took 132 cycles an MMA whatever its
+        // shape, twice what a 128 x 128 x 16 needs.
+        const uint64_t desc_a = sw128_desc(smem_u32(sA)), desc_b = sw128_desc(smem_u32(sB));
         int stage = 0;
         uint32_t phase = 0;
         int buf = 0;
@@ -1247,7 +1260,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
             TileCoord tc;
             int geom = 0;
             if (CHAIN) {
-                if (!mbar_wait(&rfull[ri], rphase, abort_flag, status0, kWaitTimeoutNs))
+                if (!wait_warp<false>(&rfull[ri], rphase, abort_flag, status0, kWaitTimeoutNs))
                     break;
                 t = ring[ri].tile;
                 tc.prob = ring[ri].prob;
@@ -1255,7 +1268,9 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
                 tc.tn = ring[ri].tn;
                 tc.valid = tc.prob >= 0;
                 geom = ring[ri].geom;
-                ring_release(ri);
+                __syncwarp();
+                if (elect_one())
+                    ring_release(ri);
                 if (++ri == kRingTiles) {
                     ri = 0;
                     rphase ^= 1u;
@@ -1271,7 +1286,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
             }
             if (!tc.valid)
                 continue;
-            if (!wait_bar<PAIR>(&tempty[buf], tphase ^ 1u, abort_flag, status0, kWaitTimeoutNs))
+            if (!wait_warp<PAIR>(&tempty[buf], tphase ^ 1u, abort_flag, status0, kWaitTimeoutNs))
                 break;
             tc_fence_after();
             const uint32_t d_tmem = tmem_base + (uint32_t)(buf * BN);
@@ -1286,31 +1301,36 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
                 uint32_t acc = 0;
                 for (int sg = 0; sg < segs; ++sg) {
                     for (int kb = 0; kb < kblocks; ++kb) {
-                        if (!mbar_wait(&full[stage], phase, abort_flag, status0, kWaitTimeoutNs))
+                        if (!wait_warp<false>(&full[stage], phase, abort_flag, status0, kWaitTimeoutNs))
                             return false;
                         tc_fence_after();
-                        const uint32_t a0 = smem_u32(sA + stage * A_BYTES);
-                        const uint32_t b0 = smem_u32(sB + stage * B_BYTES);
+                        if (elect_one()) {
+                            // Descriptor addresses count 16-byte units; a K step is 32 bytes.
+                            const uint64_t a0 = desc_a + (uint32_t)(stage * (A_BYTES >> 4));
+                            const uint64_t b0 = desc_b + (uint32_t)(stage * (B_BYTES >> 4));
 #pragma unroll
-                        for (int kk = 0; kk < kBK / 16; ++kk) {
-                            const uint64_t ad = sw128_desc(a0 + kk * 32), bd = sw128_desc(b0 + kk * 32);
-                            if (F8) {
-                                if (PAIR)
-                                    mma_e4m3_pair(d_tmem, ad, bd, id, acc);
-                                else
-                                    mma_e4m3(d_tmem, ad, bd, id, acc);
-                            } else {
-                                if (PAIR)
-                                    mma_bf16_pair(d_tmem, ad, bd, id, acc);
-                                else
-                                    mma_bf16(d_tmem, ad, bd, id, acc);
+                            for (int kk = 0; kk < kBK / 16; ++kk) {
+                                const uint64_t ad = a0 + 2 * kk, bd = b0 + 2 * kk;
+                                const uint32_t on = kk == 0 ? acc : 1u;
+                                if (F8) {
+                                    if (PAIR)
+                                        mma_e4m3_pair(d_tmem, ad, bd, id, on);
+                                    else
+                                        mma_e4m3(d_tmem, ad, bd, id, on);
+                                } else {
+                                    if (PAIR)
+                                        mma_bf16_pair(d_tmem, ad, bd, id, on);
+                                    else
+                                        mma_bf16(d_tmem, ad, bd, id, on);
+                                }
                             }
-                            acc = 1;
+                            if (PAIR)
+                                mma_commit_both(&empty[stage]);
+                            else
+                                mma_commit(&empty[stage]);
                         }
-                        if (PAIR)
-                            mma_commit_both(&empty[stage]);
-                        else
-                            mma_commit(&empty[stage]);
+                        __syncwarp();
+                        acc = 1;
                         if (++stage == STAGES) {
                             stage = 0;
                             phase ^= 1u;
@@ -1322,20 +1342,26 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
             ok = geom_fp8(geom) ? k_loop(BoolTag<true>{}) : k_loop(BoolTag<false>{});
             if (!ok)
                 break;
-            if (PAIR)
-                mma_commit_both(&tfull[buf]);
-            else
-                mma_commit(&tfull[buf]);
+            if (elect_one()) {
+                if (PAIR)
+                    mma_commit_both(&tfull[buf]);
+                else
+                    mma_commit(&tfull[buf]);
+            }
+            __syncwarp();
             if (++buf == 2) {
                 buf = 0;
                 tphase ^= 1u;
             }
         }
         // Drain: every MMA issued so far completes before tensor memory is freed.
-        if (PAIR)
-            mma_commit_pair_local(drain);
-        else
-            mma_commit(drain);
+        if (elect_one()) {
+            if (PAIR)
+                mma_commit_pair_local(drain);
+            else
+                mma_commit(drain);
+        }
+        __syncwarp();
         volatile int no_abort = 0;
         mbar_wait(drain, 0, &no_abort, nullptr, kWaitTimeoutNs / 4);
     } else if (warp >= 2 && warp < kSchedWarp) {
@@ -1478,7 +1504,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
                         const bool meets = Spec::sym && (c0 & ~(int64_t)63) < warp_row0 + 32;
                         const bool unit = !Spec::pair && !meets;  // staged with its neighbour
                         if (!unit || !(ch & 1)) {  // the staging's last stores have been read
-                            if (lane == 0)
+                            if (elect_one())
                                 bulk_wait_read0();
                             __syncwarp();
                         }
@@ -1499,7 +1525,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
                         if (!unit || (nx >> 1) != (ch >> 1)) {  // a block, or a unit's last chunk
                             fence_async_smem();
                             __syncwarp();
-                            if (lane == 0) {
+                            if (elect_one()) {
                                 const int x = unit ? (int)(c0 & ~(int64_t)63) : (int)c0, y = (int)warp_row0;
                                 const CUtensorMap *m = h.maps;
                                 if (unit) {
@@ -1524,7 +1550,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
                 }
             };
             if (!CHAIN) {  // the previous tile's stores have read the staging
-                if (lane == 0)
+                if (elect_one())
                     bulk_wait_read0();
                 __syncwarp();
             }
@@ -1563,7 +1589,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
                 // ordered before lane 0's arrival by __syncwarp, its TMA stores by their
                 // completion.
                 __syncwarp();
-                if (lane == 0) {
+                if (elect_one()) {
                     bulk_wait_all0();
                     fence_async_global();
                     mbar_arrive(&pdone[entry]);
@@ -1572,7 +1598,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
             }
         }
         // All TMA stores of this warp complete before the CTA may exit.
-        if (lane == 0)
+        if (elect_one())
             bulk_wait_all0();
         __syncwarp();
     }

@@ -137,6 +137,14 @@ __device__ __forceinline__ bool wait_bar(uint64_t *bar, uint32_t parity, volatil
                    : mbar_wait(bar, parity, abort_flag, status, limit_ns);
 }
 
+// A wait by a whole warp, with one answer for all its lanes.
+template <bool CLUSTER>
+__device__ __forceinline__ bool wait_warp(uint64_t *bar, uint32_t parity, volatile int *abort_flag,
+                                          int *status, uint64_t limit_ns)
+{
+    return __all_sync(0xffffffffu, wait_bar<CLUSTER>(bar, parity, abort_flag, status, limit_ns));
+}
+
 __device__ __forceinline__ uint32_t cluster_rank()
 {
     uint32_t r;
