@@ -22,10 +22,10 @@
 // Two accumulator buffers of BN FP32 columns each let the epilogue of one tile
 // overlap the MMAs of the next.
 //
-// CTA-pair mode (PAIR): a cluster of two CTAs computes one 256 x 256 tile with
-// tcgen05.mma.cta_group::2. Each CTA stages its own 128 rows of L and one half
-// (128 rows) of the tile's R, so a pipeline stage is 32 KiB instead of 48 KiB
-// and every operand byte crosses L2 -> SM once per pair instead of once per CTA.
+// CTA-pair mode (PAIR): a cluster of two CTAs computes one 256 x 256 (or 256 x 128)
+// tile with tcgen05.mma.cta_group::2. Each CTA stages its own 128 rows of L and one half
+// (128 or 64 rows) of the tile's R, so a pipeline stage is 32 KiB instead of 48 KiB (24
+// instead of 32) and every operand byte crosses L2 -> SM once per pair instead of once per CTA.
 // The even CTA (leader) issues the MMAs for both, its barriers collect both
 // CTAs' TMA bytes and both CTAs' epilogue releases; MMA completion is multicast
 // to both CTAs, whose epilogues each drain their own 128 x 256 accumulator.
@@ -93,7 +93,7 @@ __device__ __forceinline__ const TcProblem &prob_at(const TcLaunch &L, int p)
 // Dense problems: column-major over the tile grid. Symmetric problems: only
 // tiles holding some element with row <= col; column tn holds r (tn + 1) row
 // tiles (r = BN / TM), so the first tile of column tn is r tn (tn + 1) / 2
-// (ROWMAJOR_SYM with square tiles: row-major instead, see below).
+// (tiles taller than wide, and ROWMAJOR_SYM with square tiles: see below).
 // A role's tile indices only increase, so the problem search gallops forward from
 // the previous answer (`hint`) instead of bisecting the whole table: a few
 // dependent loads of the tile prefix sums instead of log2(problems).
@@ -137,6 +137,20 @@ __device__ TileCoord decode_tile(const TcLaunch &L, int t, int &hint)
         return tc;
     }
     constexpr int r = BN / TM;
+    if (r == 0) {
+        // Tiles twice as tall as wide: columns 2 j and 2 j + 1 hold j + 1 row tiles each, the
+        // first of them from index j (j + 1) on.
+        int j = (int)((sqrtf(4.0f * (float)local + 1.0f) - 1.0f) * 0.5f);
+        while (j > 0 && j * (j + 1) > local)
+            --j;
+        while ((j + 1) * (j + 2) <= local)
+            ++j;
+        const int rem = local - j * (j + 1);
+        tc.tn = 2 * j + (rem > j ? 1 : 0);
+        tc.tm = rem > j ? rem - (j + 1) : rem;
+        tc.valid = (tc.tm < P.tiles_m) && (tc.tn < P.tiles_n);
+        return tc;
+    }
     if (ROWMAJOR_SYM && r == 1) {
         // Square tiles: row-major over the upper triangle (row tm holds columns
         // tm .. T - 1, first index tm T - tm (tm - 1) / 2), so that the strips of a
@@ -901,7 +915,7 @@ template <int BN, int STAGES, bool CHAIN, bool PAIR, bool STRIPS>
 __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_constant__ TcLaunch L)
 {
     static_assert(!STRIPS || CHAIN, "strip dependencies exist in fused launches only");
-    static_assert(!PAIR || BN == 256, "CTA pairs compute 256 x 256 tiles");
+    static_assert(!PAIR || BN == 256 || BN == 128, "CTA pairs compute 256 x 256 or 256 x 128 tiles");
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                                 ~static_cast<uintptr_t>(1023));
@@ -1683,6 +1697,8 @@ cudaError_t launch_width(const TcLaunch &l, int bn, int total_tiles, int num_sms
         return launch_kernel<128, 5, CHAIN, false>(l, total_tiles, num_sms, s);
     if (bn == kBnPair)
         return launch_kernel<256, 5, CHAIN, true>(l, total_tiles, num_sms, s);
+    if (bn == kBnPair128)
+        return launch_kernel<128, 6, CHAIN, true>(l, total_tiles, num_sms, s);
     return cudaErrorInvalidValue;
 }
 
@@ -1705,22 +1721,17 @@ cudaError_t tc_gemm_launch_fused(const TcLaunch &l, int bn, int total_tiles, int
 
 int tc_num_tiles(const TcProblem &p, int bn)
 {
-    if (!p.sym)
-        return p.tiles_m * p.tiles_n;
-    const int r = tile_cols(bn) / tile_rows(bn);
-    return r * p.tiles_n * (p.tiles_n + 1) / 2;
+    return p.sym ? sym_tiles(bn, p.tiles_n) : p.tiles_m * p.tiles_n;
 }
 
 int tc_valid_ctas(const TcProblem &p, int bn)
 {
     int n = 0;
-    if (!p.sym) {
+    if (!p.sym)
         n = p.tiles_m * p.tiles_n;
-    } else {
-        const int r = tile_cols(bn) / tile_rows(bn);
+    else
         for (int tn = 0; tn < p.tiles_n; ++tn)
-            n += std::min(r * (tn + 1), p.tiles_m);
-    }
+            n += std::min(sym_rows(bn, tn), p.tiles_m);
     return n * ctas_per_tile(bn);
 }
 

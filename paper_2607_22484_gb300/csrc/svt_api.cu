@@ -1263,20 +1263,31 @@ void evict_plans(svt_ctx *ctx, size_t max_entries)
 }
 
 // Tile mode of a fused solve when none is requested or tuned, from whole-solve timings on
-// GB300 (BF16 tier, 20 steps): 128 x 128 tiles while the small side is at most 1536 (more
-// tiles per product keep all SMs busy: 1.31x over 128 x 256 at 1024^2), CTA pairs above
-// (1.01x at 2048^2, 1.035x at 3072^2 and 4096^2, 1.04x at 8192 x 2048, 1.08x at 6144^2,
-// 8192^2 and 16384 x 4096).
-int fused_auto_width(int64_t m, int64_t n)
+// GB300 (20 steps, us; 128 x 128 tiles / pairs on 256 x 128 / pairs on 256 x 256):
+//   BF16  512^2 510 / 540 / 692, 1000^2 697 / 710 / 986, 1536^2 947 / 953 / 1164, 1792^2 1189 /
+//         1174 / 1296, 2048^2 1452 / 1405 / 1435, 2304^2 2146 / 2036 / 1800, 8192 x 512 1165 /
+//         1117 / 1391, 8192 x 2048 3146 / 2984 / 2812
+//   FP32  512^2 775 / 774 / 1056, 1000^2 1130 / 1080 / 1493, 1700^2 2390 / 2226 / 2295, 2400 x 600
+//         1321 / 1189 / 1677, 8192 x 512 2613 / 2306 / 3135, 2048^2 3248 / 3097 / 2829
+// 256 x 256 tiles move the fewest operand bytes but leave SMs without a tile until the smaller
+// side is about 1800. Below, pairs on 256 x 128 move 24 KiB per k-block and CTA where 128 x 128
+// tiles move 32, and cost about 300 cycles a tile more (the pair's barriers): they pay from 24
+// k-blocks per product on, the mean over a step of the P chain (X^T X over the larger side, Y^2
+// and X Z over the smaller), each hi/lo segment counted.
+int fused_auto_width(int64_t m, int64_t n, const Resolved &r)
 {
-    return std::min(m, n) <= 1536 ? 128 : kBnPair;
+    const int64_t M = std::max(m, n), N = std::min(m, n);
+    if (N > 1792)
+        return kBnPair;
+    const int64_t segs = r.prec == SVT_FP32 ? 3 : 1;
+    return (M + 2 * N) * segs >= 24 * 3 * kBK ? kBnPair128 : 128;
 }
 
 svt_status get_plan(svt_ctx *ctx, int64_t m, int64_t n, const Resolved &r, size_t ws_base,
                     size_t ws_avail, Plan **out, int force_bn, std::shared_ptr<Plan> *keep)
 {
     if (force_bn == 0 && r.fuse && r.prec != SVT_FP64)
-        force_bn = fused_auto_width(m, n);
+        force_bn = fused_auto_width(m, n, r);
     Key k{m, n, r.iters, r.prec, r.schedule, r.norm, r.polish, r.mode, r.hp_steps, r.ell0, r.delta,
           ws_base, force_bn, r.fuse, r.out64, r.fp8_p, r.fp8_s, r.fp8_s_y2};
     auto it = ctx->plans.find(k);
@@ -1657,9 +1668,13 @@ svt_status svt_autotune(svt_ctx_t ctx, const float *A, int64_t m, int64_t n, int
         double best = -1.0;
         int best_w = 0;
         size_t n_tc = 0;
-        for (int w = 0; w < 3 && st == SVT_OK; ++w) {
+        // The three modes, and the automatic choice where it is another one (the last).
+        std::vector<int> cand(widths, widths + 3);
+        if (fused_auto_width(m, n, r) == kBnPair128)
+            cand.push_back(kBnPair128);
+        for (size_t w = 0; w < cand.size() && st == SVT_OK; ++w) {
             Plan *plan = nullptr;
-            st = get_plan(ctx, m, n, r, 0, ctx->ws_bytes, &plan, widths[w]);
+            st = get_plan(ctx, m, n, r, 0, ctx->ws_bytes, &plan, cand[w]);
             if (st != SVT_OK)
                 break;
             if (!plan->fused)
@@ -1681,7 +1696,7 @@ svt_status svt_autotune(svt_ctx_t ctx, const float *A, int64_t m, int64_t n, int
             cudaEventElapsedTime(&t, e0, e1);
             if (best < 0.0 || t < best) {
                 best = t;
-                best_w = widths[w];
+                best_w = cand[w];
                 n_tc = plan->tc.size();
             }
         }
@@ -1691,7 +1706,8 @@ svt_status svt_autotune(svt_ctx_t ctx, const float *A, int64_t m, int64_t n, int
             return st;
         if (best_w == 0)
             return SVT_OK;  // no width runs fused: keep the automatic choice
-        choice.assign(n_tc, best_w);
+        if (best_w != kBnPair128)  // else nothing is stored: later solves choose it themselves
+            choice.assign(n_tc, best_w);
     } else {
         std::vector<double> ms[3];
         const bool prev_profile = ctx->profile;
@@ -1746,7 +1762,10 @@ svt_status svt_autotune(svt_ctx_t ctx, const float *A, int64_t m, int64_t n, int
         else
             ++it;
     }
-    ctx->tuning[tune_key(m, n, r)] = choice;
+    if (choice.empty())
+        ctx->tuning.erase(tune_key(m, n, r));
+    else
+        ctx->tuning[tune_key(m, n, r)] = choice;
     return SVT_OK;
 }
 

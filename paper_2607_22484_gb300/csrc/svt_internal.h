@@ -28,12 +28,28 @@ constexpr int kBK = 64;           // K per pipeline stage: one 128-byte swizzle 
 // Tile-width codes of the product kernel. 128 and 256: one CTA per 128 x bn
 // output tile. kBnPair: a cluster of two CTAs per 256 x 256 tile
 // (tcgen05 cta_group::2), each CTA holding 128 x 256 of it and staging half of
-// the tile's R rows.
+// the tile's R rows. kBnPair128: such a cluster per 256 x 128 tile (chosen by
+// fused_auto_width, not an option value).
 constexpr int kBnPair = 512;
-inline int tile_rows(int bn) { return bn == kBnPair ? 2 * kBM : kBM; }
-inline int tile_cols(int bn) { return bn == kBnPair ? 256 : bn; }
-inline int r_box_rows(int bn) { return bn == kBnPair ? 128 : bn; }  // R rows one CTA loads
-inline int ctas_per_tile(int bn) { return bn == kBnPair ? 2 : 1; }
+constexpr int kBnPair128 = 384;
+inline bool is_pair(int bn) { return bn == kBnPair || bn == kBnPair128; }
+inline int tile_rows(int bn) { return is_pair(bn) ? 2 * kBM : kBM; }
+inline int tile_cols(int bn) { return bn == kBnPair ? 256 : (bn == kBnPair128 ? 128 : bn); }
+inline int r_box_rows(int bn) { return is_pair(bn) ? tile_cols(bn) / 2 : bn; }  // R rows one CTA loads
+inline int ctas_per_tile(int bn) { return is_pair(bn) ? 2 : 1; }
+// Tiles of a symmetric product with n tile columns, and the row tiles of column tn: those that
+// hold some element on or above the diagonal.
+inline int sym_rows(int bn, int tn)
+{
+    return tile_cols(bn) >= tile_rows(bn) ? tile_cols(bn) / tile_rows(bn) * (tn + 1) : tn / 2 + 1;
+}
+inline int sym_tiles(int bn, int n)
+{
+    if (tile_cols(bn) >= tile_rows(bn))
+        return tile_cols(bn) / tile_rows(bn) * n * (n + 1) / 2;
+    const int j = n / 2;  // columns 2 i and 2 i + 1 hold i + 1 row tiles each
+    return j * (j + 1) + (n % 2) * (j + 1);
+}
 
 enum CKind : int { C_NONE = 0, C_BF16 = 1, C_PAIR = 2, C_F32 = 3, C_F64 = 4 };
 enum OKind : int { O_NONE = 0, O_BF16 = 1, O_PAIR = 2, O_F32 = 3, O_F64 = 4, O_E4M3 = 5 };

@@ -36,3 +36,21 @@ def test_epilogue_edges(m, n, prec):
         if first is None:
             first = y
         assert float((y - first).double().norm()) <= 1e-5 * float(first.double().norm()), o
+
+
+@pytest.mark.parametrize("m,n,prec", [(700, 523, "fp32"), (531, 900, "fp32"), (1100, 257, "fp32"),
+                                      (4100, 300, "bf16"), (260, 4300, "bf16"), (1500, 1601, "bf16"),
+                                      (2600, 130, "fp32")])
+def test_pairs_of_256x128(m, n, prec):
+    """Shapes that the automatic choice runs on CTA pairs of 256 x 128 tiles (long K), ragged in
+    both directions, against 128 x 128 tiles: 1e-5, the bound between execution paths."""
+    g = torch.Generator(device="cuda")
+    g.manual_seed(m + n)
+    a = torch.randn(m, n, generator=g, device="cuda") / max(m, n) ** 0.5
+    ctx = pkg.Context(0, workspace_bytes=pkg.workspace_bytes(m, n, prec=prec))
+    for o in (dict(), dict(mode="rank_r"), dict(polish=False), dict(schedule="ns3")):
+        sts = [torch.zeros(1, dtype=torch.int32, device="cuda") for _ in range(2)]
+        y = ctx.polar(a, 0.5, status=sts[0], prec=prec, iters=8, **o)
+        ref = ctx.polar(a, 0.5, status=sts[1], prec=prec, iters=8, tile=128, **o)
+        assert int(sts[0]) == int(sts[1]) == 0
+        assert float((y - ref).double().norm()) <= 1e-5 * float(ref.double().norm()), o
