@@ -222,12 +222,14 @@ __device__ __forceinline__ void store4_f64(void *out, int64_t row, int64_t col, 
 // (BF16 hi and optional lo parts, or FP64). 256 threads: thread t loads rows
 // (t >> 4) + 16 k, columns 4 (t & 15) .. + 3, and stores the transposed tile the same
 // way from shared memory. vec_in: A's rows 16-byte aligned; st_al: BF16 outputs
-// 8-byte aligned at columns that are multiples of 4.
+// 8-byte aligned at columns that are multiples of 4. raw: the copy that holds A itself, not
+// A / alpha (1: the same-orientation one, 2: the transposed one, 0: none).
 template <bool F64>
 __device__ __forceinline__ void split64_block(const float *__restrict__ A, int64_t m, int64_t n,
                                               int64_t lda, float tau, void *xs_hi, void *xs_lo,
                                               int64_t ld_s, void *xt_hi, void *xt_lo, int64_t ld_t,
-                                              double *scal, int bx, int by, bool vec_in, bool st_al)
+                                              double *scal, int bx, int by, bool vec_in, bool st_al,
+                                              int raw = 0)
 {
     __shared__ float tile[64][65];
     const double nrm2 = scal[SC_NRM_A2];
@@ -260,8 +262,9 @@ __device__ __forceinline__ void split64_block(const float *__restrict__ A, int64
         }
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
-            v[e] *= inv_alpha;
-            tile[li][4 * cq + e] = v[e];
+            tile[li][4 * cq + e] = raw == 2 ? v[e] : v[e] * inv_alpha;
+            if (raw != 1)
+                v[e] *= inv_alpha;
         }
         if (xs_hi && i < m && j < n) {
             if (F64)
@@ -319,11 +322,11 @@ __global__ void __launch_bounds__(256) ingest_split_kernel(const float *__restri
                                                            int64_t n, int64_t lda, float tau,
                                                            void *xs_hi, void *xs_lo, int64_t ld_s,
                                                            void *xt_hi, void *xt_lo, int64_t ld_t,
-                                                           double *scal)
+                                                           double *scal, int raw)
 {
     split64_block<F64>(A, m, n, lda, tau, xs_hi, xs_lo, ld_s, xt_hi, xt_lo, ld_t, scal, blockIdx.x,
                        blockIdx.y, rows_vec(A, lda),
-                       bf16_outs_aligned(xs_hi, xs_lo, xt_hi, xt_lo, ld_s, ld_t));
+                       bf16_outs_aligned(xs_hi, xs_lo, xt_hi, xt_lo, ld_s, ld_t), raw);
 }
 
 __global__ void finalize_kernel(double *scal, int *status, svt_status *user)
@@ -554,17 +557,17 @@ cudaError_t ingest_reduce_launch(const float *A, int64_t m, int64_t n, int64_t l
 
 cudaError_t ingest_split_launch(const float *A, int64_t m, int64_t n, int64_t lda, float tau,
                                 int f64, void *xs_hi, void *xs_lo, int64_t ld_s, void *xt_hi,
-                                void *xt_lo, int64_t ld_t, double *scal, int *status,
+                                void *xt_lo, int64_t ld_t, double *scal, int *status, int raw,
                                 cudaStream_t s)
 {
     (void)status;
     dim3 grid((unsigned)((n + 63) / 64), (unsigned)((m + 63) / 64));
     if (f64)
         ingest_split_kernel<true><<<grid, 256, 0, s>>>(A, m, n, lda, tau, xs_hi, nullptr, ld_s,
-                                                       xt_hi, nullptr, ld_t, scal);
+                                                       xt_hi, nullptr, ld_t, scal, raw);
     else
         ingest_split_kernel<false><<<grid, 256, 0, s>>>(A, m, n, lda, tau, xs_hi, xs_lo, ld_s,
-                                                        xt_hi, xt_lo, ld_t, scal);
+                                                        xt_hi, xt_lo, ld_t, scal, raw);
     return cudaGetLastError();
 }
 

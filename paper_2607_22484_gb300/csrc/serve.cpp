@@ -275,8 +275,11 @@ ServeState *state_of(svt_ctx *ctx)
     return ctx->serve;
 }
 
+// The grouped kernels cover the default pipeline: with a P chain and a polish step.
 bool grouped_kinds(const Plan &P)
 {
+    if (P.opt.mode != SVT_MODE_SVT)
+        return false;
     for (const Op &op : P.ops)
         if (op.kind != OP_MEMSET && op.kind != OP_REDUCE && op.kind != OP_SPLIT &&
             op.kind != OP_TC && op.kind != OP_FINAL)

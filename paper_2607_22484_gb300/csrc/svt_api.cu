@@ -763,10 +763,7 @@ struct Builder {
             }
             if (!emit(s2))
                 return false;
-            if (skipP) {
-                P.ops.push_back({OP_PREP, 1, 0});  // B = A (no P term)
-                P.kernel_launches += 1;
-            }
+            // Rank-r mode: the ingest has written B = A in X0's place.
         } else {
             P.ops.push_back({OP_PREP, skipP ? 1 : 0, 0});  // B = A - tau X, S' = S
             P.kernel_launches += 1;
@@ -920,8 +917,12 @@ svt_status run_ops(svt_ctx *ctx, Plan &P, const CallArgs &a, cudaStream_t s, siz
             break;
         case OP_SPLIT: {
             // same orientation as A: X (tall) when !wide, X^T when wide.
-            const Buf &same = P.wide ? L.Xt[0] : L.X[0];
-            const Buf &tran = P.wide ? L.X[0] : L.Xt[0];
+            // Without a P chain X0 has no reader: its copy is B = A (with a polish step; else
+            // OP_PREP writes B).
+            const bool b_is_a = skipP && (P.opt.polish || f64);
+            const Buf &x0 = b_is_a ? L.B : L.X[0];
+            const Buf &same = P.wide ? L.Xt[0] : x0;
+            const Buf &tran = P.wide ? x0 : L.Xt[0];
             void *same_lo = same.has_lo ? base + same.lo : nullptr;
             void *tran_lo = tran.has_lo ? base + tran.lo : nullptr;
             if (!f64 && !pairs) {  // BF16 tier: lo part of X0^T only, for the Gram
@@ -932,7 +933,7 @@ svt_status run_ops(svt_ctx *ctx, Plan &P, const CallArgs &a, cudaStream_t s, siz
             }
             err = ingest_split_launch(a.A, P.m, P.n, a.lda, a.tau, f64 ? 1 : 0, base + same.hi,
                                       same_lo, same.ld, base + tran.hi, tran_lo, tran.ld, scal,
-                                      status, s);
+                                      status, b_is_a ? (P.wide ? 2 : 1) : 0, s);
             break;
         }
         case OP_TC: {
@@ -1277,7 +1278,9 @@ void evict_plans(svt_ctx *ctx, size_t max_entries)
 int fused_auto_width(int64_t m, int64_t n, const Resolved &r)
 {
     const int64_t M = std::max(m, n), N = std::min(m, n);
-    if (N > 1792)
+    // Rank-r mode has half the tiles (one chain), so finer ones pay up to 2048 (2048 x 8192: 1221
+    // against 1555 us; 2304^2: 1714 against 1465).
+    if (N > (r.mode == SVT_MODE_RANK_R ? 2048 : 1792))
         return kBnPair;
     const int64_t segs = r.prec == SVT_FP32 ? 3 : 1;
     return (M + 2 * N) * segs >= 24 * 3 * kBK ? kBnPair128 : 128;

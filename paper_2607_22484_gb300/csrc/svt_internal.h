@@ -211,10 +211,11 @@ cudaError_t ingest_reduce_launch(const float *A, int64_t m, int64_t n, int64_t l
 // Ingest: alpha = 2^round(log2 ||A||_F), X0 = A_tall / alpha written as
 //   xs (same orientation as A): hi (and lo when xs_lo), leading dim ld_s;
 //   xt (transposed): hi (and lo when xt_lo), leading dim ld_t;
-// in BF16 (f64 = 0) or FP64 (f64 = 1, hi only). Also fills the scalar slots.
+// in BF16 (f64 = 0) or FP64 (f64 = 1, hi only). Also fills the scalar slots. raw: the copy
+// that holds A itself instead (1: xs, 2: xt, 0: none).
 cudaError_t ingest_split_launch(const float *A, int64_t m, int64_t n, int64_t lda, float tau,
                                 int f64, void *xs_hi, void *xs_lo, int64_t ld_s, void *xt_hi,
-                                void *xt_lo, int64_t ld_t, double *scal, int *status,
+                                void *xt_lo, int64_t ld_t, double *scal, int *status, int raw,
                                 cudaStream_t s);
 
 // Final status: non-finite output norm -> DIVERGED (unless already set), then
