@@ -854,7 +854,7 @@ def run_ours(args, n):
         with open(tpath) as f:
             tr = json.load(f)
         src_sha = hashlib.sha256(open(os.path.join(
-            ROOT, "paper_2607_22484_gb300", "csrc", "gemm_tc.cu"), "rb").read()).hexdigest()
+            ROOT, "paper_2607_22484_gb300", "csrc", "gemm_tc_kernel.cuh"), "rb").read()).hexdigest()
         if tr.get("gemm_tc_sha256") == src_sha and tr.get("n") == n:
             traffic = tr.get("dram_bytes_per_launch")
     lat = sorted(step_ms)

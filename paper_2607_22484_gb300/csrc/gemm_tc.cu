@@ -1,1704 +1,23 @@
-// Tensor-core product kernel for sm_103a: D = sum_s L_s R_s^T with BF16
-// operands staged by TMA into 128-byte-swizzled shared memory, tcgen05.mma
-// (kind::f16, BF16 x BF16 -> FP32) accumulating in tensor memory, and a fused
-// epilogue that reads the accumulator back with tcgen05.ld. Problems flagged fp8
-// (the FP8 experiment) take e4m3 operands through kind::f8f6f4 instead; the operand
-// kind, like the epilogue's chunk loop (one copy per product kind), is chosen once
-// per tile.
-//
-// This one kernel carries every dense product of the method (Section 2): the
-// shifted Gram A^T A - tau^2 I, the polynomial steps X (a I + b X^T X +
-// c (X^T X)^2) of both polar chains, the polish step and the final combine
-// 1/2 (A - tau P)(I + S) of Proposition 1.
-//
-// Structure (persistent, one CTA per SM, 384 threads):
-//   warp 0    : TMA producer (one thread), STAGES-deep shared-memory ring.
-//   warp 1    : tensor-memory allocator and MMA issuer (one thread).
-//   warps 2-9 : epilogue; warp w reads TMEM lanes 32 (w % 4) .. 32 (w % 4) + 31, and
-//               the two warps of a lane quadrant take alternate 32-column chunks.
-//   warp 10   : tile scheduler of fused launches (one thread): takes, decodes and waits for
-//               the next tile's dependencies while the producer loads the current one.
-//   warp 11   : publisher of fused launches (one thread): releases finished tiles.
-// Two accumulator buffers of BN FP32 columns each let the epilogue of one tile
-// overlap the MMAs of the next.
-//
-// CTA-pair mode (PAIR): a cluster of two CTAs computes one 256 x 256 (or 256 x 128)
-// tile with tcgen05.mma.cta_group::2. Each CTA stages its own 128 rows of L and one half
-// (128 or 64 rows) of the tile's R, so a pipeline stage is 32 KiB instead of 48 KiB (24
-// instead of 32) and every operand byte crosses L2 -> SM once per pair instead of once per CTA.
-// The even CTA (leader) issues the MMAs for both, its barriers collect both
-// CTAs' TMA bytes and both CTAs' epilogue releases; MMA completion is multicast
-// to both CTAs, whose epilogues each drain their own 128 x 256 accumulator.
-//
-// Every wait on an mbarrier is bounded (kWaitTimeoutNs of global time); on
-// expiry the kernel records SVT_ERR_TIMEOUT in the problem's status word, the
-// other roles stop at their next wait, in-flight copies and MMAs are drained
-// (again with a bound) and tensor memory is released before the kernel returns.
+// Launches of the product kernel (gemm_tc_kernel.cuh) by tile-width code.
 #include <algorithm>
-#include <cstddef>
 
-#include <cuda_bf16.h>
-#include <cuda_fp8.h>
-#include <cuda_runtime.h>
-#include <stdint.h>
-
-#include "solve_scalars.cuh"
-#include "tc_ptx.cuh"
+#include "svt_internal.h"
 
 namespace svt {
 
 namespace {
 
-// Warp roles: producer, MMA issuer, 8 epilogue warps, tile scheduler, publisher.
-constexpr int kEpiWarps = 8;
-constexpr int kSchedWarp = 2 + kEpiWarps;
-constexpr int kPubWarp = kSchedWarp + 1;
-constexpr int kThreads = 32 * (kPubWarp + 1);
-
-// Limit of the waits on other tiles' results (the launch's debug setting, else 2 s).
-__device__ __forceinline__ uint64_t dep_limit(const TcLaunch &L)
+cudaError_t launch_width(const TcLaunch &l, bool chain, int bn, int total_tiles, int num_sms,
+                         cudaStream_t s)
 {
-    return L.dep_wait_ns ? (uint64_t)L.dep_wait_ns : kWaitTimeoutNs;
-}
-
-// Wait for strip `idx` of dependency k of problem P (see TcProblem::sdep_*), unless the
-// producing problem is already known (src_done) or found to be complete as a whole,
-// which covers every strip; a role then stops checking that source.
-__device__ __forceinline__ bool wait_strip(const TcLaunch &L, const TcProblem &P, int k, int idx,
-                                           bool &src_done, volatile int *abort_flag, int *status)
-{
-    if (src_done)
-        return true;
-    if (ld_acquire_gpu(&L.done[P.sdep_src[k]]) >= P.sdep_whole[k]) {
-        src_done = true;
-        return true;
-    }
-    return wait_counter(&L.strips[P.sdep_base[k] + idx], P.sdep_target[k], abort_flag, status,
-                        dep_limit(L));
-}
-
-// ---------------------------------------------------------------- tiles
-
-struct TileCoord {
-    int prob, tm, tn;
-    bool valid;
-};
-
-__device__ __forceinline__ const TcProblem &prob_at(const TcLaunch &L, int p)
-{
-    return L.gtab ? L.gtab[p] : L.p[p];
-}
-
-// Linear tile index -> (problem, tile row, tile column) for tiles of TM x BN.
-// Dense problems: column-major over the tile grid. Symmetric problems: only
-// tiles holding some element with row <= col; column tn holds r (tn + 1) row
-// tiles (r = BN / TM), so the first tile of column tn is r tn (tn + 1) / 2
-// (tiles taller than wide, and ROWMAJOR_SYM with square tiles: see below).
-// A role's tile indices only increase, so the problem search gallops forward from
-// the previous answer (`hint`) instead of bisecting the whole table: a few
-// dependent loads of the tile prefix sums instead of log2(problems).
-template <int BN, int TM, bool ROWMAJOR_SYM>
-__device__ TileCoord decode_tile(const TcLaunch &L, int t, int &hint)
-{
-    TileCoord tc{0, 0, 0, false};
-    int p = 0, start = 0;
-    if (L.gtab) {
-        p = hint;
-        if (p < 0 || p >= L.gcount || L.gstart[p] > t)
-            p = 0;
-        int step = 1, q = p + 1;  // first q > p with gstart[q] > t lies in (p, q]
-        while (q < L.gcount && L.gstart[q] <= t) {
-            p = q;
-            step <<= 1;
-            q = p + step;
-        }
-        int hi = (q < L.gcount ? q : L.gcount) - 1;  // last p with gstart[p] <= t
-        while (p < hi) {
-            const int mid = (p + hi + 1) >> 1;
-            if (L.gstart[mid] <= t)
-                p = mid;
-            else
-                hi = mid - 1;
-        }
-        hint = p;
-        start = L.gstart[p];
-    } else {
-        while (p + 1 < L.nprob && t >= L.tile_start[p + 1])
-            ++p;
-        start = L.tile_start[p];
-    }
-    const TcProblem &P = prob_at(L, p);
-    int local = t - start;
-    tc.prob = p;
-    if (!P.sym) {
-        tc.tm = local % P.tiles_m;
-        tc.tn = local / P.tiles_m;
-        tc.valid = true;
-        return tc;
-    }
-    constexpr int r = BN / TM;
-    if (r == 0) {
-        // Tiles twice as tall as wide: columns 2 j and 2 j + 1 hold j + 1 row tiles each, the
-        // first of them from index j (j + 1) on.
-        int j = (int)((sqrtf(4.0f * (float)local + 1.0f) - 1.0f) * 0.5f);
-        while (j > 0 && j * (j + 1) > local)
-            --j;
-        while ((j + 1) * (j + 2) <= local)
-            ++j;
-        const int rem = local - j * (j + 1);
-        tc.tn = 2 * j + (rem > j ? 1 : 0);
-        tc.tm = rem > j ? rem - (j + 1) : rem;
-        tc.valid = (tc.tm < P.tiles_m) && (tc.tn < P.tiles_n);
-        return tc;
-    }
-    if (ROWMAJOR_SYM && r == 1) {
-        // Square tiles: row-major over the upper triangle (row tm holds columns
-        // tm .. T - 1, first index tm T - tm (tm - 1) / 2), so that the strips of a
-        // symmetric product complete in order.
-        const int T = P.tiles_n;
-        auto first = [T](int i) { return i * T - i * (i - 1) / 2; };
-        const float b = 2.0f * (float)T + 1.0f;
-        int tm = (int)((b - sqrtf(fmaxf(b * b - 8.0f * (float)local, 0.0f))) * 0.5f);
-        tm = tm < 0 ? 0 : (tm > T - 1 ? T - 1 : tm);
-        while (tm > 0 && first(tm) > local)
-            --tm;
-        while (tm + 1 < T && first(tm + 1) <= local)
-            ++tm;
-        tc.tm = tm;
-        tc.tn = tm + (local - first(tm));
-        tc.valid = (tm < P.tiles_m) && (tc.tn < P.tiles_n);
-        return tc;
-    }
-    int tn = (int)((sqrtf(8.0f * (float)local / (float)r + 1.0f) - 1.0f) * 0.5f);
-    while (tn > 0 && r * tn * (tn + 1) / 2 > local)
-        --tn;
-    while (r * (tn + 1) * (tn + 2) / 2 <= local)
-        ++tn;
-    int tm = local - r * tn * (tn + 1) / 2;
-    tc.tm = tm;
-    tc.tn = tn;
-    tc.valid = (tm < P.tiles_m) && (tn < P.tiles_n);
-    return tc;
-}
-
-// ------------------------------------------------------------- epilogue
-
-struct EpiScales {
-    float alpha, beta, gamma;
-};
-
-// The FP32 scales of a problem's epilogue. Problems scaled by a norm take theta =
-// norm^theta_pow (1/2 or 1/4) from the finished sum; their FP64 roots and products run in one
-// thread per tile (FP64 is 2 lanes a cycle and SM: the eight epilogue warps computing pow each
-// held the first Z products of a solve for 23,500 cycles).
-__device__ __forceinline__ EpiScales epi_scales(const TcProblem &P, const CallRec *calls)
-{
-    const Epi &e = P.ep;
-    EpiScales s{e.falpha, e.fbeta, e.fgamma};
-    if (P.patch & PT_ALPHA_NEG_TAU)
-        s.alpha = -calls[P.call_idx].tau;
-    if (e.theta_src) {
-        const double theta = root_theta(*e.theta_src, e.theta_pow == 0.25);
-        if (theta > 0.0 && isfinite(theta)) {
-            s.alpha = (float)(e.alpha / int_pow(theta, (int)e.ea));
-            s.beta = (float)(e.beta / int_pow(theta, (int)e.eb));
-            s.gamma = (float)(e.gamma / int_pow(theta, (int)e.eg));
-        } else if (!isfinite(theta) && e.status) {
-            atomicCAS(e.status, 0, (int)SVT_ERR_DIVERGED);
-        }  // theta == 0: the chain's matrix is zero; nothing to scale
-    }
-    return s;
-}
-
-__device__ __forceinline__ bool aligned16(const void *p)
-{
-    return (reinterpret_cast<uintptr_t>(p) & 15u) == 0;
-}
-
-// The fields of the current problem that the epilogue reads for every 32 x 32
-// block, loaded once per change of problem into registers: the problem table
-// lives in global memory, and every memory-clobbering TMA or fence instruction
-// of the epilogue would otherwise force these loads to be repeated.
-struct EpiHot {
-    const void *c0, *c1;
-    void *o0, *o1, *t0, *t1;
-    const CUtensorMap *maps;  // mapO[0..1], mapT[0..1], mapU[0..1] of the problem
-    double *norm_acc;
-    const double *diag, *dss;
-    int64_t ldc, ldo, ldt;
-    float alpha, beta, gamma;
-    int M, N, sym, otma, ttma, wide_tma, c_kind, c_trans, o_kind, o_trans, t_kind;
-    void *f0;          // e4m3 copy (FP8 experiment), null: none
-    int64_t ldf;
-    float fscale;
-};
-
-// Raw C values of one lane: for the generic loop its 32-column row segment, BF16 hi in q[0..3]
-// (lo of a pair in q[4..7]) or FP32 in q[0..7]; for the specialised ones its fragment of the
-// 32 x 32 block, BF16 pairs of block (g, k) in word 4 k + g (lo of a pair 16 further on).
-struct CRaw {
-    uint4 q[8];
-    __device__ __forceinline__ uint32_t &word(int i)
-    {
-        uint4 &x = q[i >> 2];
-        return (i & 3) == 0 ? x.x : ((i & 3) == 1 ? x.y : ((i & 3) == 2 ? x.z : x.w));
-    }
-};
-
-// Issue the loads of C(r, c0 .. c0 + 31) into registers. Returns false where the
-// vector form does not apply (no C, row outside, transposed C, a ragged right edge,
-// or a row address that is not 16-byte aligned); c_apply then reads C directly.
-__device__ __forceinline__ bool c_load(const EpiHot &h, int64_t r, int64_t c0, bool full_row,
-                                       CRaw &cr)
-{
-    if (h.c_kind == C_NONE || h.c_trans || !full_row)
-        return false;
-    const int64_t off = r * h.ldc + c0;
-    if (h.c_kind == C_F32) {
-        const float *p = static_cast<const float *>(h.c0) + off;
-        if (!aligned16(p))
-            return false;
-#pragma unroll
-        for (int q = 0; q < 8; ++q)
-            cr.q[q] = __ldg(reinterpret_cast<const uint4 *>(p) + q);
-        return true;
-    }
-    const __nv_bfloat16 *ph = static_cast<const __nv_bfloat16 *>(h.c0) + off;
-    const __nv_bfloat16 *pl = static_cast<const __nv_bfloat16 *>(h.c1) + off;
-    if (!aligned16(ph) || (h.c_kind == C_PAIR && !aligned16(pl)))
-        return false;
-#pragma unroll
-    for (int q = 0; q < 4; ++q)
-        cr.q[q] = __ldg(reinterpret_cast<const uint4 *>(ph) + q);
-    if (h.c_kind == C_PAIR) {
-#pragma unroll
-        for (int q = 0; q < 4; ++q)
-            cr.q[4 + q] = __ldg(reinterpret_cast<const uint4 *>(pl) + q);
-    }
-    return true;
-}
-
-// v[i] += beta * C(r, c0 + i) for i < ncol, from registers loaded by c_load (vec)
-// or read directly (any layout, alignment or edge).
-__device__ __forceinline__ void c_apply(const EpiHot &h, const CRaw &cr, bool vec, int64_t r,
-                                        int64_t c0, int ncol, bool row_ok, float *v)
-{
-    if (h.c_kind == C_NONE || !row_ok)
-        return;
-    const float beta = h.beta;
-    if (vec) {
-        if (h.c_kind == C_F32) {
-#pragma unroll
-            for (int q = 0; q < 8; ++q) {
-                v[4 * q] += beta * __uint_as_float(cr.q[q].x);
-                v[4 * q + 1] += beta * __uint_as_float(cr.q[q].y);
-                v[4 * q + 2] += beta * __uint_as_float(cr.q[q].z);
-                v[4 * q + 3] += beta * __uint_as_float(cr.q[q].w);
-            }
-            return;
-        }
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const __nv_bfloat162 *b = reinterpret_cast<const __nv_bfloat162 *>(&cr.q[q]);
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const float2 f = __bfloat1622float2(b[j]);
-                v[q * 8 + 2 * j] += beta * f.x;
-                v[q * 8 + 2 * j + 1] += beta * f.y;
-            }
-        }
-        if (h.c_kind == C_PAIR) {
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const __nv_bfloat162 *b = reinterpret_cast<const __nv_bfloat162 *>(&cr.q[4 + q]);
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    const float2 f = __bfloat1622float2(b[j]);
-                    v[q * 8 + 2 * j] += beta * f.x;
-                    v[q * 8 + 2 * j + 1] += beta * f.y;
-                }
-            }
-        }
-        return;
-    }
-#pragma unroll
-    for (int i = 0; i < 32; ++i) {
-        if (i >= ncol)
-            continue;
-        const int64_t c = c0 + i;
-        const int64_t off = h.c_trans ? c * h.ldc + r : r * h.ldc + c;
-        float x;
-        if (h.c_kind == C_F32)
-            x = static_cast<const float *>(h.c0)[off];
-        else {
-            x = __bfloat162float(static_cast<const __nv_bfloat16 *>(h.c0)[off]);
-            if (h.c_kind == C_PAIR)
-                x += __bfloat162float(static_cast<const __nv_bfloat16 *>(h.c1)[off]);
-        }
-        v[i] += beta * x;
-    }
-}
-
-// Fallback staging: 32 x 32 floats, element (a, b) at a * 32 + (b ^ a); rows and
-// columns are both free of bank conflicts.
-__device__ __forceinline__ int xs_idx(int a, int b) { return a * 32 + (b ^ a); }
-
-// e4m3 bytes of scale * v, saturated (the FP8 experiment's operand copies), in the
-// layout store_block uses: 16 rows x 32 bytes per instruction. Kept out of line so
-// that the BF16 epilogue's code is what it is without it.
-__device__ __noinline__ void store_block_e4m3(const float *st, void *p0, int64_t ld, int64_t r0,
-                                              int64_t c0, int64_t M, int64_t N, bool trans,
-                                              bool symdiag, int lane, float scale)
-{
-    const int64_t orow0 = trans ? c0 : r0, ocol0 = trans ? r0 : c0;
-    const int64_t orows = trans ? N : M, ocols = trans ? M : N;
-    // e4m3 bytes of scale * v, saturated: 16 rows x 32 bytes per instruction
-#pragma unroll
-    for (int k = 0; k < 2; ++k) {
-        const int a = k * 16 + (lane >> 1);
-        const int q = lane & 1;  // columns 16 q .. 16 q + 15
-        const int64_t R = orow0 + a;
-        float x[16];
-#pragma unroll
-        for (int j = 0; j < 16; ++j) {
-            const int b = q * 16 + j;
-            int sa, sb;
-            if (trans) { sa = b; sb = a; }
-            else if (symdiag && a > b) { sa = b; sb = a; }
-            else { sa = a; sb = b; }
-            x[j] = scale * st[xs_idx(sa, sb)];
-        }
-        if (R >= orows)
-            continue;
-        const int64_t C = ocol0 + q * 16;
-        uint8_t *p = static_cast<uint8_t *>(p0) + R * ld + C;
-        if (C + 16 <= ocols && aligned16(p)) {
-            uint32_t w[4];
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const uint32_t lo = __nv_cvt_float2_to_fp8x2(make_float2(x[4 * j], x[4 * j + 1]),
-                                                             __NV_SATFINITE, __NV_E4M3);
-                const uint32_t hi = __nv_cvt_float2_to_fp8x2(make_float2(x[4 * j + 2], x[4 * j + 3]),
-                                                             __NV_SATFINITE, __NV_E4M3);
-                w[j] = lo | (hi << 16);
-            }
-            *reinterpret_cast<uint4 *>(p) = make_uint4(w[0], w[1], w[2], w[3]);
-        } else {
-#pragma unroll
-            for (int j = 0; j < 16; ++j)
-                if (C + j < ocols)
-                    p[j] = __nv_cvt_float_to_fp8(x[j], __NV_SATFINITE, __NV_E4M3);
-        }
-    }
-}
-
-// Store a 32 x 32 block held in shared memory `st` (st[a][b] = value of tile
-// element (r0 + a, c0 + b)) to global memory, coalesced: warp lanes cover whole
-// row segments (8 rows x 64 B for BF16, 4 rows x 128 B for FP32 per instruction).
-//   trans = 0: element (r0 + a, c0 + b) -> p[(r0 + a) * ld + c0 + b];
-//              symdiag: the block sits on the diagonal and (a > b) takes st[b][a].
-//   trans = 1: element (r0 + b, c0 + a) -> p[(c0 + a) * ld + r0 + b].
-// Only elements with row < M and col < N (tile coordinates) are written.
-__device__ __forceinline__ void store_block(const float *st, int kind, void *p0, void *p1,
-                                            int64_t ld, int64_t r0, int64_t c0, int64_t M,
-                                            int64_t N, bool trans, bool symdiag, int lane)
-{
-    // output rows: tile rows (trans = 0) or tile columns (trans = 1)
-    const int64_t orow0 = trans ? c0 : r0, ocol0 = trans ? r0 : c0;
-    const int64_t orows = trans ? N : M, ocols = trans ? M : N;
-    if (kind == O_BF16 || kind == O_PAIR) {
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            const int a = k * 8 + (lane >> 2);  // output row within the block
-            const int q = lane & 3;             // 16-byte chunk: columns 8q .. 8q + 7
-            const int64_t R = orow0 + a;
-            float x[8];
-#pragma unroll
-            for (int j = 0; j < 8; ++j) {
-                const int b = q * 8 + j;
-                int sa, sb;  // staging coordinates
-                if (trans) { sa = b; sb = a; }
-                else if (symdiag && a > b) { sa = b; sb = a; }
-                else { sa = a; sb = b; }
-                x[j] = st[xs_idx(sa, sb)];
-            }
-            if (R >= orows)
-                continue;
-            const int64_t C = ocol0 + q * 8;
-            const int64_t off = R * ld + C;
-            if (C + 8 <= ocols && aligned16(static_cast<__nv_bfloat16 *>(p0) + off) &&
-                (kind != O_PAIR || aligned16(static_cast<__nv_bfloat16 *>(p1) + off))) {
-                uint32_t hw[4], lw[4];
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    __nv_bfloat162 h2 = __floats2bfloat162_rn(x[2 * j], x[2 * j + 1]);
-                    hw[j] = *reinterpret_cast<uint32_t *>(&h2);
-                    __nv_bfloat162 l2 = __floats2bfloat162_rn(x[2 * j] - __low2float(h2),
-                                                              x[2 * j + 1] - __high2float(h2));
-                    lw[j] = *reinterpret_cast<uint32_t *>(&l2);
-                }
-                *reinterpret_cast<uint4 *>(static_cast<__nv_bfloat16 *>(p0) + off) =
-                    make_uint4(hw[0], hw[1], hw[2], hw[3]);
-                if (kind == O_PAIR)
-                    *reinterpret_cast<uint4 *>(static_cast<__nv_bfloat16 *>(p1) + off) =
-                        make_uint4(lw[0], lw[1], lw[2], lw[3]);
-            } else {
-#pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                    if (C + j < ocols) {
-                        __nv_bfloat16 h = __float2bfloat16_rn(x[j]);
-                        static_cast<__nv_bfloat16 *>(p0)[off + j] = h;
-                        if (kind == O_PAIR)
-                            static_cast<__nv_bfloat16 *>(p1)[off + j] =
-                                __float2bfloat16_rn(x[j] - __bfloat162float(h));
-                    }
-                }
-            }
-        }
-    } else if (kind == O_F32) {
-#pragma unroll
-        for (int k = 0; k < 8; ++k) {
-            const int a = k * 4 + (lane >> 3);
-            const int q = lane & 7;  // columns 4q .. 4q + 3
-            const int64_t R = orow0 + a;
-            float x[4];
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const int b = q * 4 + j;
-                int sa, sb;
-                if (trans) { sa = b; sb = a; }
-                else if (symdiag && a > b) { sa = b; sb = a; }
-                else { sa = a; sb = b; }
-                x[j] = st[xs_idx(sa, sb)];
-            }
-            if (R >= orows)
-                continue;
-            const int64_t C = ocol0 + q * 4;
-            const int64_t off = R * ld + C;
-            if (C + 4 <= ocols && aligned16(static_cast<float *>(p0) + off)) {
-                *reinterpret_cast<float4 *>(static_cast<float *>(p0) + off) =
-                    make_float4(x[0], x[1], x[2], x[3]);
-            } else {
-#pragma unroll
-                for (int j = 0; j < 4; ++j)
-                    if (C + j < ocols)
-                        static_cast<float *>(p0)[off + j] = x[j];
-            }
-        }
-    }
-}
-
-// Byte offset of element (row, col) of a 32 x 32 staging block laid out the way
-// the TMA unit reads it: FP32 rows of 128 B with the 128-byte swizzle (16-byte
-// chunk index XOR row % 8), BF16 rows of 64 B with the 64-byte swizzle (chunk
-// index XOR (row / 2) % 4). Both orders of writing -- a lane per row with 16-byte
-// vectors, or a lane per column with scalars -- are free of bank conflicts.
-__device__ __forceinline__ uint32_t stg_off_f32(int row, int col)
-{
-    return (uint32_t)(row * 128 + ((((col >> 2) ^ (row & 7))) << 4) + (col & 3) * 4);
-}
-__device__ __forceinline__ uint32_t stg_off_b16(int row, int col)
-{
-    return (uint32_t)(row * 64 + ((((col >> 3) ^ ((row >> 1) & 3))) << 4) + (col & 7) * 2);
-}
-
-// Stage the warp's 32 x 32 block (lane = block row, x[] = its 32 columns) and
-// store it with one or two TMA stores (one bulk group): at tile coordinates
-// (x = c0, y = r0), or transposed at (x = r0, y = c0). `kind` is O_F32, O_BF16 or
-// O_PAIR (hi through m0, lo through m1). The warp owns NSTG 4 KiB staging slots
-// (1024-byte aligned) used in turn, so a store's shared-memory read overlaps the
-// staging of the next NSTG - 1 blocks; an FP32 block fills a slot, BF16 hi and lo
-// take its two halves.
-template <int NSTG>
-__device__ __forceinline__ void tma_store_block(const float *x, int kind, bool trans,
-                                                const CUtensorMap *m0, const CUtensorMap *m1,
-                                                int r0, int c0, uint8_t *stg_base, int &slot,
-                                                int lane)
-{
-    uint8_t *stg0 = stg_base + slot * 4096, *stg1 = stg0 + 2048;
-    if (++slot == NSTG)
-        slot = 0;
-    if (elect_one())
-        bulk_wait_read<NSTG - 1>();  // the store that last used this slot has read it
-    __syncwarp();
-    if (kind == O_F32) {
-        if (!trans) {
-#pragma unroll
-            for (int q = 0; q < 8; ++q)
-                *reinterpret_cast<float4 *>(stg0 + stg_off_f32(lane, 4 * q)) =
-                    make_float4(x[4 * q], x[4 * q + 1], x[4 * q + 2], x[4 * q + 3]);
-        } else {
-#pragma unroll
-            for (int c = 0; c < 32; ++c)
-                *reinterpret_cast<float *>(stg0 + stg_off_f32(c, lane)) = x[c];
-        }
-    } else {
-        const bool pair = (kind == O_PAIR);
-        if (!trans) {
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                uint32_t hw[4], lw[4];
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    __nv_bfloat162 h2 = __floats2bfloat162_rn(x[8 * q + 2 * j], x[8 * q + 2 * j + 1]);
-                    hw[j] = *reinterpret_cast<uint32_t *>(&h2);
-                    __nv_bfloat162 l2 = __floats2bfloat162_rn(x[8 * q + 2 * j] - __low2float(h2),
-                                                              x[8 * q + 2 * j + 1] - __high2float(h2));
-                    lw[j] = *reinterpret_cast<uint32_t *>(&l2);
-                }
-                *reinterpret_cast<uint4 *>(stg0 + stg_off_b16(lane, 8 * q)) =
-                    make_uint4(hw[0], hw[1], hw[2], hw[3]);
-                if (pair)
-                    *reinterpret_cast<uint4 *>(stg1 + stg_off_b16(lane, 8 * q)) =
-                        make_uint4(lw[0], lw[1], lw[2], lw[3]);
-            }
-        } else {
-#pragma unroll
-            for (int c = 0; c < 32; ++c) {
-                __nv_bfloat16 h = __float2bfloat16_rn(x[c]);
-                *reinterpret_cast<__nv_bfloat16 *>(stg0 + stg_off_b16(c, lane)) = h;
-                if (pair)
-                    *reinterpret_cast<__nv_bfloat16 *>(stg1 + stg_off_b16(c, lane)) =
-                        __float2bfloat16_rn(x[c] - __bfloat162float(h));
-            }
-        }
-    }
-    fence_async_smem();
-    __syncwarp();
-    if (elect_one()) {
-        const int sx = trans ? r0 : c0, sy = trans ? c0 : r0;
-        tma_store_2d(m0, sx, sy, stg0);
-        if (kind == O_PAIR)
-            tma_store_2d(m1, sx, sy, stg1);
-        bulk_commit();
-    }
-}
-
-// Rest of the epilogue of one 32 x 32 block after alpha D + beta C: the identity
-// term (or the FP64 shifted-Gram diagonal) on the diagonal, the squared-norm
-// contribution, then the stores. lane = tile row r0 + lane, columns c0 .. c0 + 31.
-// Values are staged in shared memory and stored coalesced to every requested
-// destination: the output (row-major or transposed), the extra transposed copy
-// and, for symmetric products, the mirror.
-template <int NSTG>
-__device__ __forceinline__ void epilogue_finish(const EpiHot &h, int64_t r0, int64_t c0, float *v,
-                                                double &nrm, uint8_t *stg, int &slot, int lane)
-{
-    const int64_t r = r0 + lane;
-    const bool row_ok = r < h.M;
-    const int64_t rem = (int64_t)h.N - c0;
-    const int ncol = rem < 32 ? (int)rem : 32;
-    const bool diag_block = (r0 == c0);
-    if (diag_block) {  // this lane's diagonal element is column i == lane
-        const bool dg = h.diag != nullptr;
-        const float dval = (dg && row_ok) ? (float)(h.diag[r] * h.dss[0] - h.dss[1]) : 0.f;
-        const float g = h.gamma;
-#pragma unroll
-        for (int i = 0; i < 32; ++i)
-            if (i == lane)
-                v[i] = dg ? dval : v[i] + g;
-    }
-    if (h.norm_acc && row_ok) {
-        // FP32 within the row's 32 values (relative error <= 32 * 2^-24), FP64 across.
-        float acc = 0.f;
-#pragma unroll
-        for (int i = 0; i < 32; ++i) {
-            float w = (i < ncol) ? 1.f : 0.f;
-            if (h.sym) {
-                const int64_t c = c0 + i;
-                w = (r < c) ? 2.f * w : (r == c ? w : 0.f);
-            }
-            acc = fmaf(w * v[i], v[i], acc);
-        }
-        nrm += (double)acc;
-    }
-    const bool symdiag = h.sym && diag_block;
-    // Outputs through TMA stores (all but diagonal blocks of symmetric products).
-    const bool o_tma = h.otma && h.o_kind != O_NONE && !symdiag;
-    if (o_tma)
-        tma_store_block<NSTG>(v, h.o_kind, h.o_trans != 0, &h.maps[0], &h.maps[1], (int)r0,
-                              (int)c0, stg, slot, lane);
-    if (h.sym && !diag_block && h.otma)  // mirror of a block strictly above the diagonal
-        tma_store_block<NSTG>(v, h.o_kind, true, &h.maps[0], &h.maps[1], (int)r0, (int)c0, stg,
-                              slot, lane);
-    if (h.ttma && h.t_kind != O_NONE)
-        tma_store_block<NSTG>(v, h.t_kind, true, &h.maps[2], &h.maps[3], (int)r0, (int)c0, stg,
-                              slot, lane);
-    const bool need_plain = (h.o_kind != O_NONE && !o_tma) || (h.sym && !diag_block && !h.otma) ||
-                            (h.t_kind != O_NONE && !h.ttma) || h.f0 != nullptr;
-    if (!need_plain)
-        return;
-    // Coalesced plain-store path: stage with a swizzled pitch, then whole row segments.
-    if (elect_one())
-        bulk_wait_read0();
-    __syncwarp();
-    float *st = reinterpret_cast<float *>(stg);
-#pragma unroll
-    for (int i = 0; i < 32; ++i)
-        st[xs_idx(lane, i)] = v[i];
-    __syncwarp();
-    if (h.o_kind != O_NONE && !o_tma)
-        store_block(st, h.o_kind, h.o0, h.o1, h.ldo, r0, c0, h.M, h.N, h.o_trans != 0, symdiag, lane);
-    if (h.sym && !diag_block && !h.otma)
-        store_block(st, h.o_kind, h.o0, h.o1, h.ldo, r0, c0, h.M, h.N, true, false, lane);
-    if (h.t_kind != O_NONE && !h.ttma)
-        store_block(st, h.t_kind, h.t0, h.t1, h.ldt, r0, c0, h.M, h.N, true, false, lane);
-    if (h.f0) {  // the e4m3 copy, mirrored like the output for symmetric products
-        store_block_e4m3(st, h.f0, h.ldf, r0, c0, h.M, h.N, false, symdiag, lane, h.fscale);
-        if (h.sym && !diag_block)
-            store_block_e4m3(st, h.f0, h.ldf, r0, c0, h.M, h.N, true, false, lane, h.fscale);
-    }
-    __syncwarp();
-}
-
-// Product kinds whose epilogue runs a specialised chunk loop (chosen once per tile):
-// BF16 or hi/lo-pair output through TMA stores, no norm, no FP64 diagonal, no e4m3
-// copy, untransposed output, and one of
-//   symmetric, no C                 (Y = X^T X, Y = S^2, S Z)
-//   symmetric, C of the output kind (Z = a I + b Y + c Y^2)
-//   general, no C, transposed copy of the output kind (X Z and its X^T)
-// Everything else runs the generic loop (code -1). Code = 3 * (output is a pair) +
-// (0 symmetric, 1 symmetric with C, 2 general with copy).
-template <int S>
-struct EpiSpec {
-    static constexpr int code = S;
-    static constexpr bool generic = S < 0;
-    static constexpr bool pair = S >= 3;
-    static constexpr bool sym = S >= 0 && S % 3 != 2;
-    static constexpr bool has_c = S >= 0 && S % 3 == 1;
-};
-
-__device__ __forceinline__ int epi_spec(const EpiHot &h)
-{
-    if ((h.o_kind != O_BF16 && h.o_kind != O_PAIR) || !h.otma || h.o_trans || h.norm_acc || h.f0 ||
-        h.diag || !h.wide_tma)
-        return -1;
-    const bool pair = h.o_kind == O_PAIR;
-    const int base = pair ? 3 : 0;
-    if (h.sym && h.t_kind == O_NONE) {
-        if (h.c_kind == C_NONE)
-            return base;
-        if (h.c_kind == (pair ? C_PAIR : C_BF16) && !h.c_trans)
-            return base + 1;
-        return -1;
-    }
-    if (!h.sym && h.t_kind == h.o_kind && h.ttma && h.c_kind == C_NONE && h.gamma == 0.f)
-        return base + 2;
-    return -1;
-}
-
-// Issue the loads of this lane's fragment of C's 32 x 32 block at (r0, c0). Columns past the
-// matrix lie in the row padding of the workspace buffers (rows padded to 64 elements).
-template <bool PAIRED>
-__device__ __forceinline__ void c_load_frag(const EpiHot &h, int64_t r0, int64_t c0, int lane, CRaw &cr)
-{
-#pragma unroll
-    for (int g = 0; g < 4; ++g) {
-        const int64_t r = r0 + 8 * g + (lane >> 2);
-        const bool ok = r < h.M;
-        const int64_t off = r * h.ldc + c0 + 2 * (lane & 3);
-        const __nv_bfloat16 *ph = static_cast<const __nv_bfloat16 *>(h.c0) + off;
-        const __nv_bfloat16 *pl = static_cast<const __nv_bfloat16 *>(h.c1) + off;
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            cr.word(4 * k + g) = ok ? *reinterpret_cast<const uint32_t *>(ph + 8 * k) : 0u;
-            if (PAIRED)
-                cr.word(16 + 4 * k + g) = ok ? *reinterpret_cast<const uint32_t *>(pl + 8 * k) : 0u;
-        }
-    }
-}
-
-// How a specialised epilogue stages a 32 x 32 block for its TMA stores: as half of a 64-column
-// unit (BF16 only: one 64 x 32 box in place, one 32 x 64 box mirrored), by itself, or by itself
-// on the diagonal of a symmetric product (one box holding both triangles).
-// A warp's TMA stores and the waits for them run in one elected lane (the same for a given mask:
-// bulk groups belong to the thread that commits them).
-constexpr int kStgSlots = 2;                  // 4 KiB staging slots of an epilogue warp
-constexpr int kStgBytes = kStgSlots * 4096;
-
-enum StageMode { STAGE_UNIT, STAGE_BLOCK, STAGE_DIAG };
-
-// Offsets in the warp's 8 KiB of staging. STAGE_UNIT: the 64-column rows (128-byte swizzle) at 0,
-// the mirrored rows at kStgMirror64. Else: in place at 0, mirrored at kStgMirror, the lo parts
-// kStgLo further on (64-byte swizzle).
-constexpr uint32_t kStgMirror = 2048, kStgLo = 4096, kStgMirror64 = 4096;
-
-// Stage one part (hi or lo) of a block: w[k][g] holds this lane's pair of 8 x 8 block (g, k).
-// Four blocks g of one k per stmatrix; the transposing form writes their mirror. half: which 32
-// columns of the unit.
-template <int MODE>
-__device__ __forceinline__ void stage_part(uint32_t (&w)[4][4], uint32_t stg, int half, int lane)
-{
-    const int g = lane >> 3, j = lane & 7;
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        uint32_t da, ma;
-        if (MODE == STAGE_UNIT) {
-            const int row = 32 * half + 8 * k + j;
-            da = stg + lane * 128 + (((4 * half + k) ^ j) << 4);
-            ma = stg + kStgMirror64 + row * 64 + ((g ^ ((row >> 1) & 3)) << 4);
-        } else {
-            const int row = 8 * k + j;
-            da = stg + lane * 64 + ((k ^ ((lane >> 1) & 3)) << 4);
-            ma = stg + (MODE == STAGE_DIAG ? 0u : kStgMirror) + row * 64 + ((g ^ ((row >> 1) & 3)) << 4);
-        }
-        if (MODE == STAGE_DIAG) {
-            // The block's own lower triangle is not part of the result: its 8 x 8 blocks are
-            // the mirrors of those above the diagonal, and the ones on it mirror themselves.
-            w[k][k] = mirror_diag(w[k][k], lane);
-            const uint32_t dummy = stg + kStgMirror + 16 * j;
-            if (g > k)
-                da = dummy;
-            if (g >= k)
-                ma = dummy;
-        }
-        stmatrix4<false>(da, w[k]);
-        stmatrix4<true>(ma, w[k]);
-    }
-}
-
-// Value arithmetic and staging of one 32 x 32 block of a specialised product: v = alpha D +
-// beta C + gamma I from the accumulator at taddr, rounded to BF16 (and lo parts) in the staging.
-//
-// The accumulator is read as matrix fragments, so the staging takes 8 stmatrix a part where the
-// row-per-thread form took 4 16-byte and 32 two-byte stores and converted every value twice.
-template <int S, int MODE>
-__device__ __forceinline__ void spec_block(const EpiHot &h, CRaw &cr, uint32_t taddr, int64_t r0,
-                                           int64_t c0, uint32_t stg, int half, int lane)
-{
-    using Spec = EpiSpec<S>;
-    float v[2][16];
-    tmem_ld_frag32(taddr, v[0]);
-    tmem_ld_frag32(taddr + (16u << 16), v[1]);
-    tmem_ld_wait();
-    const bool edge = h.N - c0 < 32;
-    uint32_t w[4][4];
-    float x[4][4][2];
-#pragma unroll
-    for (int k = 0; k < 4; ++k)
-#pragma unroll
-        for (int g = 0; g < 4; ++g) {
-            float a = __fmul_rn(v[g >> 1][4 * k + 2 * (g & 1)], h.alpha);
-            float b = __fmul_rn(v[g >> 1][4 * k + 2 * (g & 1) + 1], h.alpha);
-            if (Spec::has_c) {
-                float2 c = bf16x2(cr.word(4 * k + g));
-                if (Spec::pair) {
-                    const float2 l = bf16x2(cr.word(16 + 4 * k + g));
-                    if (edge) {  // a row that ends in this chunk adds the parts' sum
-                        c.x += l.x;
-                        c.y += l.y;
-                    }
-                    a = fmaf(h.beta, c.x, a);
-                    b = fmaf(h.beta, c.y, b);
-                    if (!edge) {
-                        a = fmaf(h.beta, l.x, a);
-                        b = fmaf(h.beta, l.y, b);
-                    }
-                } else {
-                    a = fmaf(h.beta, c.x, a);
-                    b = fmaf(h.beta, c.y, b);
-                }
-            }
-            if (MODE == STAGE_DIAG && g == k) {
-                const int row = lane >> 2, col = 2 * (lane & 3);
-                if (row == col)
-                    a += h.gamma;
-                if (row == col + 1)
-                    b += h.gamma;
-            }
-            const __nv_bfloat162 h2 = __floats2bfloat162_rn(a, b);
-            w[k][g] = *reinterpret_cast<const uint32_t *>(&h2);
-            if (Spec::pair) {
-                x[k][g][0] = a - __low2float(h2);
-                x[k][g][1] = b - __high2float(h2);
-            }
-        }
-    stage_part<MODE>(w, stg, half, lane);
-    if (Spec::pair) {
-#pragma unroll
-        for (int k = 0; k < 4; ++k)
-#pragma unroll
-            for (int g = 0; g < 4; ++g) {
-                const __nv_bfloat162 l2 = __floats2bfloat162_rn(x[k][g][0], x[k][g][1]);
-                w[k][g] = *reinterpret_cast<const uint32_t *>(&l2);
-            }
-        stage_part<MODE>(w, stg + kStgLo, half, lane);
-    }
-}
-
-// Load the epilogue fields of problem P (with the per-call fields of a grouped or
-// fused launch) into registers.
-__device__ __forceinline__ void load_hot(EpiHot &h, const TcProblem &P, const CallRec *calls,
-                                         const EpiScales &sc)
-{
-    const Epi &e = P.ep;
-    h.c0 = e.c0;
-    h.c1 = e.c1;
-    h.ldc = e.ldc;
-    h.o0 = e.o0;
-    h.o1 = e.o1;
-    h.ldo = e.ldo;
-    h.t0 = e.t0;
-    h.t1 = e.t1;
-    h.ldt = e.ldt;
-    h.maps = &P.mapO[0];
-    h.norm_acc = e.norm_acc;
-    h.diag = e.diag;
-    h.dss = e.dss;
-    h.M = P.M;
-    h.N = P.N;
-    h.sym = P.sym;
-    h.otma = P.o_tma;
-    h.ttma = P.t_tma;
-    h.wide_tma = P.u_tma;
-    h.c_kind = e.c_kind;
-    h.c_trans = e.c_trans;
-    h.o_kind = e.o_kind;
-    h.o_trans = e.o_trans;
-    h.t_kind = e.t_kind;
-    h.f0 = e.f0;
-    h.ldf = e.ldf;
-    h.fscale = e.fscale;
-    if (P.patch) {  // grouped / fused launch: per-call fields
-        const CallRec &cr = calls[P.call_idx];
-        if (P.patch & PT_C_IS_A) {
-            h.c0 = cr.A;
-            h.ldc = cr.lda;
-        }
-        if (P.patch & PT_O_IS_Y) {
-            h.o0 = cr.Y;
-            h.ldo = cr.ldy;
-            h.otma = 0;
-        }
-    }
-    h.alpha = sc.alpha;
-    h.beta = sc.beta;
-    h.gamma = sc.gamma;
-}
-
-// --------------------------------------------------------------- kernel
-
-constexpr int kRingTiles = 4;  // fused launches: tiles in flight between the roles
-
-// A tile handed from the scheduler to the other roles (and to the peer CTA of a pair), with its
-// epilogue's scales and what the producer and the MMA issuer would otherwise load from the
-// problem table between two tiles.
-struct RingTile {
-    int tile;  // index in the launch (-1: no more tiles)
-    int prob;  // -1: nothing to compute
-    int tm, tn;
-    float alpha, beta, gamma;
-    int geom;  // see pack_geom
-};
-
-// k-blocks of a segment in bits 0..15 (K < 2^21), segments in 16..17, their L and R parts in
-// 18..20 and 21..23, e4m3 operands in 24, "the operands' dependencies are met" in 25.
-constexpr int kGeomReady = 1 << 25;
-__device__ __forceinline__ int pack_geom(const TcProblem &P)
-{
-    // A k-block is one 128-byte swizzle row: 64 BF16 or 128 e4m3 elements.
-    const int kshift = P.fp8 ? 7 : 6;
-    int g = (P.K + (1 << kshift) - 1) >> kshift;
-    g |= P.nseg << 16 | (P.fp8 ? 1 << 24 : 0);
-#pragma unroll
-    for (int k = 0; k < 3; ++k)
-        g |= P.segL[k] << (18 + k) | P.segR[k] << (21 + k);
-    return g;
-}
-__device__ __forceinline__ int geom_kblocks(int g) { return g & 0xffff; }
-__device__ __forceinline__ int geom_segs(int g) { return (g >> 16) & 3; }
-__device__ __forceinline__ int geom_l(int g, int sg) { return (g >> (18 + sg)) & 1; }
-__device__ __forceinline__ int geom_r(int g, int sg) { return (g >> (21 + sg)) & 1; }
-__device__ __forceinline__ bool geom_fp8(int g) { return (g >> 24) & 1; }
-
-template <int BN, int STAGES, bool CHAIN, bool PAIR, bool STRIPS>
-__global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_constant__ TcLaunch L)
-{
-    static_assert(!STRIPS || CHAIN, "strip dependencies exist in fused launches only");
-    static_assert(!PAIR || BN == 256 || BN == 128, "CTA pairs compute 256 x 256 or 256 x 128 tiles");
-    extern __shared__ uint8_t smem_raw[];
-    uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
-                                                ~static_cast<uintptr_t>(1023));
-    constexpr int A_BYTES = kBM * kBK * 2;
-    constexpr int B_ROWS = PAIR ? BN / 2 : BN;  // rows of R this CTA stages per k-block
-    constexpr int B_BYTES = B_ROWS * kBK * 2;
-    constexpr int TILE_ROWS = PAIR ? 2 * kBM : kBM;
-    uint8_t *sA = smem;
-    uint8_t *sB = smem + STAGES * A_BYTES;
-    uint8_t *stage_all = sB + STAGES * B_BYTES;  // 1024-aligned
-    uint64_t *full = reinterpret_cast<uint64_t *>(stage_all + kEpiWarps * kStgBytes);
-    uint64_t *empty = full + STAGES;
-    uint64_t *tfull = empty + STAGES;
-    uint64_t *tempty = tfull + 2;
-    uint64_t *drain = tempty + 2;
-    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(drain + 1);
-    volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_slot + 1);
-    int *skip_flag = reinterpret_cast<int *>(tmem_slot + 2);
-    // Fused launches: the ring of tiles from the scheduler to the other roles; pdone[i]: the
-    // epilogue warps' parts of the tile in entry i are in global memory; ptaken: the producer's
-    // latest tile can start.
-    uint64_t *rfull = reinterpret_cast<uint64_t *>(
-        (reinterpret_cast<uintptr_t>(tmem_slot + 3) + 7) & ~static_cast<uintptr_t>(7));
-    uint64_t *rempty = rfull + kRingTiles;
-    uint64_t *pdone = rempty + kRingTiles;
-    uint64_t *ptaken = pdone + kRingTiles;
-    volatile RingTile *ring = reinterpret_cast<volatile RingTile *>(
-        (reinterpret_cast<uintptr_t>(ptaken + 1) + 15) & ~static_cast<uintptr_t>(15));
-    const CallRec *calls = L.calls ? L.calls : &L.call_inline;
-
-    const int warp = threadIdx.x >> 5;
-    const int lane = threadIdx.x & 31;
-    int *status0 = prob_at(L, 0).ep.status;
-    // CTA pairs: rank 0 (leader) issues the MMAs and hands out tile ids.
-    const uint32_t rank = PAIR ? cluster_rank() : 0u;
-    const bool leader = rank == 0;
-
-    if (threadIdx.x == 0) {
-        for (int s = 0; s < STAGES; ++s) {
-            mbar_init(&full[s], 1);
-            mbar_init(&empty[s], 1);
-        }
-        for (int b = 0; b < 2; ++b) {
-            mbar_init(&tfull[b], 1);
-            // Pairs: one release per epilogue warp of both CTAs, on the leader's barrier.
-            mbar_init(&tempty[b], PAIR ? 2 * kEpiWarps : 32 * kEpiWarps);
-        }
-        mbar_init(drain, 1);
-        for (int i = 0; i < kRingTiles; ++i) {
-            mbar_init(&rfull[i], 1);
-            // Consumers of a ring entry: producer, MMA issuer, epilogue warps and publisher;
-            // for pairs also the peer's (which issues no MMAs).
-            mbar_init(&rempty[i], PAIR ? 2 * (2 + kEpiWarps) + 1 : 3 + kEpiWarps);
-            mbar_init(&pdone[i], kEpiWarps);
-        }
-        mbar_init(ptaken, 1);
-        *abort_flag = 0;
-        // A solve whose earlier launch already timed out does no further work.
-        *skip_flag = (status0 && *reinterpret_cast<volatile int *>(status0) == (int)SVT_ERR_TIMEOUT);
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    }
-    if (PAIR) {
-        // The peer's barriers exist before either CTA signals them.
-        __syncthreads();
-        cluster_sync_all();
-    }
-    if (warp == 1) {
-        tmem_alloc<PAIR>(tmem_slot, 2 * BN);
-        tmem_relinquish<PAIR>();
-    }
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-    const uint32_t tmem_base = *tmem_slot;
-    const int total = *skip_flag ? 0
-                                 : (L.gtab ? (L.tile_hi > 0 ? L.tile_hi : L.gstart[L.gcount])
-                                           : L.tile_start[L.nprob]);
-    // Static schedule (non-fused launches): CTA (pair) i takes tiles i, i + grid, ...
-    const int t_first = PAIR ? (int)(blockIdx.x >> 1) : (int)blockIdx.x;
-    const int t_step = PAIR ? (int)(gridDim.x >> 1) : (int)gridDim.x;
-
-    // Take over ring entry ri: wait for it, read it, and release it at once (`keep`: the
-    // caller releases it later).
-    auto ring_release = [&](int ri) {
-        if (PAIR && !leader)
-            mbar_arrive_remote(peer_addr(&rempty[ri], 0));
-        else
-            mbar_arrive(&rempty[ri]);
-    };
-    if (warp == kSchedWarp && lane == 0) {
-        // ------------------------------------------------ tile scheduler (fused launches)
-        // Takes tiles in table order, one ahead of the one the producer is loading, so that the
-        // counter's round trip, the decoding, the tensor maps' and problem fields' fetches and
-        // the dependency wait of a tile run beside the copies of the tile before it (in the
-        // producer they cost 2200 cycles between tiles). With the publisher: 256-matrix batch
-        // 10.03 -> 8.68 ms, single solves 1 to 2 % faster.
-        if (CHAIN && (!PAIR || leader)) {
-            int ri = 0, hint = 0;
-            uint32_t rphase = 0, taken = 0;
-            int dep_prob = -1;  // problem whose whole dependencies have been waited for
-            bool src_done[2] = {false, false};
-            for (bool first = true;; first = false) {
-                if (!first) {
-                    if (!mbar_wait(ptaken, taken, abort_flag, status0, kWaitTimeoutNs))
-                        break;
-                    taken ^= 1u;
-                }
-                if (!wait_bar<PAIR>(&rempty[ri], rphase ^ 1u, abort_flag, status0, kWaitTimeoutNs))
-                    break;
-                const int next = L.tile_lo + atomicAdd(L.tile_counter, 1);
-                int t = next < total ? next : -1;
-                TileCoord tc{-1, 0, 0, false};
-                if (t >= 0)
-                    tc = decode_tile<BN, TILE_ROWS, STRIPS>(L, t, hint);
-                EpiScales sc{1.f, 0.f, 0.f};
-                int geom = 0;
-                bool ok = true;
-                if (tc.valid) {
-                    const TcProblem &P = prob_at(L, tc.prob);
-                    // The fields that the other roles read, into L1, and the tensor maps of the
-                    // first segment into the descriptor cache.
-                    const char *pb = reinterpret_cast<const char *>(&P.o_tma);
-                    const int nlines =
-                        (int)((sizeof(TcProblem) - offsetof(TcProblem, o_tma) + 127) / 128) + 1;
-                    for (int k = 0; k < nlines; ++k)
-                        asm volatile("prefetch.L1 [%0];" ::"l"(pb + 128 * k));
-                    prefetch_tensormap(&P.mapL[P.segL[0]]);
-                    prefetch_tensormap(&P.mapR[P.segR[0]]);
-                    geom = pack_geom(P);
-                    // Operands are results of earlier problems. Strip launches wait here until
-                    // the strips this tile reads are complete (L: the strip of this tile's row,
-                    // R: of its column), and so do tiles whose scales come from a norm. Other
-                    // tiles are handed on; where their dependencies are not met yet the producer
-                    // waits itself, which leaves no hand-over between the last counter and the
-                    // first copy.
-                    const bool wait_here = STRIPS || P.ep.theta_src;
-                    bool ready = true;
-                    if (!STRIPS || tc.prob != dep_prob) {  // strips: once per problem, counts only grow
-                        for (int d = 0; d < 2 && ok; ++d)
-                            if (P.dep[d] >= 0) {
-                                if (wait_here)
-                                    ok = wait_counter(&L.done[P.dep[d]], P.dep_target[d], abort_flag,
-                                                      status0, dep_limit(L));
-                                else
-                                    ready = ready && ld_acquire_gpu(&L.done[P.dep[d]]) >= P.dep_target[d];
-                            }
-                    }
-                    if (ready)
-                        geom |= kGeomReady;
-                    if (STRIPS) {
-                        if (tc.prob != dep_prob) {
-                            dep_prob = tc.prob;
-                            src_done[0] = !P.sdep_mode[0];
-                            src_done[1] = !P.sdep_mode[1];
-                        }
-                        for (int q = 0; q < 2 && ok; ++q)
-                            if (!src_done[q])
-                                ok = wait_strip(L, P, q, q ? tc.tn : tc.tm, src_done[q], abort_flag,
-                                                status0);
-                        if (P.ep.theta_src)  // the norm its scales come from is complete
-                            for (int d = 0; d < P.nwdep && ok; ++d)
-                                ok = wait_counter(&L.done[P.wdep[d]], P.wdep_target[d], abort_flag,
-                                                  status0, dep_limit(L));
-                    }
-                    if (ok) {
-                        sc = epi_scales(P, calls);
-                        fence_async_global();  // the TMA reads of the tile come after the acquire
-                    }
-                }
-                if (!ok) {  // the wait gave up: end the ring, also for the peer CTA
-                    t = -1;
-                    tc.valid = false;
-                }
-                const int ent[8] = {t, tc.valid ? tc.prob : -1, tc.tm, tc.tn, __float_as_int(sc.alpha),
-                                    __float_as_int(sc.beta), __float_as_int(sc.gamma), geom};
-                volatile int *w = reinterpret_cast<volatile int *>(&ring[ri]);
-#pragma unroll
-                for (int k = 0; k < 8; ++k)
-                    w[k] = ent[k];
-                if (PAIR) {
-                    const uint32_t pw = peer_addr((const void *)&ring[ri], 1);
-#pragma unroll
-                    for (int k = 0; k < 8; ++k)
-                        st_remote_u32(pw + 4 * k, ent[k]);
-                    mbar_arrive_remote(peer_addr(&rfull[ri], 1));
-                }
-                mbar_arrive(&rfull[ri]);
-                if (++ri == kRingTiles) {
-                    ri = 0;
-                    rphase ^= 1u;
-                }
-                if (t < 0)
-                    break;
-            }
-        }
-    } else if (warp == kPubWarp && lane == 0) {
-        // ------------------------------------------------ publisher (fused launches)
-        // Releases a tile's results to the tiles that read them: once every epilogue warp's
-        // stores are complete, one GPU-scope fence (cumulative over what the warps released to
-        // this thread) and the increment of the problem's counter. The fence takes 1700 to 2200
-        // cycles, which the epilogue warps, each fencing for itself, spent between tiles.
-        if (CHAIN) {
-            int ri = 0;
-            uint32_t rphase = 0, par = 0;  // bit i: parity of pdone[i]'s next use
-            for (;;) {
-                if (!wait_bar<PAIR>(&rfull[ri], rphase, abort_flag, status0, kWaitTimeoutNs))
-                    break;
-                const int t = ring[ri].tile, prob = ring[ri].prob, tm = ring[ri].tm, tn = ring[ri].tn;
-                if (prob >= 0) {
-                    const TcProblem &P = prob_at(L, prob);
-                    const int pid = P.pid;
-                    if (!mbar_wait(&pdone[ri], (par >> ri) & 1u, abort_flag, status0, kWaitTimeoutNs))
-                        break;
-                    par ^= 1u << ri;
-                    fence_async_global();
-                    asm volatile("fence.acq_rel.gpu;" ::: "memory");
-                    red_add_relaxed(&L.done[pid], kEpiWarps);
-                    if (STRIPS && P.strip_base >= 0) {  // the strips this tile completes a part of
-                        int *sp = L.strips + P.strip_base;
-                        red_add_relaxed(sp + tm, kEpiWarps);
-                        if (!P.sym)
-                            red_add_relaxed(sp + P.tiles_m + tn, kEpiWarps);
-                        else if (tn != tm)
-                            red_add_relaxed(sp + tn, kEpiWarps);
-                    }
-                }
-                // Released only now: entry ri, and with it pdone[ri], comes round again after this.
-                ring_release(ri);
-                if (++ri == kRingTiles) {
-                    ri = 0;
-                    rphase ^= 1u;
-                }
-                if (t < 0)
-                    break;
-            }
-        }
-    } else if (warp == 0) {
-        // ------------------------------------------------ TMA producer
-        int stage = 0;
-        uint32_t phase = 0;
-        uint32_t issued = 0, issued_parity = 0;  // bit s: stage s loaded / parity of its last load
-        bool ok = true;
-        int ri = 0;
-        uint32_t rphase = 0;
-        int hint = 0;
-        for (int t = t_first; ok; t += t_step) {
-            TileCoord tc;
-            int geom = 0;
-            if (CHAIN) {
-                if (!wait_warp<PAIR>(&rfull[ri], rphase, abort_flag, status0, kWaitTimeoutNs))
-                    break;
-                t = ring[ri].tile;
-                tc.prob = ring[ri].prob;
-                tc.tm = ring[ri].tm;
-                tc.tn = ring[ri].tn;
-                tc.valid = tc.prob >= 0;
-                geom = ring[ri].geom;
-                __syncwarp();
-                if (elect_one())
-                    ring_release(ri);
-                if (++ri == kRingTiles) {
-                    ri = 0;
-                    rphase ^= 1u;
-                }
-                // The scheduler takes the next tile once this one can start: a CTA holding two
-                // tiles that wait would keep work from CTAs that are idle.
-                if (t < 0)
-                    break;
-                if (!tc.valid && (!PAIR || leader) && elect_one())
-                    mbar_arrive(ptaken);
-            } else {
-                if (t >= total)
-                    break;
-                tc = decode_tile<BN, TILE_ROWS, STRIPS>(L, t, hint);
-            }
-            if (!tc.valid)
-                continue;
-            const TcProblem &P = prob_at(L, tc.prob);
-            if (!CHAIN)
-                geom = pack_geom(P);
-            const int kshift = geom_fp8(geom) ? 7 : 6, kblocks = geom_kblocks(geom);
-            const int row0 = (PAIR ? 2 * tc.tm + (int)rank : tc.tm) * kBM;
-            const int col0 = tc.tn * BN + (int)rank * B_ROWS;
-            if (CHAIN) {
-                if (!(geom & kGeomReady)) {
-                    if (lane == 0)
-                        for (int d = 0; d < 2 && ok; ++d)
-                            if (P.dep[d] >= 0)
-                                ok = wait_counter(&L.done[P.dep[d]], P.dep_target[d], abort_flag,
-                                                  status0, dep_limit(L));
-                    ok = __shfl_sync(0xffffffffu, (int)ok, 0);
-                }
-                if (!ok)
-                    break;
-                if ((!PAIR || leader) && elect_one())
-                    mbar_arrive(ptaken);
-                fence_async_global();  // the TMA reads below come after the acquire
-            }
-            for (int sg = 0; sg < geom_segs(geom) && ok; ++sg) {
-                const CUtensorMap *mL = &P.mapL[geom_l(geom, sg)];
-                const CUtensorMap *mR = &P.mapR[geom_r(geom, sg)];
-                for (int kb = 0; kb < kblocks; ++kb) {
-                    if (!wait_warp<PAIR>(&empty[stage], phase ^ 1u, abort_flag, status0, kWaitTimeoutNs)) {
-                        ok = false;
-                        break;
-                    }
-                    if (!elect_one()) {
-                        // the elected lane issues the copies
-                    } else if (PAIR) {
-                        // Both CTAs' bytes complete on the leader's barrier.
-                        const uint32_t fb = peer_addr(&full[stage], 0);
-                        if (leader)
-                            mbar_expect_tx(&full[stage], 2u * (uint32_t)(A_BYTES + B_BYTES));
-                        tma_load_2d_pair(sA + stage * A_BYTES, mL, kb << kshift, row0, fb);
-                        tma_load_2d_pair(sB + stage * B_BYTES, mR, kb << kshift, col0, fb);
-                    } else {
-                        mbar_expect_tx(&full[stage], (uint32_t)(A_BYTES + B_BYTES));
-                        tma_load_2d(sA + stage * A_BYTES, mL, kb << kshift, row0, &full[stage]);
-                        tma_load_2d(sB + stage * B_BYTES, mR, kb << kshift, col0, &full[stage]);
-                    }
-                    issued |= 1u << stage;
-                    issued_parity = (issued_parity & ~(1u << stage)) | (phase << stage);
-                    if (++stage == STAGES) {
-                        stage = 0;
-                        phase ^= 1u;
-                    }
-                }
-            }
-        }
-        // Drain: the last copy into every stage must have landed before exit. The
-        // peer of a pair sees its copies land through the leader's MMA consuming them.
-        for (int s = 0; s < STAGES; ++s)
-            if ((issued >> s) & 1u) {
-                volatile int no_abort = 0;
-                if (!PAIR || leader)
-                    mbar_wait(&full[s], (issued_parity >> s) & 1u, &no_abort, nullptr, kWaitTimeoutNs / 4);
-                else
-                    mbar_wait_cluster(&empty[s], (issued_parity >> s) & 1u, &no_abort, nullptr,
-                                      kWaitTimeoutNs / 4);
-            }
-    } else if (warp == 1 && (!PAIR || leader)) {
-        // ------------------------------------------------ MMA issuer
-        // The whole warp runs the loop and one elected lane issues: its operands then live in
-        // uniform registers. A loop that only lane 0 ran took 132 cycles an MMA whatever its
-        // shape, twice what a 128 x 128 x 16 needs.
-        const uint64_t desc_a = sw128_desc(smem_u32(sA)), desc_b = sw128_desc(smem_u32(sB));
-        int stage = 0;
-        uint32_t phase = 0;
-        int buf = 0;
-        uint32_t tphase = 0;
-        bool ok = true;
-        int ri = 0;
-        uint32_t rphase = 0;
-        int hint = 0;
-        for (int t = t_first; ok; t += t_step) {
-            TileCoord tc;
-            int geom = 0;
-            if (CHAIN) {
-                if (!wait_warp<false>(&rfull[ri], rphase, abort_flag, status0, kWaitTimeoutNs))
-                    break;
-                t = ring[ri].tile;
-                tc.prob = ring[ri].prob;
-                tc.tm = ring[ri].tm;
-                tc.tn = ring[ri].tn;
-                tc.valid = tc.prob >= 0;
-                geom = ring[ri].geom;
-                __syncwarp();
-                if (elect_one())
-                    ring_release(ri);
-                if (++ri == kRingTiles) {
-                    ri = 0;
-                    rphase ^= 1u;
-                }
-                if (t < 0)
-                    break;
-            } else {
-                if (t >= total)
-                    break;
-                tc = decode_tile<BN, TILE_ROWS, STRIPS>(L, t, hint);
-                if (tc.valid)
-                    geom = pack_geom(prob_at(L, tc.prob));
-            }
-            if (!tc.valid)
-                continue;
-            if (!wait_warp<PAIR>(&tempty[buf], tphase ^ 1u, abort_flag, status0, kWaitTimeoutNs))
-                break;
-            tc_fence_after();
-            const uint32_t d_tmem = tmem_base + (uint32_t)(buf * BN);
-            // The tile's k-loop, one copy per operand kind chosen once per tile, so that
-            // the BF16 loop carries no test of the kind: for each segment and k-block,
-            // wait for the stage's copies, issue four MMAs over its 128 bytes of each row
-            // (K = 16 BF16 or 32 e4m3 elements each) and release the stage.
-            auto k_loop = [&](auto f8_tag) -> bool {
-                constexpr bool F8 = decltype(f8_tag)::value;
-                constexpr uint32_t id = F8 ? idesc_e4m3(TILE_ROWS, BN) : idesc_bf16(TILE_ROWS, BN);
-                const int kblocks = geom_kblocks(geom), segs = geom_segs(geom);
-                uint32_t acc = 0;
-                for (int sg = 0; sg < segs; ++sg) {
-                    for (int kb = 0; kb < kblocks; ++kb) {
-                        if (!wait_warp<false>(&full[stage], phase, abort_flag, status0, kWaitTimeoutNs))
-                            return false;
-                        tc_fence_after();
-                        if (elect_one()) {
-                            // Descriptor addresses count 16-byte units; a K step is 32 bytes.
-                            const uint64_t a0 = desc_a + (uint32_t)(stage * (A_BYTES >> 4));
-                            const uint64_t b0 = desc_b + (uint32_t)(stage * (B_BYTES >> 4));
-#pragma unroll
-                            for (int kk = 0; kk < kBK / 16; ++kk) {
-                                const uint64_t ad = a0 + 2 * kk, bd = b0 + 2 * kk;
-                                const uint32_t on = kk == 0 ? acc : 1u;
-                                if (F8) {
-                                    if (PAIR)
-                                        mma_e4m3_pair(d_tmem, ad, bd, id, on);
-                                    else
-                                        mma_e4m3(d_tmem, ad, bd, id, on);
-                                } else {
-                                    if (PAIR)
-                                        mma_bf16_pair(d_tmem, ad, bd, id, on);
-                                    else
-                                        mma_bf16(d_tmem, ad, bd, id, on);
-                                }
-                            }
-                            if (PAIR)
-                                mma_commit_both(&empty[stage]);
-                            else
-                                mma_commit(&empty[stage]);
-                        }
-                        __syncwarp();
-                        acc = 1;
-                        if (++stage == STAGES) {
-                            stage = 0;
-                            phase ^= 1u;
-                        }
-                    }
-                }
-                return true;
-            };
-            ok = geom_fp8(geom) ? k_loop(BoolTag<true>{}) : k_loop(BoolTag<false>{});
-            if (!ok)
-                break;
-            if (elect_one()) {
-                if (PAIR)
-                    mma_commit_both(&tfull[buf]);
-                else
-                    mma_commit(&tfull[buf]);
-            }
-            __syncwarp();
-            if (++buf == 2) {
-                buf = 0;
-                tphase ^= 1u;
-            }
-        }
-        // Drain: every MMA issued so far completes before tensor memory is freed.
-        if (elect_one()) {
-            if (PAIR)
-                mma_commit_pair_local(drain);
-            else
-                mma_commit(drain);
-        }
-        __syncwarp();
-        volatile int no_abort = 0;
-        mbar_wait(drain, 0, &no_abort, nullptr, kWaitTimeoutNs / 4);
-    } else if (warp >= 2 && warp < kSchedWarp) {
-        // ------------------------------------------------ epilogue
-        const int quad = warp & 3;  // TMEM lane quadrant this warp may access
-        const int half = (warp - 2) >> 2;  // two warps per quadrant split the column chunks
-        uint8_t *stage_buf = stage_all + (warp - 2) * kStgBytes;
-        int slot = 0;  // next staging slot of this warp
-        int buf = 0;
-        uint32_t tphase = 0;
-        int last_prob = -1;
-        bool c_done = true;
-        int ri = 0;
-        uint32_t rphase = 0;
-        int hint = 0;
-        for (int t = t_first;; t += t_step) {
-            TileCoord tc;
-            EpiScales sc;
-            int entry = 0;  // the tile's ring entry
-            if (CHAIN) {
-                if (!wait_bar<PAIR>(&rfull[ri], rphase, abort_flag, status0, kWaitTimeoutNs))
-                    break;
-                t = ring[ri].tile;
-                tc.prob = ring[ri].prob;
-                tc.tm = ring[ri].tm;
-                tc.tn = ring[ri].tn;
-                tc.valid = tc.prob >= 0;
-                sc = EpiScales{ring[ri].alpha, ring[ri].beta, ring[ri].gamma};
-                entry = ri;
-                __syncwarp();
-                if (lane == 0)
-                    ring_release(ri);
-                if (++ri == kRingTiles) {
-                    ri = 0;
-                    rphase ^= 1u;
-                }
-                if (t < 0)
-                    break;
-            } else {
-                if (t >= total)
-                    break;
-                tc = decode_tile<BN, TILE_ROWS, STRIPS>(L, t, hint);
-            }
-            if (!tc.valid)
-                continue;
-            const TcProblem &P = prob_at(L, tc.prob);
-            if (CHAIN && !STRIPS && P.ep.c_kind != C_NONE) {
-                // C is an earlier result: make it visible to these loads.
-                for (int d = 0; d < 2; ++d)
-                    if (P.dep[d] >= 0 && lane == 0)
-                        wait_counter(&L.done[P.dep[d]], P.dep_target[d], abort_flag, status0,
-                                     dep_limit(L));
-                __syncwarp();
-            }
-            if (STRIPS) {
-                // C is an earlier result: make it visible to these loads; earlier readers of the
-                // buffers this tile overwrites must be done.
-                if (lane == 0) {
-                    if (tc.prob != last_prob) {  // once per problem: counts only grow
-                        if (P.ep.c_kind != C_NONE)
-                            for (int d = 0; d < 2; ++d)
-                                if (P.dep[d] >= 0)
-                                    wait_counter(&L.done[P.dep[d]], P.dep_target[d], abort_flag,
-                                                 status0, dep_limit(L));
-                        for (int d = 0; d < P.nwdep; ++d)
-                            wait_counter(&L.done[P.wdep[d]], P.wdep_target[d], abort_flag,
-                                         status0, dep_limit(L));
-                        c_done = !P.sdep_mode[2];
-                    }
-                    if (!c_done)
-                        wait_strip(L, P, 2, tc.tm, c_done, abort_flag, status0);
-                }
-                __syncwarp();
-            }
-            if (PAIR)
-                tc.tm = 2 * tc.tm + (int)rank;  // this CTA's 128-row half of the tile
-            EpiHot h;  // per tile: its registers are free outside the tile's loops
-            if (!CHAIN)
-                sc = epi_scales(P, calls);
-            load_hot(h, P, calls, sc);
-            const int spec = epi_spec(h);
-            last_prob = tc.prob;
-            const int64_t warp_row0 = (int64_t)tc.tm * kBM + quad * 32;
-            const int64_t row = warp_row0 + lane;
-            const bool row_ok = row < h.M;
-            // This warp's 32-column chunks: both of every other 64-column unit, skipping chunks
-            // right of N or wholly below the diagonal (warp-uniform).
-            auto next_chunk = [&](int ch) {
-                for (; ch < BN / 32; ch += (ch & 1) ? 3 : 1) {
-                    const int64_t c0 = (int64_t)tc.tn * BN + ch * 32;
-                    if (c0 < h.N && warp_row0 < h.M && !(h.sym && warp_row0 > c0 + 31))
-                        break;
-                }
-                return ch;
-            };
-            auto after = [&](int ch) { return next_chunk(ch + ((ch & 1) ? 3 : 1)); };
-            auto full_row = [&](int ch) {
-                return row_ok && (int64_t)h.N - ((int64_t)tc.tn * BN + ch * 32) >= 32;
-            };
-            int ch = next_chunk(2 * half);
-            // The first chunk's C is loaded while the accumulator is still being computed.
-            CRaw cr;
-            bool cvec = false;
-            if (ch < BN / 32) {
-                if (spec == 1)
-                    c_load_frag<false>(h, warp_row0, (int64_t)tc.tn * BN + ch * 32, lane, cr);
-                else if (spec == 4)
-                    c_load_frag<true>(h, warp_row0, (int64_t)tc.tn * BN + ch * 32, lane, cr);
-                else if (spec < 0)
-                    cvec = c_load(h, row, (int64_t)tc.tn * BN + ch * 32, full_row(ch), cr);
-            }
-            if (!wait_bar<PAIR>(&tfull[buf], tphase, abort_flag, status0, kWaitTimeoutNs))
-                break;
-            tc_fence_after();
-            double nrm = 0.0;
-            const uint32_t acc0 = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(buf * BN);
-            // The chunk loop, one copy per product kind (epi_spec, chosen once per tile):
-            // the specialised copies carry no tests of output, C, norm and copy kinds.
-            auto chunk_loop = [&](auto spec_tag) {
-                using Spec = decltype(spec_tag);
-#pragma unroll 1
-                while (ch < BN / 32) {
-                    const int nx = after(ch);
-                    const int64_t c0 = (int64_t)tc.tn * BN + ch * 32;
-                    if constexpr (Spec::generic) {
-                        const int64_t rem = (int64_t)h.N - c0;
-                        float v[32];
-                        tmem_ld32(acc0 + (uint32_t)(ch * 32), v);
-#pragma unroll
-                        for (int i = 0; i < 32; ++i)
-                            v[i] *= h.alpha;
-                        c_apply(h, cr, cvec, row, c0, rem < 32 ? (int)rem : 32, row_ok, v);
-                        // The next chunk's C is in flight while this chunk is stored.
-                        if (nx < BN / 32)
-                            cvec = c_load(h, row, (int64_t)tc.tn * BN + nx * 32, full_row(nx), cr);
-                        epilogue_finish<kStgSlots>(h, warp_row0, c0, v, nrm, stage_buf, slot, lane);
-                    } else {
-                        constexpr int S = Spec::code;
-                        const uint32_t stg = smem_u32(stage_buf);
-                        const bool meets = Spec::sym && (c0 & ~(int64_t)63) < warp_row0 + 32;
-                        const bool unit = !Spec::pair && !meets;  // staged with its neighbour
-                        if (!unit || !(ch & 1)) {  // the staging's last stores have been read
-                            if (elect_one())
-                                bulk_wait_read0();
-                            __syncwarp();
-                        }
-                        const bool diag = Spec::sym && c0 == warp_row0;
-                        const uint32_t ta = acc0 + (uint32_t)(ch * 32);
-                        if (unit) {
-                            if constexpr (!Spec::pair)
-                                spec_block<S, STAGE_UNIT>(h, cr, ta, warp_row0, c0, stg, ch & 1, lane);
-                        } else if (diag) {
-                            if constexpr (Spec::sym)
-                                spec_block<S, STAGE_DIAG>(h, cr, ta, warp_row0, c0, stg, 0, lane);
-                        } else {
-                            spec_block<S, STAGE_BLOCK>(h, cr, ta, warp_row0, c0, stg, 0, lane);
-                        }
-                        // The next chunk's C is in flight while this chunk is stored.
-                        if (Spec::has_c && nx < BN / 32)
-                            c_load_frag<Spec::pair>(h, warp_row0, (int64_t)tc.tn * BN + nx * 32, lane, cr);
-                        if (!unit || (nx >> 1) != (ch >> 1)) {  // a block, or a unit's last chunk
-                            fence_async_smem();
-                            __syncwarp();
-                            if (elect_one()) {
-                                const int x = unit ? (int)(c0 & ~(int64_t)63) : (int)c0, y = (int)warp_row0;
-                                const CUtensorMap *m = h.maps;
-                                if (unit) {
-                                    tma_store_2d(&m[4], x, y, stage_buf);
-                                    tma_store_2d(&m[5], y, x, stage_buf + kStgMirror64);
-                                } else {
-                                    const CUtensorMap *mm = Spec::sym ? m : m + 2;
-                                    tma_store_2d(&m[0], x, y, stage_buf);
-                                    if (!diag)
-                                        tma_store_2d(&mm[0], y, x, stage_buf + kStgMirror);
-                                    if (Spec::pair) {
-                                        tma_store_2d(&m[1], x, y, stage_buf + kStgLo);
-                                        if (!diag)
-                                            tma_store_2d(&mm[1], y, x, stage_buf + kStgLo + kStgMirror);
-                                    }
-                                }
-                                bulk_commit();
-                            }
-                        }
-                    }
-                    ch = nx;
-                }
-            };
-            if (!CHAIN) {  // the previous tile's stores have read the staging
-                if (elect_one())
-                    bulk_wait_read0();
-                __syncwarp();
-            }
-            switch (spec) {
-            case 0: chunk_loop(EpiSpec<0>{}); break;
-            case 1: chunk_loop(EpiSpec<1>{}); break;
-            case 2: chunk_loop(EpiSpec<2>{}); break;
-            case 3: chunk_loop(EpiSpec<3>{}); break;
-            case 4: chunk_loop(EpiSpec<4>{}); break;
-            case 5: chunk_loop(EpiSpec<5>{}); break;
-            default: chunk_loop(EpiSpec<-1>{}); break;
-            }
-            if (h.norm_acc) {
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1)
-                    nrm += __shfl_xor_sync(0xffffffffu, nrm, o);
-                if (lane == 0 && nrm != 0.0)
-                    atomicAdd(h.norm_acc, nrm);
-            }
-            tc_fence_before();
-            if (PAIR) {
-                // One release per warp, on the leader's barrier (it issues the next MMAs).
-                __syncwarp();
-                if (lane == 0)
-                    mbar_arrive_remote(peer_addr(&tempty[buf], 0));
-            } else {
-                mbar_arrive(&tempty[buf]);
-            }
-            if (++buf == 2) {
-                buf = 0;
-                tphase ^= 1u;
-            }
-            if (CHAIN) {
-                // This warp's part of the tile is in global memory: tell the publisher. The
-                // lanes' plain stores (diagonal blocks of symmetric products, ragged edges) are
-                // ordered before lane 0's arrival by __syncwarp, its TMA stores by their
-                // completion.
-                __syncwarp();
-                if (elect_one()) {
-                    bulk_wait_all0();
-                    fence_async_global();
-                    mbar_arrive(&pdone[entry]);
-                }
-                __syncwarp();
-            }
-        }
-        // All TMA stores of this warp complete before the CTA may exit.
-        if (elect_one())
-            bulk_wait_all0();
-        __syncwarp();
-    }
-
-    tc_fence_before();
-    __syncthreads();
-    if (PAIR)
-        cluster_sync_all();  // neither CTA leaves while its peer may still signal it
-    if (warp == 1) {
-        __syncwarp();
-        tc_fence_after();
-        tmem_dealloc<PAIR>(tmem_base, 2 * BN);
-    }
-}
-
-static_assert(offsetof(TcProblem, mapT) == offsetof(TcProblem, mapO) + 2 * sizeof(CUtensorMap) &&
-                  offsetof(TcProblem, mapU) == offsetof(TcProblem, mapT) + 2 * sizeof(CUtensorMap),
-              "the epilogue addresses mapO, mapT and mapU as one array");
-
-template <int BN, int STAGES, bool PAIR>
-constexpr int smem_bytes()
-{
-    return STAGES * (kBM + (PAIR ? BN / 2 : BN)) * kBK * 2 +
-           kEpiWarps * kStgBytes /* epilogue staging */ + 1024 /* alignment slack */ +
-           512 /* barriers, tile ring */;
-}
-
-// One launch of the product kernel over total_tiles tiles (tile-width code's
-// tiles: CTA pairs for kBnPair). Persistent: at most one CTA (pair) per SM (pair).
-template <int BN, int STAGES, bool CHAIN, bool PAIR, bool STRIPS = false>
-cudaError_t launch_kernel(const TcLaunch &l, int total_tiles, int num_sms, cudaStream_t s)
-{
-    constexpr int smem = smem_bytes<BN, STAGES, PAIR>();
-    static_assert(smem <= 232448, "shared memory per CTA");
-    auto kern = tc_gemm_kernel<BN, STAGES, CHAIN, PAIR, STRIPS>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e != cudaSuccess)
-        return e;
-    if (total_tiles <= 0)
-        return cudaSuccess;
-    cudaLaunchConfig_t cfg = {};
-    cfg.blockDim = dim3(kThreads, 1, 1);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    int grid = total_tiles < num_sms ? total_tiles : num_sms;
-    if (PAIR) {
-        attr[0].id = cudaLaunchAttributeClusterDimension;
-        attr[0].val.clusterDim.x = 2;
-        attr[0].val.clusterDim.y = 1;
-        attr[0].val.clusterDim.z = 1;
-        cfg.attrs = attr;
-        cfg.numAttrs = 1;
-        // Pairs that can be resident at once (SMs pair up within a GPC).
-        static int max_pairs = -1;
-        if (max_pairs < 0) {
-            cfg.gridDim = dim3((unsigned)(num_sms & ~1), 1, 1);
-            int nc = 0;
-            if (cudaOccupancyMaxActiveClusters(&nc, kern, &cfg) != cudaSuccess || nc <= 0) {
-                cudaGetLastError();
-                nc = num_sms / 2;
-            }
-            max_pairs = nc;
-        }
-        const int cap = std::min(max_pairs, num_sms / 2);  // a caller's SM budget caps it too
-        const int pairs = std::max(1, std::min(total_tiles, cap));
-        grid = 2 * pairs;
-    }
-    cfg.gridDim = dim3((unsigned)grid, 1, 1);
-    return cudaLaunchKernelEx(&cfg, kern, l);
-}
-
-template <bool CHAIN>
-cudaError_t launch_width(const TcLaunch &l, int bn, int total_tiles, int num_sms, cudaStream_t s)
-{
-    // 128 x 128 tiles serve small problems (short K): 5 stages and two staging slots
-    // per epilogue warp, so that stores overlap; the wide tiles keep every byte for
-    // pipeline stages.
     if (bn == 256)
-        return launch_kernel<256, 3, CHAIN, false>(l, total_tiles, num_sms, s);
+        return tc_launch_256(l, chain, total_tiles, num_sms, s);
     if (bn == 128)
-        return launch_kernel<128, 5, CHAIN, false>(l, total_tiles, num_sms, s);
+        return tc_launch_128(l, chain, total_tiles, num_sms, s);
     if (bn == kBnPair)
-        return launch_kernel<256, 5, CHAIN, true>(l, total_tiles, num_sms, s);
+        return tc_launch_pair(l, chain, false, total_tiles, num_sms, s);
     if (bn == kBnPair128)
-        return launch_kernel<128, 6, CHAIN, true>(l, total_tiles, num_sms, s);
+        return tc_launch_pair128(l, chain, total_tiles, num_sms, s);
     return cudaErrorInvalidValue;
 }
 
@@ -1709,14 +28,10 @@ cudaError_t tc_gemm_launch_fused(const TcLaunch &l, int bn, int total_tiles, int
 {
     TcLaunch g = l;
     g.nprob = 0;
-    if (strips) {  // square tiles only: per-strip dependencies
-        if (bn == 128)
-            return launch_kernel<128, 5, true, false, true>(g, total_tiles, num_sms, s);
-        if (bn == kBnPair)
-            return launch_kernel<256, 5, true, true, true>(g, total_tiles, num_sms, s);
-        return cudaErrorInvalidValue;
-    }
-    return launch_width<true>(g, bn, total_tiles, num_sms, s);
+    if (strips)  // per-strip dependencies
+        return bn == kBnPair ? tc_launch_pair(g, true, true, total_tiles, num_sms, s)
+                             : cudaErrorInvalidValue;
+    return launch_width(g, true, bn, total_tiles, num_sms, s);
 }
 
 int tc_num_tiles(const TcProblem &p, int bn)
@@ -1739,7 +54,7 @@ cudaError_t tc_gemm_launch(const TcLaunch &l, int bn, int num_sms, cudaStream_t 
 {
     if (l.gtab)
         return cudaErrorInvalidValue;
-    return launch_width<false>(l, bn, l.tile_start[l.nprob], num_sms, s);
+    return launch_width(l, false, bn, l.tile_start[l.nprob], num_sms, s);
 }
 
 } // namespace svt

@@ -194,9 +194,16 @@ int tc_valid_ctas(const TcProblem &p, int bn);
 cudaError_t tc_gemm_launch(const TcLaunch &l, int bn, int num_sms, cudaStream_t s);
 // Fused launch: l.gtab / l.gstart / l.gcount hold every product of a solve in
 // dependency order; l.tile_counter and l.done point to zeroed device counters.
-// strips: the table carries per-strip dependencies (square tiles: bn 128 or kBnPair).
+// strips: the table carries per-strip dependencies (bn kBnPair only).
 cudaError_t tc_gemm_launch_fused(const TcLaunch &l, int bn, int total_tiles, int num_sms,
                                  cudaStream_t s, bool strips = false);
+// One launch of the product kernel in one tile configuration (each in its own translation unit).
+cudaError_t tc_launch_128(const TcLaunch &l, bool chain, int total_tiles, int num_sms, cudaStream_t s);
+cudaError_t tc_launch_256(const TcLaunch &l, bool chain, int total_tiles, int num_sms, cudaStream_t s);
+cudaError_t tc_launch_pair(const TcLaunch &l, bool chain, bool strips, int total_tiles, int num_sms,
+                           cudaStream_t s);
+cudaError_t tc_launch_pair128(const TcLaunch &l, bool chain, int total_tiles, int num_sms,
+                              cudaStream_t s);
 constexpr int kEpiWarpsPublic = 8;  // completion count per tile of a fused launch
 cudaError_t f64_gemm_launch(const F64Launch &l, cudaStream_t s);
 
