@@ -12,12 +12,12 @@
 // 1/2 (A - tau P)(I + S) of Proposition 1.
 //
 // Structure (persistent, one CTA per SM, 384 threads):
-//   warp 0    : TMA producer (one thread), STAGES-deep shared-memory ring.
-//   warp 1    : tensor-memory allocator and MMA issuer (one thread).
+//   warp 0    : TMA producer (an elected lane), STAGES-deep shared-memory ring.
+//   warp 1    : tensor-memory allocator and MMA issuer (an elected lane).
 //   warps 2-9 : epilogue; warp w reads TMEM lanes 32 (w % 4) .. 32 (w % 4) + 31, and
-//               the two warps of a lane quadrant take alternate 32-column chunks.
-//   warp 10   : tile scheduler of fused launches (one thread): takes, decodes and waits for
-//               the next tile's dependencies while the producer loads the current one.
+//               the two warps of a lane quadrant take alternate 64-column units.
+//   warp 10   : tile scheduler of fused launches: takes and decodes the next tile and checks
+//               its dependencies while the producer loads the current one.
 //   warp 11   : publisher of fused launches (one thread): releases finished tiles.
 // Two accumulator buffers of BN FP32 columns each let the epilogue of one tile
 // overlap the MMAs of the next.
@@ -91,47 +91,15 @@ __device__ __forceinline__ const TcProblem &prob_at(const TcLaunch &L, int p)
     return L.gtab ? L.gtab[p] : L.p[p];
 }
 
-// Linear tile index -> (problem, tile row, tile column) for tiles of TM x BN.
+// The tile of index `local` within problem p, for tiles of TM x BN.
 // Dense problems: column-major over the tile grid. Symmetric problems: only
 // tiles holding some element with row <= col; column tn holds r (tn + 1) row
 // tiles (r = BN / TM), so the first tile of column tn is r tn (tn + 1) / 2
 // (tiles taller than wide, and ROWMAJOR_SYM with square tiles: see below).
-// A role's tile indices only increase, so the problem search gallops forward from
-// the previous answer (`hint`) instead of bisecting the whole table: a few
-// dependent loads of the tile prefix sums instead of log2(problems).
 template <int BN, int TM, bool ROWMAJOR_SYM>
-__device__ TileCoord decode_tile(const TcLaunch &L, int t, int &hint)
+__device__ TileCoord tile_coord(const TcProblem &P, int p, int local)
 {
-    TileCoord tc{0, 0, 0, false};
-    int p = 0, start = 0;
-    if (L.gtab) {
-        p = hint;
-        if (p < 0 || p >= L.gcount || L.gstart[p] > t)
-            p = 0;
-        int step = 1, q = p + 1;  // first q > p with gstart[q] > t lies in (p, q]
-        while (q < L.gcount && L.gstart[q] <= t) {
-            p = q;
-            step <<= 1;
-            q = p + step;
-        }
-        int hi = (q < L.gcount ? q : L.gcount) - 1;  // last p with gstart[p] <= t
-        while (p < hi) {
-            const int mid = (p + hi + 1) >> 1;
-            if (L.gstart[mid] <= t)
-                p = mid;
-            else
-                hi = mid - 1;
-        }
-        hint = p;
-        start = L.gstart[p];
-    } else {
-        while (p + 1 < L.nprob && t >= L.tile_start[p + 1])
-            ++p;
-        start = L.tile_start[p];
-    }
-    const TcProblem &P = prob_at(L, p);
-    int local = t - start;
-    tc.prob = p;
+    TileCoord tc{p, 0, 0, false};
     if (!P.sym) {
         tc.tm = local % P.tiles_m;
         tc.tn = local / P.tiles_m;
@@ -140,8 +108,8 @@ __device__ TileCoord decode_tile(const TcLaunch &L, int t, int &hint)
     }
     constexpr int r = BN / TM;
     if (r == 0) {
-        // Tiles twice as tall as wide: columns 2 j and 2 j + 1 hold j + 1 row tiles each, the
-        // first of them from index j (j + 1) on.
+        // Tiles twice as tall as wide (256 x 128): columns 2 j and 2 j + 1 hold j + 1
+        // row tiles each, the first of them from index j (j + 1) on.
         int j = (int)((sqrtf(4.0f * (float)local + 1.0f) - 1.0f) * 0.5f);
         while (j > 0 && j * (j + 1) > local)
             --j;
@@ -181,6 +149,33 @@ __device__ TileCoord decode_tile(const TcLaunch &L, int t, int &hint)
     tc.tn = tn;
     tc.valid = (tm < P.tiles_m) && (tn < P.tiles_n);
     return tc;
+}
+
+// Tile t of a launch with its problems by value (not fused).
+template <int BN, int TM, bool ROWMAJOR_SYM>
+__device__ TileCoord decode_tile(const TcLaunch &L, int t)
+{
+    int p = 0;
+    while (p + 1 < L.nprob && t >= L.tile_start[p + 1])
+        ++p;
+    return tile_coord<BN, TM, ROWMAJOR_SYM>(L.p[p], p, t - L.tile_start[p]);
+}
+
+// Problem of tile t in a fused launch's table, by a whole warp. Its tiles' indices only increase,
+// so the search goes on from the previous answer (`p`, first tile `start`), 32 problems a load: in
+// a batch a CTA's next tile is some twenty problems on, which took one thread nine dependent loads.
+__device__ __forceinline__ void find_problem(const TcLaunch &L, int t, int lane, int &p, int &start)
+{
+    for (;;) {
+        const int q = p + 1 + lane;
+        const int first = q < L.gcount ? L.gstart[q] : 0x7fffffff;
+        const int n = __popc(__ballot_sync(0xffffffffu, first <= t));  // starts increase: a prefix
+        if (n > 0)
+            start = __shfl_sync(0xffffffffu, first, n - 1);
+        p += n;
+        if (n < 32)
+            return;
+    }
 }
 
 // ------------------------------------------------------------- epilogue
@@ -998,6 +993,8 @@ struct RingTile {
     int geom;  // see pack_geom
 };
 
+constexpr int kMaxMaps = 2;  // tensor maps of an operand: hi and lo part
+
 // k-blocks of a segment in bits 0..15 (K < 2^21), segments in 16..17, their L and R parts in
 // 18..20 and 21..23, e4m3 operands in 24, "the operands' dependencies are met" in 25.
 constexpr int kGeomReady = 1 << 25;
@@ -1112,45 +1109,54 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
         else
             mbar_arrive(&rempty[ri]);
     };
-    if (warp == kSchedWarp && lane == 0) {
+    if (warp == kSchedWarp) {
         // ------------------------------------------------ tile scheduler (fused launches)
         // Takes tiles in table order, one ahead of the one the producer is loading, so that the
         // counter's round trip, the decoding, the tensor maps' and problem fields' fetches and
-        // the dependency wait of a tile run beside the copies of the tile before it (in the
+        // the dependency check of a tile run beside the copies of the tile before it (in the
         // producer they cost 2200 cycles between tiles). With the publisher: 256-matrix batch
-        // 10.03 -> 8.68 ms, single solves 1 to 2 % faster.
+        // 10.03 -> 8.68 ms, single solves 1 to 2 % faster. The whole warp works on one tile.
         if (CHAIN && (!PAIR || leader)) {
-            int ri = 0, hint = 0;
+            int ri = 0, prob = 0, start = 0;
             uint32_t rphase = 0, taken = 0;
             int dep_prob = -1;  // problem whose whole dependencies have been waited for
-            bool src_done[2] = {false, false};
+            bool src_done[2] = {false, false};  // lane 0: its strip dependencies that are complete
             for (bool first = true;; first = false) {
                 if (!first) {
-                    if (!mbar_wait(ptaken, taken, abort_flag, status0, kWaitTimeoutNs))
+                    if (!wait_warp<false>(ptaken, taken, abort_flag, status0, kWaitTimeoutNs))
                         break;
                     taken ^= 1u;
                 }
-                if (!wait_bar<PAIR>(&rempty[ri], rphase ^ 1u, abort_flag, status0, kWaitTimeoutNs))
+                if (!wait_warp<PAIR>(&rempty[ri], rphase ^ 1u, abort_flag, status0, kWaitTimeoutNs))
                     break;
-                const int next = L.tile_lo + atomicAdd(L.tile_counter, 1);
-                int t = next < total ? next : -1;
+                int t = 0;
+                if (lane == 0)
+                    t = L.tile_lo + atomicAdd(L.tile_counter, 1);
+                t = __shfl_sync(0xffffffffu, t, 0);
+                if (t >= total)
+                    t = -1;
                 TileCoord tc{-1, 0, 0, false};
-                if (t >= 0)
-                    tc = decode_tile<BN, TILE_ROWS, STRIPS>(L, t, hint);
+                if (t >= 0) {
+                    find_problem(L, t, lane, prob, start);
+                    tc = tile_coord<BN, TILE_ROWS, STRIPS>(L.gtab[prob], prob, t - start);
+                }
                 EpiScales sc{1.f, 0.f, 0.f};
                 int geom = 0;
                 bool ok = true;
                 if (tc.valid) {
-                    const TcProblem &P = prob_at(L, tc.prob);
-                    // The fields that the other roles read, into L1, and the tensor maps of the
-                    // first segment into the descriptor cache.
+                    const TcProblem &P = L.gtab[tc.prob];
+                    // The fields that the other roles read, into L1, and the tensor maps into the
+                    // descriptor cache.
                     const char *pb = reinterpret_cast<const char *>(&P.o_tma);
-                    const int nlines =
+                    constexpr int nlines =
                         (int)((sizeof(TcProblem) - offsetof(TcProblem, o_tma) + 127) / 128) + 1;
-                    for (int k = 0; k < nlines; ++k)
-                        asm volatile("prefetch.L1 [%0];" ::"l"(pb + 128 * k));
-                    prefetch_tensormap(&P.mapL[P.segL[0]]);
-                    prefetch_tensormap(&P.mapR[P.segR[0]]);
+                    static_assert(nlines <= 32 && kMaxMaps <= 32, "one prefetch a lane");
+                    if (lane < nlines)
+                        asm volatile("prefetch.L1 [%0];" ::"l"(pb + 128 * lane));
+                    if (lane < (P.nseg > 1 ? kMaxMaps : 1)) {  // hi, then lo parts
+                        prefetch_tensormap(&P.mapL[lane]);
+                        prefetch_tensormap(&P.mapR[lane]);
+                    }
                     geom = pack_geom(P);
                     // Operands are results of earlier problems. Strip launches wait here until
                     // the strips this tile reads are complete (L: the strip of this tile's row,
@@ -1158,35 +1164,41 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
                     // tiles are handed on; where their dependencies are not met yet the producer
                     // waits itself, which leaves no hand-over between the last counter and the
                     // first copy.
-                    const bool wait_here = STRIPS || P.ep.theta_src;
                     bool ready = true;
-                    if (!STRIPS || tc.prob != dep_prob) {  // strips: once per problem, counts only grow
-                        for (int d = 0; d < 2 && ok; ++d)
-                            if (P.dep[d] >= 0) {
-                                if (wait_here)
-                                    ok = wait_counter(&L.done[P.dep[d]], P.dep_target[d], abort_flag,
-                                                      status0, dep_limit(L));
-                                else
-                                    ready = ready && ld_acquire_gpu(&L.done[P.dep[d]]) >= P.dep_target[d];
+                    if (STRIPS || P.ep.theta_src) {
+                        if (lane == 0) {
+                            if (!STRIPS || tc.prob != dep_prob)  // strips: once per problem, counts only grow
+                                for (int d = 0; d < 2 && ok; ++d)
+                                    if (P.dep[d] >= 0)
+                                        ok = wait_counter(&L.done[P.dep[d]], P.dep_target[d],
+                                                          abort_flag, status0, dep_limit(L));
+                            if (STRIPS) {
+                                if (tc.prob != dep_prob) {
+                                    src_done[0] = !P.sdep_mode[0];
+                                    src_done[1] = !P.sdep_mode[1];
+                                }
+                                for (int q = 0; q < 2 && ok; ++q)
+                                    if (!src_done[q])
+                                        ok = wait_strip(L, P, q, q ? tc.tn : tc.tm, src_done[q],
+                                                        abort_flag, status0);
+                                if (P.ep.theta_src)  // the norm its scales come from is complete
+                                    for (int d = 0; d < P.nwdep && ok; ++d)
+                                        ok = wait_counter(&L.done[P.wdep[d]], P.wdep_target[d],
+                                                          abort_flag, status0, dep_limit(L));
                             }
+                        }
+                        dep_prob = tc.prob;
+                        ok = __shfl_sync(0xffffffffu, (int)ok, 0);
+                    } else if (tc.prob != dep_prob) {  // met once, met for every later tile
+                        const int d = lane < 2 ? P.dep[lane] : -1;
+                        ready = __all_sync(0xffffffffu,
+                                           d < 0 || ld_acquire_gpu(&L.done[d]) >= P.dep_target[lane & 1]);
+                        if (ready)
+                            dep_prob = tc.prob;
                     }
+                    __syncwarp();  // the lanes' acquires come before what follows in the others
                     if (ready)
                         geom |= kGeomReady;
-                    if (STRIPS) {
-                        if (tc.prob != dep_prob) {
-                            dep_prob = tc.prob;
-                            src_done[0] = !P.sdep_mode[0];
-                            src_done[1] = !P.sdep_mode[1];
-                        }
-                        for (int q = 0; q < 2 && ok; ++q)
-                            if (!src_done[q])
-                                ok = wait_strip(L, P, q, q ? tc.tn : tc.tm, src_done[q], abort_flag,
-                                                status0);
-                        if (P.ep.theta_src)  // the norm its scales come from is complete
-                            for (int d = 0; d < P.nwdep && ok; ++d)
-                                ok = wait_counter(&L.done[P.wdep[d]], P.wdep_target[d], abort_flag,
-                                                  status0, dep_limit(L));
-                    }
                     if (ok) {
                         sc = epi_scales(P, calls);
                         fence_async_global();  // the TMA reads of the tile come after the acquire
@@ -1198,18 +1210,22 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
                 }
                 const int ent[8] = {t, tc.valid ? tc.prob : -1, tc.tm, tc.tn, __float_as_int(sc.alpha),
                                     __float_as_int(sc.beta), __float_as_int(sc.gamma), geom};
-                volatile int *w = reinterpret_cast<volatile int *>(&ring[ri]);
+                int word = ent[0];  // lane k < 8 writes word k
 #pragma unroll
-                for (int k = 0; k < 8; ++k)
-                    w[k] = ent[k];
-                if (PAIR) {
-                    const uint32_t pw = peer_addr((const void *)&ring[ri], 1);
-#pragma unroll
-                    for (int k = 0; k < 8; ++k)
-                        st_remote_u32(pw + 4 * k, ent[k]);
-                    mbar_arrive_remote(peer_addr(&rfull[ri], 1));
+                for (int q = 1; q < 8; ++q)
+                    word = lane == q ? ent[q] : word;
+                if (lane < 8) {
+                    reinterpret_cast<volatile int *>(&ring[ri])[lane] = word;
+                    if (PAIR)
+                        st_remote_u32(peer_addr((const void *)&ring[ri], 1) + 4 * lane, word);
                 }
-                mbar_arrive(&rfull[ri]);
+                __syncwarp();
+                if (elect_one()) {
+                    if (PAIR)
+                        mbar_arrive_remote(peer_addr(&rfull[ri], 1));
+                    mbar_arrive(&rfull[ri]);
+                }
+                __syncwarp();
                 if (++ri == kRingTiles) {
                     ri = 0;
                     rphase ^= 1u;
@@ -1267,7 +1283,6 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
         bool ok = true;
         int ri = 0;
         uint32_t rphase = 0;
-        int hint = 0;
         for (int t = t_first; ok; t += t_step) {
             TileCoord tc;
             int geom = 0;
@@ -1296,7 +1311,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
             } else {
                 if (t >= total)
                     break;
-                tc = decode_tile<BN, TILE_ROWS, STRIPS>(L, t, hint);
+                tc = decode_tile<BN, TILE_ROWS, STRIPS>(L, t);
             }
             if (!tc.valid)
                 continue;
@@ -1376,7 +1391,6 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
         bool ok = true;
         int ri = 0;
         uint32_t rphase = 0;
-        int hint = 0;
         for (int t = t_first; ok; t += t_step) {
             TileCoord tc;
             int geom = 0;
@@ -1401,7 +1415,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
             } else {
                 if (t >= total)
                     break;
-                tc = decode_tile<BN, TILE_ROWS, STRIPS>(L, t, hint);
+                tc = decode_tile<BN, TILE_ROWS, STRIPS>(L, t);
                 if (tc.valid)
                     geom = pack_geom(prob_at(L, tc.prob));
             }
@@ -1497,7 +1511,6 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
         bool c_done = true;
         int ri = 0;
         uint32_t rphase = 0;
-        int hint = 0;
         for (int t = t_first;; t += t_step) {
             TileCoord tc;
             EpiScales sc;
@@ -1524,7 +1537,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
             } else {
                 if (t >= total)
                     break;
-                tc = decode_tile<BN, TILE_ROWS, STRIPS>(L, t, hint);
+                tc = decode_tile<BN, TILE_ROWS, STRIPS>(L, t);
             }
             if (!tc.valid)
                 continue;
