@@ -16,9 +16,9 @@ CSRC = os.path.join(HERE, "csrc")
 OUT = os.path.join(HERE, "libsvt.so")
 BUILD = os.path.join(ROOT, "_build")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
-SOURCES = ["gemm_tc_128.cu", "gemm_tc_256.cu", "gemm_tc_pair.cu", "gemm_tc_pair128.cu", "gemm_tc.cu",
-           "small_solve.cu", "aux_kernels.cu", "svt_api.cu", "serve.cpp", "schedule.cpp", "noalloc.cu",
-           "completion.cu", "autotune_schedule.cu"]
+SOURCES = ["gemm_tc_64.cu", "gemm_tc_128.cu", "gemm_tc_256.cu", "gemm_tc_pair.cu", "gemm_tc_pair128.cu",
+           "gemm_tc.cu", "small_solve.cu", "aux_kernels.cu", "svt_api.cu", "serve.cpp", "schedule.cpp",
+           "noalloc.cu", "completion.cu", "autotune_schedule.cu"]
 
 
 def _nvcc() -> str:

@@ -10,6 +10,8 @@ namespace {
 cudaError_t launch_width(const TcLaunch &l, bool chain, int bn, int total_tiles, int num_sms,
                          cudaStream_t s)
 {
+    if (bn == kBn64)
+        return tc_launch_64(l, chain, total_tiles, num_sms, s);
     if (bn == 256)
         return tc_launch_256(l, chain, total_tiles, num_sms, s);
     if (bn == 128)

@@ -108,7 +108,7 @@ __device__ TileCoord tile_coord(const TcProblem &P, int p, int local)
     }
     constexpr int r = BN / TM;
     if (r == 0) {
-        // Tiles twice as tall as wide (256 x 128): columns 2 j and 2 j + 1 hold j + 1
+        // Tiles twice as tall as wide (256 x 128, 128 x 64): columns 2 j and 2 j + 1 hold j + 1
         // row tiles each, the first of them from index j (j + 1) on.
         int j = (int)((sqrtf(4.0f * (float)local + 1.0f) - 1.0f) * 0.5f);
         while (j > 0 && j * (j + 1) > local)
@@ -1581,21 +1581,22 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
             const int64_t warp_row0 = (int64_t)tc.tm * kBM + quad * 32;
             const int64_t row = warp_row0 + lane;
             const bool row_ok = row < h.M;
-            // This warp's 32-column chunks: both of every other 64-column unit, skipping chunks
-            // right of N or wholly below the diagonal (warp-uniform).
+            // This warp's 32-column chunks: both of every other 64-column unit (of a single unit,
+            // one), skipping chunks right of N or wholly below the diagonal (warp-uniform).
+            auto step = [](int ch) { return BN == 64 ? 2 : ((ch & 1) ? 3 : 1); };
             auto next_chunk = [&](int ch) {
-                for (; ch < BN / 32; ch += (ch & 1) ? 3 : 1) {
+                for (; ch < BN / 32; ch += step(ch)) {
                     const int64_t c0 = (int64_t)tc.tn * BN + ch * 32;
                     if (c0 < h.N && warp_row0 < h.M && !(h.sym && warp_row0 > c0 + 31))
                         break;
                 }
                 return ch;
             };
-            auto after = [&](int ch) { return next_chunk(ch + ((ch & 1) ? 3 : 1)); };
+            auto after = [&](int ch) { return next_chunk(ch + step(ch)); };
             auto full_row = [&](int ch) {
                 return row_ok && (int64_t)h.N - ((int64_t)tc.tn * BN + ch * 32) >= 32;
             };
-            int ch = next_chunk(2 * half);
+            int ch = next_chunk(BN == 64 ? half : 2 * half);
             // The first chunk's C is loaded while the accumulator is still being computed.
             CRaw cr;
             bool cvec = false;
@@ -1639,7 +1640,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
                         const uint32_t stg = smem_u32(stage_buf);
                         const bool meets = Spec::sym && (c0 & ~(int64_t)63) < warp_row0 + 32;
                         // staged with its neighbour
-                        const bool unit = !Spec::pair && Spec::mirror && !meets;
+                        const bool unit = BN > 64 && !Spec::pair && Spec::mirror && !meets;
                         if (!Spec::f32_out && (!unit || !(ch & 1))) {
                             if (elect_one())  // the staging's last stores have been read
                                 bulk_wait_read0();
@@ -1650,7 +1651,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
                         if constexpr (!Spec::mirror) {
                             spec_block<S, STAGE_PLAIN>(h, cr, ta, warp_row0, c0, stg, 0, lane, nrm);
                         } else if (unit) {
-                            if constexpr (!Spec::pair)
+                            if constexpr (BN > 64 && !Spec::pair)
                                 spec_block<S, STAGE_UNIT>(h, cr, ta, warp_row0, c0, stg, ch & 1, lane, nrm);
                         } else if (diag) {
                             if constexpr (Spec::sym)

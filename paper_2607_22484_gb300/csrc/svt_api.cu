@@ -1264,20 +1264,26 @@ void evict_plans(svt_ctx *ctx, size_t max_entries)
 }
 
 // Tile mode of a fused solve when none is requested or tuned, from whole-solve timings on
-// GB300 (20 steps, us; 128 x 128 tiles / pairs on 256 x 128 / pairs on 256 x 256):
-//   BF16  512^2 510 / 540 / 692, 1000^2 697 / 710 / 986, 1536^2 947 / 953 / 1164, 1792^2 1189 /
-//         1174 / 1296, 2048^2 1452 / 1405 / 1435, 2304^2 2146 / 2036 / 1800, 8192 x 512 1165 /
-//         1117 / 1391, 8192 x 2048 3146 / 2984 / 2812
-//   FP32  512^2 775 / 774 / 1056, 1000^2 1130 / 1080 / 1493, 1700^2 2390 / 2226 / 2295, 2400 x 600
-//         1321 / 1189 / 1677, 8192 x 512 2613 / 2306 / 3135, 2048^2 3248 / 3097 / 2829
-// 256 x 256 tiles move the fewest operand bytes but leave SMs without a tile until the smaller
-// side is about 1800. Below, pairs on 256 x 128 move 24 KiB per k-block and CTA where 128 x 128
-// tiles move 32, and cost about 300 cycles a tile more (the pair's barriers): they pay from 24
-// k-blocks per product on, the mean over a step of the P chain (X^T X over the larger side, Y^2
-// and X Z over the smaller), each hi/lo segment counted.
-int fused_auto_width(int64_t m, int64_t n, const Resolved &r)
+// GB300 (20 steps, us; 128 x 64 tiles / 128 x 128 / pairs on 256 x 128 / pairs on 256 x 256):
+//   BF16  300^2 363 / 431 / 463 / 557, 512^2 431 / 505 / 529 / 692, 1000^2 609 / 686 / 708 / 986,
+//         1100^2 734 / 728 / 733, 1536^2 1231 / 944 / 948 / 1164, 1792^2 - / 1189 / 1174 / 1296,
+//         2048^2 - / 1452 / 1405 / 1435, 2304^2 - / 2146 / 2036 / 1800, 4096 x 256 601 / 660 / 647,
+//         8192 x 512 1198 / 1176 / 1123 / 1391, 8192 x 2048 - / 3146 / 2984 / 2812
+//   FP32  300^2 519 / 626 / 651 / 840, 1000^2 1060 / 1131 / 1076 / 1493, 1100^2 1370 / 1229 /
+//         1159, 1700^2 - / 2390 / 2226 / 2295, 2400 x 600 1259 / 1310 / 1183 / 1677, 8192 x 512
+//         2652 / 2604 / 2304 / 3135, 2048^2 - / 3248 / 3097 / 2829
+// While the tiles of X Z fit the SMs at once a solve is bound by the latency of one tile after
+// another, and 128 x 64 tiles have the shortest: half the MMAs and one epilogue block a warp.
+// Past that the operand bytes decide. 256 x 256 tiles move the fewest but leave SMs without a
+// tile until the smaller side is about 1800. Below, pairs on 256 x 128 move 24 KiB per k-block and
+// CTA where 128 x 128 tiles move 32, and cost about 300 cycles a tile more (the pair's barriers):
+// they pay from 24 k-blocks per product on, the mean over a step of the P chain (X^T X over the
+// larger side, Y^2 and X Z over the smaller), each hi/lo segment counted.
+int fused_auto_width(int64_t m, int64_t n, const Resolved &r, int num_sms)
 {
     const int64_t M = std::max(m, n), N = std::min(m, n);
+    if ((M + 127) / 128 * ((N + 63) / 64) <= num_sms)
+        return kBn64;
     // Rank-r mode has half the tiles (one chain), so finer ones pay up to 2048 (2048 x 8192: 1221
     // against 1555 us; 2304^2: 1714 against 1465).
     if (N > (r.mode == SVT_MODE_RANK_R ? 2048 : 1792))
@@ -1290,7 +1296,7 @@ svt_status get_plan(svt_ctx *ctx, int64_t m, int64_t n, const Resolved &r, size_
                     size_t ws_avail, Plan **out, int force_bn, std::shared_ptr<Plan> *keep)
 {
     if (force_bn == 0 && r.fuse && r.prec != SVT_FP64)
-        force_bn = fused_auto_width(m, n, r);
+        force_bn = fused_auto_width(m, n, r, ctx->num_sms);
     Key k{m, n, r.iters, r.prec, r.schedule, r.norm, r.polish, r.mode, r.hp_steps, r.ell0, r.delta,
           ws_base, force_bn, r.fuse, r.out64, r.fp8_p, r.fp8_s, r.fp8_s_y2};
     auto it = ctx->plans.find(k);
@@ -1372,13 +1378,29 @@ static bool use_small(const svt_ctx *ctx, int64_t m, int64_t n, const Resolved &
            r.iters <= kSmallIters && !r.fp8_p && !r.fp8_s && !ctx->dbg_wait_ns;
 }
 
+// What a tuned 128 means for a fused solve: 128 x 128 tiles, or the automatic choice where that is
+// one of the finer tiles that are no option values (128 x 64, 256 x 128).
+static int narrow_mode(const svt_ctx *ctx, int64_t m, int64_t n, const Resolved &r)
+{
+    const int a = fused_auto_width(m, n, r, ctx->num_sms);
+    return a == kBn64 || a == kBnPair128 ? a : 128;
+}
+
 svt_status plan_for_solve(svt_ctx *ctx, int64_t m, int64_t n, const Resolved &r, Plan **out,
                           std::shared_ptr<Plan> *keep)
 {
-    const int fbn = r.tile ? r.tile
-                           : (use_small(ctx, m, n, r)
-                                  ? kSmallPlan
-                                  : (ctx->tuning.count(tune_key(m, n, r)) ? -1 : 0));
+    int fbn = 0;
+    if (r.tile) {
+        fbn = r.tile;
+    } else if (use_small(ctx, m, n, r)) {
+        fbn = kSmallPlan;
+    } else {
+        const auto t = ctx->tuning.find(tune_key(m, n, r));
+        if (t != ctx->tuning.end()) {
+            const bool all128 = std::all_of(t->second.begin(), t->second.end(), [](int w) { return w == 128; });
+            fbn = r.fuse && all128 ? narrow_mode(ctx, m, n, r) : -1;
+        }
+    }
     return get_plan(ctx, m, n, r, 0, ctx->ws_bytes, out, fbn, keep);
 }
 
@@ -1671,13 +1693,12 @@ svt_status svt_autotune(svt_ctx_t ctx, const float *A, int64_t m, int64_t n, int
         double best = -1.0;
         int best_w = 0;
         size_t n_tc = 0;
-        // The three modes, and the automatic choice where it is another one (the last).
-        std::vector<int> cand(widths, widths + 3);
-        if (fused_auto_width(m, n, r) == kBnPair128)
-            cand.push_back(kBnPair128);
-        for (size_t w = 0; w < cand.size() && st == SVT_OK; ++w) {
+        // The three modes; where the automatic choice is one of the finer tiles, it stands for
+        // 128 (see narrow_mode).
+        const int narrow = narrow_mode(ctx, m, n, r);
+        for (int w = 0; w < 3 && st == SVT_OK; ++w) {
             Plan *plan = nullptr;
-            st = get_plan(ctx, m, n, r, 0, ctx->ws_bytes, &plan, cand[w]);
+            st = get_plan(ctx, m, n, r, 0, ctx->ws_bytes, &plan, w ? widths[w] : narrow);
             if (st != SVT_OK)
                 break;
             if (!plan->fused)
@@ -1699,7 +1720,7 @@ svt_status svt_autotune(svt_ctx_t ctx, const float *A, int64_t m, int64_t n, int
             cudaEventElapsedTime(&t, e0, e1);
             if (best < 0.0 || t < best) {
                 best = t;
-                best_w = cand[w];
+                best_w = widths[w];
                 n_tc = plan->tc.size();
             }
         }
@@ -1709,8 +1730,7 @@ svt_status svt_autotune(svt_ctx_t ctx, const float *A, int64_t m, int64_t n, int
             return st;
         if (best_w == 0)
             return SVT_OK;  // no width runs fused: keep the automatic choice
-        if (best_w != kBnPair128)  // else nothing is stored: later solves choose it themselves
-            choice.assign(n_tc, best_w);
+        choice.assign(n_tc, best_w);
     } else {
         std::vector<double> ms[3];
         const bool prev_profile = ctx->profile;
@@ -1765,10 +1785,7 @@ svt_status svt_autotune(svt_ctx_t ctx, const float *A, int64_t m, int64_t n, int
         else
             ++it;
     }
-    if (choice.empty())
-        ctx->tuning.erase(tune_key(m, n, r));
-    else
-        ctx->tuning[tune_key(m, n, r)] = choice;
+    ctx->tuning[tune_key(m, n, r)] = choice;
     return SVT_OK;
 }
 

@@ -28,10 +28,11 @@ constexpr int kBK = 64;           // K per pipeline stage: one 128-byte swizzle 
 // Tile-width codes of the product kernel. 128 and 256: one CTA per 128 x bn
 // output tile. kBnPair: a cluster of two CTAs per 256 x 256 tile
 // (tcgen05 cta_group::2), each CTA holding 128 x 256 of it and staging half of
-// the tile's R rows. kBnPair128: such a cluster per 256 x 128 tile (chosen by
-// fused_auto_width, not an option value).
+// the tile's R rows. kBnPair128: such a cluster per 256 x 128 tile; kBn64: one CTA per
+// 128 x 64 tile (these two are chosen by fused_auto_width, they are no option values).
 constexpr int kBnPair = 512;
 constexpr int kBnPair128 = 384;
+constexpr int kBn64 = 64;
 inline bool is_pair(int bn) { return bn == kBnPair || bn == kBnPair128; }
 inline int tile_rows(int bn) { return is_pair(bn) ? 2 * kBM : kBM; }
 inline int tile_cols(int bn) { return bn == kBnPair ? 256 : (bn == kBnPair128 ? 128 : bn); }
@@ -198,6 +199,7 @@ cudaError_t tc_gemm_launch(const TcLaunch &l, int bn, int num_sms, cudaStream_t 
 cudaError_t tc_gemm_launch_fused(const TcLaunch &l, int bn, int total_tiles, int num_sms,
                                  cudaStream_t s, bool strips = false);
 // One launch of the product kernel in one tile configuration (each in its own translation unit).
+cudaError_t tc_launch_64(const TcLaunch &l, bool chain, int total_tiles, int num_sms, cudaStream_t s);
 cudaError_t tc_launch_128(const TcLaunch &l, bool chain, int total_tiles, int num_sms, cudaStream_t s);
 cudaError_t tc_launch_256(const TcLaunch &l, bool chain, int total_tiles, int num_sms, cudaStream_t s);
 cudaError_t tc_launch_pair(const TcLaunch &l, bool chain, bool strips, int total_tiles, int num_sms,
