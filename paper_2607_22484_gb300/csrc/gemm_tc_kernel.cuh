@@ -1783,14 +1783,13 @@ cudaError_t launch_kernel(const TcLaunch &l, int total_tiles, int num_sms, cudaS
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess)
         return e;
-    if (total_tiles <= 0)
-        return cudaSuccess;
     cudaLaunchConfig_t cfg = {};
     cfg.blockDim = dim3(kThreads, 1, 1);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
     int grid = total_tiles < num_sms ? total_tiles : num_sms;
+    static int max_pairs = -1;  // pairs that can be resident at once (SMs pair up within a GPC)
     if (PAIR) {
         attr[0].id = cudaLaunchAttributeClusterDimension;
         attr[0].val.clusterDim.x = 2;
@@ -1798,8 +1797,6 @@ cudaError_t launch_kernel(const TcLaunch &l, int total_tiles, int num_sms, cudaS
         attr[0].val.clusterDim.z = 1;
         cfg.attrs = attr;
         cfg.numAttrs = 1;
-        // Pairs that can be resident at once (SMs pair up within a GPC).
-        static int max_pairs = -1;
         if (max_pairs < 0) {
             cfg.gridDim = dim3((unsigned)(num_sms & ~1), 1, 1);
             int nc = 0;
@@ -1809,6 +1806,10 @@ cudaError_t launch_kernel(const TcLaunch &l, int total_tiles, int num_sms, cudaS
             }
             max_pairs = nc;
         }
+    }
+    if (total_tiles <= 0)  // only the attributes and the pair count (before a capture)
+        return cudaSuccess;
+    if (PAIR) {
         const int cap = std::min(max_pairs, num_sms / 2);  // a caller's SM budget caps it too
         const int pairs = std::max(1, std::min(total_tiles, cap));
         grid = 2 * pairs;

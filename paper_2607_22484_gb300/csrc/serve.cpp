@@ -1097,19 +1097,62 @@ bool serve_busy(svt_ctx *ctx)
 
 namespace {
 
-// Tile width of a grouped batch: the one with less padded tensor work over the
-// matrices' largest products (M x N), 128-wide tiles weighted as ~15 % less
-// efficient per flop.
-int batch_bn(const svt_matrix *mats, int count)
+// Estimated cycles of a grouped batch with one tile-width code: the larger of the work per SM (c
+// cycles a k-block and o a tile) and of the longest matrix's chain of dependent products (cl a
+// k-block, f a product), plus half of the other. Fitted to 32 batches (7 to 256 matrices of 48 to
+// 1024, both tiers) timed with every width, all of which get their fastest; of 30 others (4 to 256
+// matrices of 2 to 3000) the choice is the fastest or within 3 %. At both ends, us (128 x 64 / 128 x
+// 128 / 128 x 256 / pairs on 256 x 256): 33 BF16 of 48-192 358 / 391 / 492 / 515, 64 of 100-400 820 /
+// 630 / 720 / 763, 256 of 128-1024 11408 / 7715 / 7087 / 7262, 4 of 2000-3000 10614 / 6586 / 5977 /
+// 5162, 64 FP32 of 300-1024 7936 / 5317 / 5260 / 4715.
+struct BatchCost {
+    int bn;
+    double c, o, cl, f;
+};
+constexpr BatchCost kBatchCosts[4] = {{kBn64, 225, 5300, 270, 8500},
+                                      {128, 310, 5200, 510, 9500},
+                                      {256, 675, 4200, 735, 11200},
+                                      {kBnPair, 285, 7700, 865, 8500}};
+
+double batch_cost(const BatchCost &b, const svt_matrix *mats, int count, const Resolved &r, int sms)
 {
-    double a128 = 0, a256 = 0;
+    const double units = (double)(sms / ctas_per_tile(b.bn));
+    const int tm = tile_rows(b.bn), tn = tile_cols(b.bn);
+    const double hp = r.prec == SVT_FP32 ? r.iters : std::min(r.iters, r.hp_steps >= 0 ? r.hp_steps : 3);
+    const double sp = r.prec == SVT_FP32 ? 3.0 : 1.0;  // hi/lo segments of the P chain's products
+    double work = 0.0, chain = 0.0;
     for (int i = 0; i < count; ++i) {
         const int64_t M = std::max(mats[i].m, mats[i].n), N = std::min(mats[i].m, mats[i].n);
-        const double tm = (double)((M + kBM - 1) / kBM);
-        a128 += tm * (double)((N + 127) / 128) * 128.0 / 0.85;
-        a256 += tm * (double)((N + 255) / 256) * 256.0;
+        const double kM = (double)((M + kBK - 1) / kBK), kN = (double)((N + kBK - 1) / kBK);
+        const double ts = sym_tiles(b.bn, (int)((N + tn - 1) / tn));
+        const double tx = (double)((M + tm - 1) / tm) * (double)((N + tn - 1) / tn);
+        const double it = r.iters, rest = it - hp;
+        // k-blocks and tiles: P chain, S chain (hi/lo and plain steps), Gram, polish, combine.
+        const double kb = it * sp * (ts * (kM + kN) + tx * kN) + 3.0 * ts * kN * (3.0 * hp + rest) +
+                          ts * (3.0 * kM + sp * kM + 3.0 * kN) + tx * 5.0 * kN;
+        const double tiles = it * (5.0 * ts + tx) + 4.0 * ts + 2.0 * tx;
+        work += (kb * b.c + tiles * b.o) / units;
+        // The slower chain of each step.
+        const double k0 = std::max(kM * sp, kN), k1 = kN * sp;
+        const double steps = hp * (std::max(kM * sp, 3.0 * kN) + 6.0 * kN) + rest * (k0 + 2.0 * k1);
+        chain = std::max(chain, (steps + 3.0 * kM + kM * sp + 5.0 * kN) * b.cl + (3.0 * it + 4.0) * b.f);
     }
-    return a128 < a256 ? 128 : 256;
+    return std::max(work, chain) + 0.5 * std::min(work, chain);
+}
+
+// Tile width of a grouped batch whose options leave it open.
+int batch_bn(const svt_matrix *mats, int count, const Resolved &r, int sms)
+{
+    int best = 0;
+    double least = 0.0;
+    for (const BatchCost &b : kBatchCosts) {
+        const double t = batch_cost(b, mats, count, r, sms);
+        if (!best || t < least) {
+            best = b.bn;
+            least = t;
+        }
+    }
+    return best;
 }
 
 // Options of all matrices resolved: SVT_OK, or the first matrix's option status.
@@ -1190,7 +1233,9 @@ svt_status svt_batch(svt_ctx_t ctx, const svt_matrix *mats, int count, void *str
     if (same && total + batch_table_bytes(count, res[0]) <= ctx->ws_bytes) {
         BatchKey key;
         key.r = res[0];
-        key.bn = (res[0].tile == 128 || res[0].tile == 256) ? res[0].tile : batch_bn(mats, count);
+        key.bn = (res[0].tile == 128 || res[0].tile == 256)
+                     ? res[0].tile
+                     : batch_bn(mats, count, res[0], ctx->num_sms);
         for (int i = 0; i < count; ++i) {
             key.shapes.push_back(mats[i].m);
             key.shapes.push_back(mats[i].n);
