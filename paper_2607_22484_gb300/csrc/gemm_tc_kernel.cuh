@@ -1015,6 +1015,23 @@ __device__ __forceinline__ int geom_l(int g, int sg) { return (g >> (18 + sg)) &
 __device__ __forceinline__ int geom_r(int g, int sg) { return (g >> (21 + sg)) & 1; }
 __device__ __forceinline__ bool geom_fp8(int g) { return (g >> 24) & 1; }
 
+// k-blocks per pipeline slot (one pair of barriers). With 128 x 64 tiles a k-block's four MMAs take
+// 134 cycles, while the waits, the vote and the branches of one round of the producer's and of the
+// issuer's loop took some 350 and 400 cycles, whatever the tile: slots of two k-blocks halve that
+// (420 -> 311 cycles a k-block with the inlined waits of wait_warp; 1000 x 1001 709 -> 689 us). The
+// larger tiles have 269 cycles or more of MMAs a k-block, and lose more by waiting for the first two
+// k-blocks than they gain (2048 x 1024 FP32 on 256 x 128: 1218 us with one, 1245 with two).
+template <int BN, int STAGES>
+constexpr int kGroup = BN == 64 && STAGES % 2 == 0 ? 2 : 1;
+
+// k-blocks in the next slot when `left` remain: an odd one comes first, alone, so that the first
+// MMAs wait for less.
+template <int GROUP>
+__device__ __forceinline__ int slot_blocks(int left)
+{
+    return GROUP == 1 ? 1 : 2 - (left & 1);
+}
+
 template <int BN, int STAGES, bool CHAIN, bool PAIR, bool STRIPS>
 __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_constant__ TcLaunch L)
 {
@@ -1027,12 +1044,14 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
     constexpr int B_ROWS = PAIR ? BN / 2 : BN;  // rows of R this CTA stages per k-block
     constexpr int B_BYTES = B_ROWS * kBK * 2;
     constexpr int TILE_ROWS = PAIR ? 2 * kBM : kBM;
+    constexpr int GROUP = kGroup<BN, STAGES>, SLOTS = STAGES / GROUP;
+    static_assert(STAGES % GROUP == 0, "whole slots");
     uint8_t *sA = smem;
     uint8_t *sB = smem + STAGES * A_BYTES;
     uint8_t *stage_all = sB + STAGES * B_BYTES;  // 1024-aligned
     uint64_t *full = reinterpret_cast<uint64_t *>(stage_all + kEpiWarps * kStgBytes);
-    uint64_t *empty = full + STAGES;
-    uint64_t *tfull = empty + STAGES;
+    uint64_t *empty = full + SLOTS;
+    uint64_t *tfull = empty + SLOTS;
     uint64_t *tempty = tfull + 2;
     uint64_t *drain = tempty + 2;
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(drain + 1);
@@ -1058,7 +1077,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
     const bool leader = rank == 0;
 
     if (threadIdx.x == 0) {
-        for (int s = 0; s < STAGES; ++s) {
+        for (int s = 0; s < SLOTS; ++s) {
             mbar_init(&full[s], 1);
             mbar_init(&empty[s], 1);
         }
@@ -1289,12 +1308,12 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
             if (CHAIN) {
                 if (!wait_warp<PAIR>(&rfull[ri], rphase, abort_flag, status0, kWaitTimeoutNs))
                     break;
-                t = ring[ri].tile;
-                tc.prob = ring[ri].prob;
-                tc.tm = ring[ri].tm;
-                tc.tn = ring[ri].tn;
+                t = warp_uniform(ring[ri].tile);
+                tc.prob = warp_uniform(ring[ri].prob);
+                tc.tm = warp_uniform(ring[ri].tm);
+                tc.tn = warp_uniform(ring[ri].tn);
                 tc.valid = tc.prob >= 0;
-                geom = ring[ri].geom;
+                geom = warp_uniform(ring[ri].geom);
                 __syncwarp();
                 if (elect_one())
                     ring_release(ri);
@@ -1339,28 +1358,36 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
             for (int sg = 0; sg < geom_segs(geom) && ok; ++sg) {
                 const CUtensorMap *mL = &P.mapL[geom_l(geom, sg)];
                 const CUtensorMap *mR = &P.mapR[geom_r(geom, sg)];
-                for (int kb = 0; kb < kblocks; ++kb) {
+                for (int kb = 0, count; kb < kblocks; kb += count) {
                     if (!wait_warp<PAIR>(&empty[stage], phase ^ 1u, abort_flag, status0, kWaitTimeoutNs)) {
                         ok = false;
                         break;
                     }
-                    if (!elect_one()) {
-                        // the elected lane issues the copies
-                    } else if (PAIR) {
-                        // Both CTAs' bytes complete on the leader's barrier.
-                        const uint32_t fb = peer_addr(&full[stage], 0);
-                        if (leader)
-                            mbar_expect_tx(&full[stage], 2u * (uint32_t)(A_BYTES + B_BYTES));
-                        tma_load_2d_pair(sA + stage * A_BYTES, mL, kb << kshift, row0, fb);
-                        tma_load_2d_pair(sB + stage * B_BYTES, mR, kb << kshift, col0, fb);
-                    } else {
-                        mbar_expect_tx(&full[stage], (uint32_t)(A_BYTES + B_BYTES));
-                        tma_load_2d(sA + stage * A_BYTES, mL, kb << kshift, row0, &full[stage]);
-                        tma_load_2d(sB + stage * B_BYTES, mR, kb << kshift, col0, &full[stage]);
+                    count = slot_blocks<GROUP>(kblocks - kb);
+                    if (elect_one()) {
+                        // Both CTAs' bytes of a pair complete on the leader's barrier.
+                        const uint32_t fb = PAIR ? peer_addr(&full[stage], 0) : 0u;
+                        if (!PAIR || leader)
+                            mbar_expect_tx(&full[stage], (uint32_t)((PAIR ? 2 : 1) * (A_BYTES + B_BYTES) * count));
+#pragma unroll
+                        for (int j = 0; j < GROUP; ++j) {
+                            if (j >= count)
+                                break;
+                            const int x = (kb + j) << kshift;
+                            uint8_t *a = sA + (stage * GROUP + j) * A_BYTES;
+                            uint8_t *b = sB + (stage * GROUP + j) * B_BYTES;
+                            if (PAIR) {
+                                tma_load_2d_pair(a, mL, x, row0, fb);
+                                tma_load_2d_pair(b, mR, x, col0, fb);
+                            } else {
+                                tma_load_2d(a, mL, x, row0, &full[stage]);
+                                tma_load_2d(b, mR, x, col0, &full[stage]);
+                            }
+                        }
                     }
                     issued |= 1u << stage;
                     issued_parity = (issued_parity & ~(1u << stage)) | (phase << stage);
-                    if (++stage == STAGES) {
+                    if (++stage == SLOTS) {
                         stage = 0;
                         phase ^= 1u;
                     }
@@ -1369,7 +1396,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
         }
         // Drain: the last copy into every stage must have landed before exit. The
         // peer of a pair sees its copies land through the leader's MMA consuming them.
-        for (int s = 0; s < STAGES; ++s)
+        for (int s = 0; s < SLOTS; ++s)
             if ((issued >> s) & 1u) {
                 volatile int no_abort = 0;
                 if (!PAIR || leader)
@@ -1397,12 +1424,12 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
             if (CHAIN) {
                 if (!wait_warp<false>(&rfull[ri], rphase, abort_flag, status0, kWaitTimeoutNs))
                     break;
-                t = ring[ri].tile;
-                tc.prob = ring[ri].prob;
-                tc.tm = ring[ri].tm;
-                tc.tn = ring[ri].tn;
+                t = warp_uniform(ring[ri].tile);
+                tc.prob = warp_uniform(ring[ri].prob);
+                tc.tm = warp_uniform(ring[ri].tm);
+                tc.tn = warp_uniform(ring[ri].tn);
                 tc.valid = tc.prob >= 0;
-                geom = ring[ri].geom;
+                geom = warp_uniform(ring[ri].geom);
                 __syncwarp();
                 if (elect_one())
                     ring_release(ri);
@@ -1426,37 +1453,43 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
             tc_fence_after();
             const uint32_t d_tmem = tmem_base + (uint32_t)(buf * BN);
             // The tile's k-loop, one copy per operand kind chosen once per tile, so that
-            // the BF16 loop carries no test of the kind: for each segment and k-block,
-            // wait for the stage's copies, issue four MMAs over its 128 bytes of each row
-            // (K = 16 BF16 or 32 e4m3 elements each) and release the stage.
+            // the BF16 loop carries no test of the kind: for each segment and slot of
+            // GROUP k-blocks, wait for its copies, issue four MMAs over the 128 bytes of
+            // each k-block's rows (K = 16 BF16 or 32 e4m3 elements each) and release the slot.
             auto k_loop = [&](auto f8_tag) -> bool {
                 constexpr bool F8 = decltype(f8_tag)::value;
                 constexpr uint32_t id = F8 ? idesc_e4m3(TILE_ROWS, BN) : idesc_bf16(TILE_ROWS, BN);
                 const int kblocks = geom_kblocks(geom), segs = geom_segs(geom);
                 uint32_t acc = 0;
                 for (int sg = 0; sg < segs; ++sg) {
-                    for (int kb = 0; kb < kblocks; ++kb) {
+                    for (int left = kblocks, count; left > 0; left -= count) {
+                        count = slot_blocks<GROUP>(left);
                         if (!wait_warp<false>(&full[stage], phase, abort_flag, status0, kWaitTimeoutNs))
                             return false;
                         tc_fence_after();
                         if (elect_one()) {
-                            // Descriptor addresses count 16-byte units; a K step is 32 bytes.
-                            const uint64_t a0 = desc_a + (uint32_t)(stage * (A_BYTES >> 4));
-                            const uint64_t b0 = desc_b + (uint32_t)(stage * (B_BYTES >> 4));
 #pragma unroll
-                            for (int kk = 0; kk < kBK / 16; ++kk) {
-                                const uint64_t ad = a0 + 2 * kk, bd = b0 + 2 * kk;
-                                const uint32_t on = kk == 0 ? acc : 1u;
-                                if (F8) {
-                                    if (PAIR)
-                                        mma_e4m3_pair(d_tmem, ad, bd, id, on);
-                                    else
-                                        mma_e4m3(d_tmem, ad, bd, id, on);
-                                } else {
-                                    if (PAIR)
-                                        mma_bf16_pair(d_tmem, ad, bd, id, on);
-                                    else
-                                        mma_bf16(d_tmem, ad, bd, id, on);
+                            for (int j = 0; j < GROUP; ++j) {
+                                if (j >= count)
+                                    break;
+                                // Descriptor addresses count 16-byte units; a K step is 32 bytes.
+                                const uint64_t a0 = desc_a + (uint32_t)((stage * GROUP + j) * (A_BYTES >> 4));
+                                const uint64_t b0 = desc_b + (uint32_t)((stage * GROUP + j) * (B_BYTES >> 4));
+#pragma unroll
+                                for (int kk = 0; kk < kBK / 16; ++kk) {
+                                    const uint64_t ad = a0 + 2 * kk, bd = b0 + 2 * kk;
+                                    const uint32_t on = j + kk == 0 ? acc : 1u;
+                                    if (F8) {
+                                        if (PAIR)
+                                            mma_e4m3_pair(d_tmem, ad, bd, id, on);
+                                        else
+                                            mma_e4m3(d_tmem, ad, bd, id, on);
+                                    } else {
+                                        if (PAIR)
+                                            mma_bf16_pair(d_tmem, ad, bd, id, on);
+                                        else
+                                            mma_bf16(d_tmem, ad, bd, id, on);
+                                    }
                                 }
                             }
                             if (PAIR)
@@ -1466,7 +1499,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
                         }
                         __syncwarp();
                         acc = 1;
-                        if (++stage == STAGES) {
+                        if (++stage == SLOTS) {
                             stage = 0;
                             phase ^= 1u;
                         }
