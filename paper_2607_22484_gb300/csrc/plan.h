@@ -249,6 +249,10 @@ struct svt_ctx {
     std::vector<ProfRec> prof_pending;
     size_t prof_next = 0;
     std::map<svt::TuneKey, std::vector<int>> tuning;  // svt_autotune results
+    // Step coefficients and interval bounds by (schedule, iters, ell0, delta); see schedule_of.
+    std::map<std::tuple<int, int, double, double>,
+             std::pair<std::vector<double>, std::vector<double>>>
+        schedules;
     // Which grouped-batch plan's device tables are intact in the workspace (any
     // other use of the workspace resets it; the batch then re-uploads its tables).
     const void *table_owner = nullptr;

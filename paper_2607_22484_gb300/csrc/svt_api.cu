@@ -1292,6 +1292,28 @@ int fused_auto_width(int64_t m, int64_t n, const Resolved &r, int num_sms)
     return (M + 2 * N) * segs >= 24 * 3 * kBK ? kBnPair128 : 128;
 }
 
+// The steps' coefficients and interval bounds. The minimax designs of a schedule take some 350 us
+// of the host and depend on its options alone, so a context keeps them (at most 64) for the plans
+// of other shapes and workspace offsets: a new plan of the BF16 tier 440 -> 95 us.
+static bool schedule_of(svt_ctx *ctx, const Resolved &r, std::vector<double> *coef,
+                        std::vector<double> *lo)
+{
+    const auto key = std::make_tuple(r.schedule, r.iters, r.ell0, r.delta);
+    auto it = ctx->schedules.find(key);
+    if (it == ctx->schedules.end()) {
+        std::vector<double> c((size_t)std::max(1, 3 * r.iters), 0.0);
+        std::vector<double> l((size_t)std::max(1, r.iters), 0.0);
+        if (schedule_coeffs(r.schedule, r.iters, r.ell0, r.delta, c.data(), l.data()) != 0)
+            return false;
+        if (ctx->schedules.size() >= 64)
+            ctx->schedules.clear();
+        it = ctx->schedules.emplace(key, std::make_pair(std::move(c), std::move(l))).first;
+    }
+    *coef = it->second.first;
+    *lo = it->second.second;
+    return true;
+}
+
 svt_status get_plan(svt_ctx *ctx, int64_t m, int64_t n, const Resolved &r, size_t ws_base,
                     size_t ws_avail, Plan **out, int force_bn, std::shared_ptr<Plan> *keep)
 {
@@ -1326,10 +1348,7 @@ svt_status get_plan(svt_ctx *ctx, int64_t m, int64_t n, const Resolved &r, size_
     }
     if (plan->lay.total > ws_avail)
         return SVT_ERR_OOM;
-    plan->coef.assign((size_t)std::max(1, 3 * r.iters), 0.0);
-    plan->lo.assign((size_t)std::max(1, r.iters), 0.0);
-    if (schedule_coeffs(r.schedule, r.iters, r.ell0, r.delta, plan->coef.data(),
-                        plan->lo.data()) != 0)
+    if (!schedule_of(ctx, r, &plan->coef, &plan->lo))
         return SVT_ERR_INVALID;
     if (force_bn == kSmallPlan) {
         plan->small = true;
