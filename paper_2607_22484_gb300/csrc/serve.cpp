@@ -105,6 +105,7 @@ struct Request {
     svt_status result = SVT_OK;
     Plan *plan = nullptr;
     std::shared_ptr<Plan> plan_ref;  // keeps the plan alive while ops are in flight
+    std::vector<std::shared_ptr<Plan>> earlier;  // plans that earlier windows ran with
     size_t pc = 0;          // next op of the plan to issue
     bool grouped = false;   // ops limited to the kinds the grouped kernels cover
     bool large = false;     // large lane
@@ -233,6 +234,7 @@ struct ServeState {
     cudaEvent_t ring_ev[kRing] = {};  // slot k's window has been consumed
     bool ring_busy[kRing] = {};
     int ring_next = 0;
+    int win_bn = 0;  // tile-width code of the windows' products
     uint64_t windows = 0;
     FILE *metrics = nullptr;          // per-request JSON lines (svt_serve_metrics)
 };
@@ -313,6 +315,7 @@ void finish(ServeState *s, Request *r, svt_status st)
 {
     r->plan = nullptr;
     r->plan_ref.reset();
+    r->earlier.clear();
     r->result = st;
     r->state = 2;
     r->t_done = now_ms();
@@ -327,9 +330,110 @@ bool admissible(const svt_ctx *ctx, const Request *r, double now)
     return ctx->dbg_admit_delay_us <= 0 || now >= r->t_submit + 1e-3 * (double)ctx->dbg_admit_delay_us;
 }
 
+// Estimated cycles of matrices solved side by side with one tile-width code: the larger of the
+// work per SM (c cycles a k-block and o a tile) and of the longest matrix's chain of dependent
+// products (cl a k-block, f a product), plus half of the other. Fitted to 32 batches (7 to 256
+// matrices of 48 to 1024, both tiers) timed with every width, all of which get their fastest; of 30
+// others (4 to 256 matrices of 2 to 3000) the choice is the fastest or within 3 %. Some of them, us
+// (128 x 64 / 128 x 128 / 128 x 256 / pairs on 256 x 256): 33 BF16 of 48-192 358 / 391 / 492 / 515,
+// 64 of 100-400 820 / 630 / 720 / 763, 256 of 128-1024 11408 / 7715 / 7087 / 7262, 4 of 2000-3000
+// 10614 / 6586 / 5977 / 5162, 64 FP32 of 300-1024 7936 / 5317 / 5260 / 4715.
+struct BatchCost {
+    int bn;
+    double c, o, cl, f;
+};
+constexpr BatchCost kBatchCosts[4] = {{kBn64, 225, 5300, 270, 8500},
+                                      {128, 310, 5200, 510, 9500},
+                                      {256, 675, 4200, 735, 11200},
+                                      {kBnPair, 285, 7700, 865, 8500}};
+
+struct BatchLoad {
+    double work = 0.0, chain = 0.0;
+
+    void add(const BatchCost &b, int64_t m, int64_t n, const Resolved &r, int sms)
+    {
+        const double units = (double)(sms / ctas_per_tile(b.bn));
+        const int tm = tile_rows(b.bn), tn = tile_cols(b.bn);
+        const double hp = r.prec == SVT_FP32 ? r.iters : std::min(r.iters, r.hp_steps >= 0 ? r.hp_steps : 3);
+        const double sp = r.prec == SVT_FP32 ? 3.0 : 1.0;  // hi/lo segments of the P chain's products
+        const int64_t M = std::max(m, n), N = std::min(m, n);
+        const double kM = (double)((M + kBK - 1) / kBK), kN = (double)((N + kBK - 1) / kBK);
+        const double ts = sym_tiles(b.bn, (int)((N + tn - 1) / tn));
+        const double tx = (double)((M + tm - 1) / tm) * (double)((N + tn - 1) / tn);
+        const double it = r.iters, rest = it - hp;
+        // k-blocks and tiles: P chain, S chain (hi/lo and plain steps), Gram, polish, combine.
+        const double kb = it * sp * (ts * (kM + kN) + tx * kN) + 3.0 * ts * kN * (3.0 * hp + rest) +
+                          ts * (3.0 * kM + sp * kM + 3.0 * kN) + tx * 5.0 * kN;
+        const double tiles = it * (5.0 * ts + tx) + 4.0 * ts + 2.0 * tx;
+        work += (kb * b.c + tiles * b.o) / units;
+        // The slower chain of each step.
+        const double k0 = std::max(kM * sp, kN), k1 = kN * sp;
+        const double steps = hp * (std::max(kM * sp, 3.0 * kN) + 6.0 * kN) + rest * (k0 + 2.0 * k1);
+        chain = std::max(chain, (steps + 3.0 * kM + kM * sp + 5.0 * kN) * b.cl + (3.0 * it + 4.0) * b.f);
+    }
+
+    double cycles() const { return std::max(work, chain) + 0.5 * std::min(work, chain); }
+};
+
+// Chooses the windows' tile width for the active and queued small requests when one is admitted.
+// All of them run with one width, so that their products share a launch: a request that began
+// under another goes on with its plan of the new one (the same buffers and launches). A change
+// builds plans, about 95 us each, so it has to gain 15 %. Bursts of both tiers, 256-wide tiles
+// and plans with their own minimax designs against this, ms: 24 of 256-2048 7.65 / 6.60, 24 of 256-
+// 1024 4.86 / 3.53, 8 of 256-512 2.21 / 1.38, one of 512 0.74 / 0.54; a new context's first 24 of
+// 256-2048 16.0 / 9.7.
+void choose_window_bn(svt_ctx *ctx, ServeState *s, int sms)
+{
+    int best = 0;
+    double least = 0.0, now = -1.0;
+    bool running = false;
+    for (const BatchCost &b : kBatchCosts) {
+        BatchLoad l;
+        size_t n = 0;
+        for (const Request *r : s->active)
+            if (r->state == 1 && r->grouped) {
+                running = true;
+                l.add(b, r->m.m, r->m.n, r->opt, sms);
+                ++n;
+            }
+        for (const Request *r : s->queue) {
+            if (n >= (size_t)kSlots)
+                break;
+            if (r->opt.prec != SVT_FP64) {
+                l.add(b, r->m.m, r->m.n, r->opt, sms);
+                ++n;
+            }
+        }
+        if (b.bn == s->win_bn)
+            now = l.cycles();
+        if (!best || l.cycles() < least) {
+            best = b.bn;
+            least = l.cycles();
+        }
+    }
+    if (!running || now < 0.0 || now > 1.15 * least)
+        s->win_bn = best;
+}
+
+// Moves an active request to the windows' tile width.
+svt_status follow_window_bn(svt_ctx *ctx, ServeState *s, Request *r)
+{
+    Plan *plan = nullptr;
+    std::shared_ptr<Plan> ref;
+    std::lock_guard<std::mutex> g(ctx->mu);
+    const svt_status e = get_plan(ctx, r->m.m, r->m.n, r->opt, r->ws_off,
+                                  ctx->ws_bytes - kRingBytes - r->ws_off, &plan, s->win_bn, &ref);
+    if (e != SVT_OK)
+        return e;
+    r->earlier.push_back(std::move(r->plan_ref));
+    r->plan = plan;
+    r->plan_ref = std::move(ref);
+    return SVT_OK;
+}
+
 // One serving window: grouped ingest of newly admitted requests, one fused
-// product launch per tile width holding the next product stages of every active
-// request, grouped finalize of requests that reached their last op.
+// product launch holding the next product stages of every active request,
+// grouped finalize of requests that reached their last op.
 svt_status issue_window(svt_ctx *ctx, ServeState *s, int sms)
 {
     // Ring slot for this window's tables.
@@ -419,17 +523,17 @@ svt_status issue_window(svt_ctx *ctx, ServeState *s, int sms)
     // Product stages of every grouped request (including the ones just ingested), stage by
     // stage, each problem depending on the previous one of its request's chain in this window
     // (the combine on both chains; earlier windows precede on the stream).
-    std::vector<TcProblem> probs[2];
-    std::vector<int> starts[2], valid[2];
-    int tiles[2] = {0, 0};
+    std::vector<TcProblem> probs;
+    std::vector<int> starts, valid;
+    int tiles = 0;
     std::map<const Request *, std::array<int, 2>> lastp;
     const double work_cap = kWindowWork * sms / ctx->num_sms;
     double work = 0.0;
     // Bytes of everything but the problem tables, at most (aux and call records of the ingested
-    // and the finished, starts and counters of both widths).
+    // and the finished, starts and counters).
     const size_t other = (2 * kSlots) * (sizeof(AuxRec) + sizeof(CallRec)) + 16 * kAlign;
     auto table_bytes = [&](size_t extra) {
-        return (probs[0].size() + probs[1].size() + extra) * (sizeof(TcProblem) + 2 * sizeof(int)) + other;
+        return (probs.size() + extra) * (sizeof(TcProblem) + 2 * sizeof(int)) + other;
     };
     bool more = true;
     for (int stage = 0; more && (stage == 0 || work < work_cap); ++stage) {
@@ -449,7 +553,6 @@ svt_status issue_window(svt_ctx *ctx, ServeState *s, int sms)
             }
             more = true;
             work += P.tc_tensor_flops[op.idx];
-            const int g = (op.bn == 256) ? 1 : 0;
             size_t chain_at = 0;  // first entry of this launch in tc_chain
             for (int k = 0; k < op.idx; ++k)
                 chain_at += (size_t)P.tc[k].nprob;
@@ -472,20 +575,20 @@ svt_status issue_window(svt_ctx *ctx, ServeState *s, int sms)
                     }
                 tp.patch = 0;
                 const int chain = P.tc_chain[chain_at + (size_t)q];
-                const int pid = (int)probs[g].size();
+                const int pid = (int)probs.size();
                 tp.pid = pid;
                 for (int d = 0; d < 2; ++d) {
                     tp.dep[d] = chain < 2 ? (d == 0 ? last->second[chain] : -1) : last->second[d];
-                    tp.dep_target[d] = tp.dep[d] >= 0 ? kEpiWarpsPublic * valid[g][tp.dep[d]] : 0;
+                    tp.dep_target[d] = tp.dep[d] >= 0 ? kEpiWarpsPublic * valid[tp.dep[d]] : 0;
                 }
                 if (chain < 2)
                     last->second[chain] = pid;
                 else
                     last->second = {pid, pid};
-                starts[g].push_back(tiles[g]);
-                tiles[g] += tc_num_tiles(tp, op.bn);
-                valid[g].push_back(tc_valid_ctas(tp, op.bn));
-                probs[g].push_back(tp);
+                starts.push_back(tiles);
+                tiles += tc_num_tiles(tp, s->win_bn);
+                valid.push_back(tc_valid_ctas(tp, s->win_bn));
+                probs.push_back(tp);
             }
             r->pc += 1;
             if (P.ops[r->pc].kind == OP_FINAL)
@@ -502,24 +605,18 @@ svt_status issue_window(svt_ctx *ctx, ServeState *s, int sms)
     // Stage the tables.
     size_t o_aux = take(sizeof(AuxRec) * aux.size()), o_calls = take(sizeof(CallRec) * calls.size());
     size_t o_faux = take(sizeof(AuxRec) * faux.size()), o_fcalls = take(sizeof(CallRec) * fcalls.size());
-    size_t o_p[2], o_s[2], o_n[2];
-    for (int g = 0; g < 2; ++g) {
-        starts[g].push_back(tiles[g]);
-        o_p[g] = take(sizeof(TcProblem) * probs[g].size());
-        o_s[g] = take(sizeof(int) * starts[g].size());
-        o_n[g] = take(sizeof(int) * (probs[g].size() + 1));  // completion counters, tile counter
-    }
+    starts.push_back(tiles);
+    const size_t o_p = take(sizeof(TcProblem) * probs.size()), o_s = take(sizeof(int) * starts.size());
+    const size_t o_n = take(sizeof(int) * (probs.size() + 1));  // completion counters, tile counter
     if (used > kRingSlotBytes)
         return SVT_ERR_OOM;
     std::memcpy(h + o_aux, aux.data(), sizeof(AuxRec) * aux.size());
     std::memcpy(h + o_calls, calls.data(), sizeof(CallRec) * calls.size());
     std::memcpy(h + o_faux, faux.data(), sizeof(AuxRec) * faux.size());
     std::memcpy(h + o_fcalls, fcalls.data(), sizeof(CallRec) * fcalls.size());
-    for (int g = 0; g < 2; ++g) {
-        std::memcpy(h + o_p[g], probs[g].data(), sizeof(TcProblem) * probs[g].size());
-        std::memcpy(h + o_s[g], starts[g].data(), sizeof(int) * starts[g].size());
-        std::memset(h + o_n[g], 0, sizeof(int) * (probs[g].size() + 1));
-    }
+    std::memcpy(h + o_p, probs.data(), sizeof(TcProblem) * probs.size());
+    std::memcpy(h + o_s, starts.data(), sizeof(int) * starts.size());
+    std::memset(h + o_n, 0, sizeof(int) * (probs.size() + 1));
     cudaStream_t st = s->win;
     if (used && cudaMemcpyAsync(d, h, used, cudaMemcpyHostToDevice, st) != cudaSuccess)
         return SVT_ERR_CUDA;
@@ -534,18 +631,16 @@ svt_status issue_window(svt_ctx *ctx, ServeState *s, int sms)
             return SVT_ERR_CUDA;
         launched += 3;
     }
-    for (int g = 0; g < 2; ++g) {
-        if (probs[g].empty())
-            continue;
+    if (!probs.empty()) {
         TcLaunch L;
         std::memset(&L, 0, sizeof(L));
-        L.gtab = reinterpret_cast<const TcProblem *>(d + o_p[g]);
-        L.gstart = reinterpret_cast<const int *>(d + o_s[g]);
-        L.gcount = (int)probs[g].size();
+        L.gtab = reinterpret_cast<const TcProblem *>(d + o_p);
+        L.gstart = reinterpret_cast<const int *>(d + o_s);
+        L.gcount = (int)probs.size();
         L.dep_wait_ns = ctx->dbg_wait_ns;
-        L.done = reinterpret_cast<int *>(d + o_n[g]);
-        L.tile_counter = L.done + probs[g].size();
-        if (tc_gemm_launch_fused(L, g ? 256 : 128, tiles[g], sms, st) != cudaSuccess)
+        L.done = reinterpret_cast<int *>(d + o_n);
+        L.tile_counter = L.done + probs.size();
+        if (tc_gemm_launch_fused(L, s->win_bn, tiles, sms, st) != cudaSuccess)
             return SVT_ERR_CUDA;
         ++launched;
     }
@@ -726,12 +821,17 @@ bool tick(svt_ctx *ctx, ServeState *s)
             r->state = 3;
     }
     // Small lane: admit in arrival order while a slot and workspace are free.
+    const int small_sms = s->bigs.empty() ? ctx->num_sms : kSmallSms;
+    bool admitted = false;
     while (!hold_small && !s->queue.empty() && (int)s->active.size() < kSlots &&
            admissible(ctx, s->queue.front(), t_tick)) {
         Request *r = s->queue.front();
         size_t off;
         if (!s->arena.alloc(r->ws_len, &off))
             break;
+        if (!admitted)
+            choose_window_bn(ctx, s, small_sms);
+        admitted = true;
         s->queue.pop_front();
         int slot = 0;
         while (s->slot_used[slot])
@@ -747,7 +847,7 @@ bool tick(svt_ctx *ctx, ServeState *s)
             std::lock_guard<std::mutex> g(ctx->mu);
             evict_plans(ctx, 512);  // plans of active requests stay alive through plan_ref
             e = get_plan(ctx, r->m.m, r->m.n, r->opt, off, ctx->ws_bytes - kRingBytes - off, &plan,
-                         0, &r->plan_ref);
+                         r->opt.prec == SVT_FP64 ? 0 : s->win_bn, &r->plan_ref);
         }
         trace("admit", r->ticket, trace_file() ? (long long)((now_ms() - t0) * 1e3) : 0);
         if (e != SVT_OK) {
@@ -774,6 +874,19 @@ bool tick(svt_ctx *ctx, ServeState *s)
             progress = true;
         }
     // Issue one window if any request has ops left to issue.
+    for (auto it = s->active.begin(); admitted && it != s->active.end();) {
+        Request *r = *it;
+        svt_status e = SVT_OK;
+        if (r->state == 1 && r->grouped && r->plan->force_bn != s->win_bn)
+            e = follow_window_bn(ctx, s, r);
+        if (e != SVT_OK) {
+            cudaStreamSynchronize(s->win);
+            finish(s, r, e);
+            it = s->active.erase(it);
+        } else {
+            ++it;
+        }
+    }
     bool any = false;
     for (Request *r : s->active)
         if (r->state == 1)
@@ -781,7 +894,7 @@ bool tick(svt_ctx *ctx, ServeState *s)
     if (any) {
         const double t0 = trace_file() ? now_ms() : 0.0;
         NvtxRange nvtx("svt serve window");
-        svt_status e = issue_window(ctx, s, s->bigs.empty() ? ctx->num_sms : kSmallSms);
+        svt_status e = issue_window(ctx, s, small_sms);
         if (e == SVT_ERR_NOT_READY)
             return progress;
         trace("window", s->windows, trace_file() ? (long long)((now_ms() - t0) * 1e3) : 0);
@@ -1097,59 +1210,18 @@ bool serve_busy(svt_ctx *ctx)
 
 namespace {
 
-// Estimated cycles of a grouped batch with one tile-width code: the larger of the work per SM (c
-// cycles a k-block and o a tile) and of the longest matrix's chain of dependent products (cl a
-// k-block, f a product), plus half of the other. Fitted to 32 batches (7 to 256 matrices of 48 to
-// 1024, both tiers) timed with every width, all of which get their fastest; of 30 others (4 to 256
-// matrices of 2 to 3000) the choice is the fastest or within 3 %. At both ends, us (128 x 64 / 128 x
-// 128 / 128 x 256 / pairs on 256 x 256): 33 BF16 of 48-192 358 / 391 / 492 / 515, 64 of 100-400 820 /
-// 630 / 720 / 763, 256 of 128-1024 11408 / 7715 / 7087 / 7262, 4 of 2000-3000 10614 / 6586 / 5977 /
-// 5162, 64 FP32 of 300-1024 7936 / 5317 / 5260 / 4715.
-struct BatchCost {
-    int bn;
-    double c, o, cl, f;
-};
-constexpr BatchCost kBatchCosts[4] = {{kBn64, 225, 5300, 270, 8500},
-                                      {128, 310, 5200, 510, 9500},
-                                      {256, 675, 4200, 735, 11200},
-                                      {kBnPair, 285, 7700, 865, 8500}};
-
-double batch_cost(const BatchCost &b, const svt_matrix *mats, int count, const Resolved &r, int sms)
-{
-    const double units = (double)(sms / ctas_per_tile(b.bn));
-    const int tm = tile_rows(b.bn), tn = tile_cols(b.bn);
-    const double hp = r.prec == SVT_FP32 ? r.iters : std::min(r.iters, r.hp_steps >= 0 ? r.hp_steps : 3);
-    const double sp = r.prec == SVT_FP32 ? 3.0 : 1.0;  // hi/lo segments of the P chain's products
-    double work = 0.0, chain = 0.0;
-    for (int i = 0; i < count; ++i) {
-        const int64_t M = std::max(mats[i].m, mats[i].n), N = std::min(mats[i].m, mats[i].n);
-        const double kM = (double)((M + kBK - 1) / kBK), kN = (double)((N + kBK - 1) / kBK);
-        const double ts = sym_tiles(b.bn, (int)((N + tn - 1) / tn));
-        const double tx = (double)((M + tm - 1) / tm) * (double)((N + tn - 1) / tn);
-        const double it = r.iters, rest = it - hp;
-        // k-blocks and tiles: P chain, S chain (hi/lo and plain steps), Gram, polish, combine.
-        const double kb = it * sp * (ts * (kM + kN) + tx * kN) + 3.0 * ts * kN * (3.0 * hp + rest) +
-                          ts * (3.0 * kM + sp * kM + 3.0 * kN) + tx * 5.0 * kN;
-        const double tiles = it * (5.0 * ts + tx) + 4.0 * ts + 2.0 * tx;
-        work += (kb * b.c + tiles * b.o) / units;
-        // The slower chain of each step.
-        const double k0 = std::max(kM * sp, kN), k1 = kN * sp;
-        const double steps = hp * (std::max(kM * sp, 3.0 * kN) + 6.0 * kN) + rest * (k0 + 2.0 * k1);
-        chain = std::max(chain, (steps + 3.0 * kM + kM * sp + 5.0 * kN) * b.cl + (3.0 * it + 4.0) * b.f);
-    }
-    return std::max(work, chain) + 0.5 * std::min(work, chain);
-}
-
 // Tile width of a grouped batch whose options leave it open.
 int batch_bn(const svt_matrix *mats, int count, const Resolved &r, int sms)
 {
     int best = 0;
     double least = 0.0;
     for (const BatchCost &b : kBatchCosts) {
-        const double t = batch_cost(b, mats, count, r, sms);
-        if (!best || t < least) {
+        BatchLoad l;
+        for (int i = 0; i < count; ++i)
+            l.add(b, mats[i].m, mats[i].n, r, sms);
+        if (!best || l.cycles() < least) {
             best = b.bn;
-            least = t;
+            least = l.cycles();
         }
     }
     return best;
