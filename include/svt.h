@@ -125,7 +125,10 @@ typedef struct {
                                    CTA per 128 x 128 or 128 x 256 tile; 512 = a
                                    cluster of two CTAs per 256 x 256 tile
                                    (tcgen05 cta_group::2, each CTA staging half of
-                                   the tile's operands). A grouped batch takes 128
+                                   the tile's operands). The automatic choice also
+                                   has 128 x 64 and pair 256 x 128 tiles, and one
+                                   launch in shared memory for matrices of at most
+                                   128 x 128. A grouped batch takes 128
                                    or 256 from its matrices' options (0 or 512:
                                    chosen by a cost model, see svt_autotune_batch);
                                    serving chooses its own tiles. Other values:
@@ -542,7 +545,9 @@ svt_status svt_ctx_profile_read_ex(svt_ctx_t ctx, double *tc_ms, double *tc_flop
  * 128 x 256, and CTA pairs on 256 x 256), once as warm-up and `reps` times timed
  * with CUDA events on `stream`. Fused solves (opt->fuse = 1, the default) keep the
  * mode with the shortest whole solve; unfused solves keep the fastest mode per
- * product launch. The choice is stored in the context; later svt_polar /
+ * product launch. In a fused solve whose automatic choice is a finer tile than the
+ * three (128 x 64, or pairs on 256 x 128), that tile stands for 128 x 128, here and
+ * wherever a stored or imported 128 is used. The choice is stored in the context; later svt_polar /
  * svt_polar_ex calls with the same shape and options and tile = 0 use it. Y
  * receives A_tau. Synchronises `stream`.
  * Errors: as svt_polar_ex; SVT_ERR_BUSY while serving requests are in flight.
@@ -585,7 +590,8 @@ svt_status svt_autotune_schedule(svt_ctx_t ctx, const float *A, int64_t m, int64
  * svt_autotune_batch: times the grouped batch `mats` with 128- and 256-wide product
  * tiles (one untimed call each, then `reps` timed svt_batch calls on `stream`) and
  * returns the faster width in *tile_out (and its mean time per batch in *ms_out,
- * nullable). Set svt_options.tile of the batch's matrices to it. The outputs of
+ * nullable). Set svt_options.tile of the batch's matrices to it; with tile = 0 a cost
+ * model also considers 128 x 64 tiles and pairs on 256 x 256. The outputs of
  * `mats` are written by every call. Synchronous. Errors: as svt_batch;
  * SVT_ERR_INVALID for count <= 0, reps < 1 or a null tile_out.
  */

@@ -19,9 +19,9 @@
 //   * admits queued requests in arrival order while a slot is free and their
 //     workspace fits in a free range of the context's workspace (first fit),
 //   * issues one window on its stream: grouped ingest of the newly admitted,
-//     ONE fused product launch per tile width that carries the next stages of
-//     every active request (both polar chains of each), about a millisecond of
-//     work, and grouped finalize of requests that reach their last op.
+//     ONE fused product launch that carries the next stages of every active
+//     request (both polar chains of each), about a millisecond of work, and
+//     grouped finalize of requests that reach their last op.
 // A request therefore joins the very next window after memory frees up, and
 // its stages share launches with whatever else is running.
 #include <cuda_runtime.h>
