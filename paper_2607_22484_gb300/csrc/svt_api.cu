@@ -1265,15 +1265,19 @@ void evict_plans(svt_ctx *ctx, size_t max_entries)
 
 // Tile mode of a fused solve when none is requested or tuned, from whole-solve timings on
 // GB300 (20 steps, us; 128 x 64 tiles / 128 x 128 / pairs on 256 x 128 / pairs on 256 x 256):
-//   BF16  300^2 363 / 431 / 463 / 557, 512^2 431 / 505 / 529 / 692, 1000^2 609 / 686 / 708 / 986,
-//         1100^2 734 / 728 / 733, 1536^2 1231 / 944 / 948 / 1164, 1792^2 - / 1189 / 1174 / 1296,
-//         2048^2 - / 1452 / 1405 / 1435, 2304^2 - / 2146 / 2036 / 1800, 4096 x 256 601 / 660 / 647,
-//         8192 x 512 1198 / 1176 / 1123 / 1391, 8192 x 2048 - / 3146 / 2984 / 2812
-//   FP32  300^2 519 / 626 / 651 / 840, 1000^2 1060 / 1131 / 1076 / 1493, 1100^2 1370 / 1229 /
-//         1159, 1700^2 - / 2390 / 2226 / 2295, 2400 x 600 1259 / 1310 / 1183 / 1677, 8192 x 512
-//         2652 / 2604 / 2304 / 3135, 2048^2 - / 3248 / 3097 / 2829
-// While the tiles of X Z fit the SMs at once a solve is bound by the latency of one tile after
-// another, and 128 x 64 tiles have the shortest: half the MMAs and one epilogue block a warp.
+//   BF16  300^2 366 / 435 / 467 / 557, 512^2 415 / 503 / 531 / 692, 1000^2 568 / 673 / 694 / 986,
+//         1100^2 652 / 713 / 715, 1280^2 723 / 771 / 768, 1536^2 1050 / 906 / 924 / 1164, 1792^2 - /
+//         1189 / 1174 / 1296, 2048^2 - / 1452 / 1405 / 1435, 2304^2 - / 2146 / 2036 / 1800, 4096 x 256
+//         522 / 632 / 623, 2048 x 1024 690 / 752 / 753, 8192 x 512 973 / 1090 / 1036 / 1391, 8192 x
+//         2048 - / 3146 / 2984 / 2812
+//   FP32  300^2 509 / 615 / 630 / 840, 1000^2 924 / 1083 / 1032, 1100^2 1122 / 1153 / 1082, 1280^2
+//         1354 / 1306 / 1219, 1700^2 2879 / 2223 / 2101 / 2295, 2400 x 600 1071 / 1237 / 1102 / 1677,
+//         2048 x 1024 1245 / 1298 / 1210, 8192 x 512 2059 / 2366 / 2066 / 3135, 2048^2 - / 3248 /
+//         3097 / 2829
+// While a step's tiles (five symmetric products and X Z) are few per SM, a solve is bound by the
+// latency of one tile after another, and 128 x 64 tiles have the shortest: half the MMAs and one
+// epilogue block a warp. Their line is 5 tiles an SM, 4 in the FP32 tier, whose three segments make
+// operand bytes count sooner. Rank-r mode, one chain: X Z's tiles fit the SMs at once.
 // Past that the operand bytes decide. 256 x 256 tiles move the fewest but leave SMs without a
 // tile until the smaller side is about 1800. Below, pairs on 256 x 128 move 24 KiB per k-block and
 // CTA where 128 x 128 tiles move 32, and cost about 300 cycles a tile more (the pair's barriers):
@@ -1282,7 +1286,11 @@ void evict_plans(svt_ctx *ctx, size_t max_entries)
 int fused_auto_width(int64_t m, int64_t n, const Resolved &r, int num_sms)
 {
     const int64_t M = std::max(m, n), N = std::min(m, n);
-    if ((M + 127) / 128 * ((N + 63) / 64) <= num_sms)
+    const int64_t tx = (M + 127) / 128 * ((N + 63) / 64);
+    if (N <= 2048 && (r.mode == SVT_MODE_RANK_R
+                          ? tx <= num_sms
+                          : 5 * sym_tiles(kBn64, (int)((N + 63) / 64)) + tx <=
+                                (r.prec == SVT_FP32 ? 4 : 5) * (int64_t)num_sms))
         return kBn64;
     // Rank-r mode has half the tiles (one chain), so finer ones pay up to 2048 (2048 x 8192: 1221
     // against 1555 us; 2304^2: 1714 against 1465).

@@ -1,6 +1,6 @@
-"""Solves on 128 x 64 tiles: the automatic choice while ceil(M/128) ceil(N/64) tiles fit the SMs at
-once (152). Shapes at both sides of that line and of multiples of 64 and 128, tall and wide, with each
-option that changes the products; against 128 x 128 tiles and the oracle.
+"""Solves on 128 x 64 tiles: the automatic choice while a step's tiles are few per SM. Shapes at both
+sides of that line (of each tier and of rank-r mode) and of multiples of 64 and 128, tall and wide, with
+each option that changes the products; against 128 x 128 tiles and the oracle.
 
 Tolerances: the tiers' (2e-2, 1e-4) against Eq. 1; 1e-5 between execution paths of one solve."""
 import numpy as np
@@ -18,7 +18,8 @@ BOUND = {"bf16": 2e-2, "fp32": 1e-4}
 
 @pytest.mark.parametrize("prec", ["bf16", "fp32"])
 @pytest.mark.parametrize("m,n", [(129, 1), (129, 65), (190, 64), (1000, 63), (257, 256), (384, 705),
-                                 (960, 1216), (961, 1216), (2432, 512), (2433, 512)])
+                                 (960, 1216), (961, 1216), (2432, 512), (2433, 512),
+                                 (1152, 1088), (1300, 1290), (520, 8100), (9000, 500)])
 def test_tiles_128x64(m, n, prec):
     k = min(m, n)
     hi = max(1, k // 4)
