@@ -8,8 +8,11 @@
 // which its tiles may read and write:
 //
 // * chain mode (strips = false): every product waits for the whole previous
-//   product of its chain (P or S; the combine for both). The chains only read what
-//   their own earlier products or the ingest wrote, so this orders every access.
+//   product of its chain (P or S; the combine for both), and for the other chain's
+//   latest product that used a buffer it writes, or wrote one it uses, unless its
+//   chain has waited for that one before. The shifted Gram needs it: it opens the S
+//   chain and reads X0^T, which the P chain's second X Z overwrites, and over a long
+//   K its three segments take longer than the short products up to that write.
 // * strip mode (strips = true, square tiles): from the buffers each product reads
 //   and writes. A read of a buffer written earlier in the launch waits for the
 //   strip it reads: rows of L for the tile's row, rows of R for its column, the C
@@ -20,6 +23,7 @@
 //   its scales are computed from.
 #pragma once
 
+#include <algorithm>
 #include <map>
 #include <vector>
 
@@ -49,7 +53,7 @@ struct DepResult {
 
 // per_cta: completion increments per CTA tile (epilogue warps); per_tile: per
 // scheduled tile (per_cta x CTAs per tile); strip_capacity: strip counters
-// available. Returns false when the conditions do not fit the table's slots.
+// available (strip mode). Returns false when the conditions do not fit the table's slots.
 inline bool derive_fused_deps(const std::vector<DepProduct> &ps, bool strips, int per_cta,
                               int per_tile, int strip_capacity, std::vector<DepResult> &out)
 {
@@ -60,25 +64,57 @@ inline bool derive_fused_deps(const std::vector<DepProduct> &ps, bool strips, in
     std::map<const void *, Writer> writers;
     std::map<const void *, std::vector<int>> readers;
     std::map<const double *, int> norm_writer;
-    int lastp[2] = {-1, -1};
+    // chain mode: each chain's latest product, the latest of the other chain that it comes
+    // after, and the latest product of each chain that read and that wrote a buffer
+    int lastp[2] = {-1, -1}, seen[2] = {-1, -1};
+    struct Use {
+        const void *buf;
+        int rd[2], wr[2];
+    };
+    std::vector<Use> uses;
+    auto use_of = [&uses](const void *b) -> Use & {
+        for (Use &u : uses)
+            if (u.buf == b)
+                return u;
+        uses.push_back({b, {-1, -1}, {-1, -1}});
+        return uses.back();
+    };
     int strip_next = 0;
     for (int pid = 0; pid < (int)ps.size(); ++pid) {
         const DepProduct &p = ps[pid];
         DepResult &d = out[pid];
         if (!strips) {
+            const void *reads[3] = {p.l, p.r, p.c}, *writes[3] = {p.o, p.t, p.f};
             if (p.chain < 2) {
+                const int other = 1 - p.chain;
+                int need = -1;
+                for (const void *b : reads)
+                    if (b)
+                        need = std::max(need, use_of(b).wr[other]);
+                for (const void *b : writes)
+                    if (b)
+                        need = std::max({need, use_of(b).rd[other], use_of(b).wr[other]});
                 d.dep[0] = lastp[p.chain];
+                if (need > seen[p.chain])
+                    d.dep[1] = seen[p.chain] = need;
+                lastp[p.chain] = pid;
             } else {
                 d.dep[0] = lastp[0];
                 d.dep[1] = lastp[1];
+                lastp[0] = lastp[1] = seen[0] = seen[1] = pid;
             }
             for (int k = 0; k < 2; ++k)
                 if (d.dep[k] >= 0)
                     d.dep_target[k] = per_cta * ps[d.dep[k]].valid;
-            if (p.chain < 2)
-                lastp[p.chain] = pid;
-            else
-                lastp[0] = lastp[1] = pid;
+            for (int c = 0; c < 2; ++c)
+                if (p.chain == c || p.chain == 2) {
+                    for (const void *b : reads)
+                        if (b)
+                            use_of(b).rd[c] = pid;
+                    for (const void *b : writes)
+                        if (b)
+                            use_of(b).wr[c] = pid;
+                }
             continue;
         }
         d.strip_base = strip_next;

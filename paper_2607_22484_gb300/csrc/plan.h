@@ -16,6 +16,7 @@
 
 #include <nvtx3/nvToolsExt.h>
 
+#include "fused_deps.h"
 #include "small_solve.h"
 #include "svt_internal.h"
 
@@ -156,6 +157,29 @@ struct Plan {
     bool small = false;
     SmallSolve small_args;          // all but the call's pointers, strides and tau
 };
+
+// Entry `at` of the plan's problems (in tc order) as the dependency derivation sees it, with the
+// tiles of tile-width code bn.
+inline DepProduct dep_product(const Plan &P, size_t at, const TcProblem &tp, int bn)
+{
+    const Plan::ProbIO &io = P.tc_io[at];
+    return {io.l, io.r, io.c, io.o, io.t, io.o_trans, tp.sym, P.tc_chain[at], tp.tiles_m, tp.tiles_n,
+            tc_valid_ctas(tp, bn), io.theta_src, io.norm_acc, io.f};
+}
+
+// Chain-mode dependencies of a launch that holds products of several solves: ps and pid are one
+// solve's products in program order and their places in `probs`. Fills those entries' dep fields.
+inline void set_chain_deps(std::vector<TcProblem> &probs, const std::vector<DepProduct> &ps,
+                           const std::vector<int> &pid)
+{
+    std::vector<DepResult> deps;
+    derive_fused_deps(ps, false, kEpiWarpsPublic, 0, 0, deps);  // (chain mode refuses nothing)
+    for (size_t k = 0; k < ps.size(); ++k)
+        for (int d = 0; d < 2; ++d) {
+            probs[pid[k]].dep[d] = deps[k].dep[d] >= 0 ? pid[deps[k].dep[d]] : -1;
+            probs[pid[k]].dep_target[d] = deps[k].dep_target[d];
+        }
+}
 
 // force_bn code of the plans that run as one small_solve launch.
 constexpr int kSmallPlan = 1;

@@ -27,7 +27,6 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
-#include <array>
 #include <chrono>
 #include <condition_variable>
 #include <cstdio>
@@ -521,12 +520,16 @@ svt_status issue_window(svt_ctx *ctx, ServeState *s, int sms)
         r->pc += 3;
     }
     // Product stages of every grouped request (including the ones just ingested), stage by
-    // stage, each problem depending on the previous one of its request's chain in this window
-    // (the combine on both chains; earlier windows precede on the stream).
+    // stage, with the dependencies between a request's products of this window (earlier windows
+    // precede on the stream).
     std::vector<TcProblem> probs;
-    std::vector<int> starts, valid;
+    std::vector<int> starts;
     int tiles = 0;
-    std::map<const Request *, std::array<int, 2>> lastp;
+    struct Part {  // a request's products in this window
+        std::vector<DepProduct> ps;
+        std::vector<int> pid;
+    };
+    std::map<const Request *, Part> parts;
     const double work_cap = kWindowWork * sms / ctx->num_sms;
     double work = 0.0;
     // Bytes of everything but the problem tables, at most (aux and call records of the ingested
@@ -556,7 +559,7 @@ svt_status issue_window(svt_ctx *ctx, ServeState *s, int sms)
             size_t chain_at = 0;  // first entry of this launch in tc_chain
             for (int k = 0; k < op.idx; ++k)
                 chain_at += (size_t)P.tc[k].nprob;
-            auto last = lastp.emplace(r, std::array<int, 2>{-1, -1}).first;
+            Part &part = parts[r];
             for (int q = 0; q < l.nprob; ++q) {
                 TcProblem tp = l.p[q];
                 for (const PatchRec &pr : P.patches)
@@ -574,20 +577,11 @@ svt_status issue_window(svt_ctx *ctx, ServeState *s, int sms)
                             tp.ep.falpha = -r->m.tau;
                     }
                 tp.patch = 0;
-                const int chain = P.tc_chain[chain_at + (size_t)q];
-                const int pid = (int)probs.size();
-                tp.pid = pid;
-                for (int d = 0; d < 2; ++d) {
-                    tp.dep[d] = chain < 2 ? (d == 0 ? last->second[chain] : -1) : last->second[d];
-                    tp.dep_target[d] = tp.dep[d] >= 0 ? kEpiWarpsPublic * valid[tp.dep[d]] : 0;
-                }
-                if (chain < 2)
-                    last->second[chain] = pid;
-                else
-                    last->second = {pid, pid};
+                tp.pid = (int)probs.size();
+                part.ps.push_back(dep_product(P, chain_at + (size_t)q, tp, s->win_bn));
+                part.pid.push_back(tp.pid);
                 starts.push_back(tiles);
                 tiles += tc_num_tiles(tp, s->win_bn);
-                valid.push_back(tc_valid_ctas(tp, s->win_bn));
                 probs.push_back(tp);
             }
             r->pc += 1;
@@ -595,6 +589,8 @@ svt_status issue_window(svt_ctx *ctx, ServeState *s, int sms)
                 fin.push_back(r);
         }
     }
+    for (const auto &p : parts)
+        set_chain_deps(probs, p.second.ps, p.second.pid);
     // Finalize records.
     std::vector<AuxRec> faux;
     std::vector<CallRec> fcalls;
@@ -1018,11 +1014,12 @@ svt_status build_batch(svt_ctx *ctx, ServeState *s, const svt_matrix *mats, int 
                                            reinterpret_cast<uint8_t *>(aux.data()),
                                            reinterpret_cast<uint8_t *>(aux.data() + count)));
     // One persistent launch for every product of every matrix: stage-major order
-    // (stage k of all matrices, then stage k + 1), each problem depending on the
-    // previous problem of its matrix's chain (the combine on both chains).
+    // (stage k of all matrices, then stage k + 1), with the dependencies between each
+    // matrix's own products.
     std::vector<TcProblem> probs;
-    std::vector<int> starts, valid;
-    std::vector<std::array<int, 2>> lastp(count, std::array<int, 2>{-1, -1});
+    std::vector<int> starts;
+    std::vector<std::vector<DepProduct>> ps(count);
+    std::vector<std::vector<int>> pids(count);
     std::vector<std::vector<int>> chain_base(count);
     for (int i = 0; i < count; ++i) {
         const Plan &P = *plans[i];
@@ -1042,7 +1039,6 @@ svt_status build_batch(svt_ctx *ctx, ServeState *s, const svt_matrix *mats, int 
             const TcLaunch &l = P.tc[li];
             for (int q = 0; q < l.nprob; ++q) {
                 TcProblem tp = l.p[q];
-                const int chain = P.tc_chain[chain_base[i][li] + q];
                 tp.patch = 0;
                 for (const PatchRec &pr : P.patches)
                     if (pr.kind == OP_TC && pr.launch == li && pr.prob == q)
@@ -1051,28 +1047,16 @@ svt_status build_batch(svt_ctx *ctx, ServeState *s, const svt_matrix *mats, int 
                 if (tp.patch & PT_O_IS_Y)
                     tp.o_tma = 0;  // per-call output: plain stores
                 tp.pid = (int)probs.size();
-                tp.dep[0] = tp.dep[1] = -1;
-                tp.dep_target[0] = tp.dep_target[1] = 0;
-                if (chain < 2) {
-                    tp.dep[0] = lastp[i][chain];
-                } else {
-                    tp.dep[0] = lastp[i][0];
-                    tp.dep[1] = lastp[i][1];
-                }
-                for (int d = 0; d < 2; ++d)
-                    if (tp.dep[d] >= 0)
-                        tp.dep_target[d] = kEpiWarpsPublic * valid[tp.dep[d]];
+                ps[i].push_back(dep_product(P, (size_t)(chain_base[i][li] + q), tp, bn));
+                pids[i].push_back(tp.pid);
                 starts.push_back(total);
                 total += tc_num_tiles(tp, bn);
-                valid.push_back(tc_valid_ctas(tp, bn));
-                if (chain < 2)
-                    lastp[i][chain] = tp.pid;
-                else
-                    lastp[i][0] = lastp[i][1] = tp.pid;
                 probs.push_back(tp);
             }
         }
     }
+    for (int i = 0; i < count; ++i)
+        set_chain_deps(probs, ps[i], pids[i]);
     starts.push_back(total);
     TcProblem *dp = reinterpret_cast<TcProblem *>(tbase + take(sizeof(TcProblem) * probs.size()));
     int *ds = reinterpret_cast<int *>(tbase + take(sizeof(int) * starts.size()));

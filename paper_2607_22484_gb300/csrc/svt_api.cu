@@ -1123,8 +1123,8 @@ svt_status run_plan_segment(svt_ctx *ctx, Plan &P, const CallArgs &a, cudaStream
 
 namespace {
 
-// One persistent launch for all products of the plan: problems in program order,
-// each depending on the previous problem of its chain (the combine on both chains).
+// One persistent launch for all products of the plan: problems in program order, with the
+// conditions that fused_deps.h derives.
 // Eligible when the products are contiguous in the op list and share one tile width.
 svt_status build_fused(svt_ctx *ctx, Plan &P)
 {
@@ -1165,8 +1165,6 @@ svt_status build_fused(svt_ctx *ctx, Plan &P)
         const TcLaunch &l = P.tc[li];
         for (int q = 0; q < l.nprob; ++q) {
             TcProblem tp = l.p[q];
-            const Plan::ProbIO io = P.tc_io[ci];
-            const int chain = P.tc_chain[ci++];
             tp.pid = (int)probs.size();
             tp.patch = 0;
             tp.call_idx = 0;
@@ -1175,8 +1173,7 @@ svt_status build_fused(svt_ctx *ctx, Plan &P)
                     tp.patch |= pr.flags;
             if (tp.patch & PT_O_IS_Y)
                 tp.o_tma = 0;  // the caller's output: plain coalesced stores
-            dps.push_back({io.l, io.r, io.c, io.o, io.t, io.o_trans, tp.sym, chain, tp.tiles_m,
-                           tp.tiles_n, tc_valid_ctas(tp, bn), io.theta_src, io.norm_acc, io.f});
+            dps.push_back(dep_product(P, ci++, tp, bn));
             starts.push_back(total);
             total += tc_num_tiles(tp, bn);
             const int kb = tp.fp8 ? 2 * kBK : kBK;
