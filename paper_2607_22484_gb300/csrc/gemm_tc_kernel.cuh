@@ -1348,6 +1348,9 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
                                 ok = wait_counter(&L.done[P.dep[d]], P.dep_target[d], abort_flag,
                                                   status0, dep_limit(L));
                     ok = __shfl_sync(0xffffffffu, (int)ok, 0);
+                    // Lane 0's acquire comes before the copies of whichever lane is elected: a
+                    // shuffle does not order memory.
+                    __syncwarp();
                 }
                 if (!ok)
                     break;
