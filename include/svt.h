@@ -490,7 +490,8 @@ typedef enum {
     SVT_DEBUG_ADMIT_DELAY_US = 2,
     /* value in nanoseconds: the product kernel's waits on other tiles' results (its
      * device-side dependency counters) give up after this long instead of 2 s and
-     * report SVT_ERR_TIMEOUT in the solve's status; 1 makes any wait that is not
+     * report SVT_ERR_TIMEOUT in the solve's status (in a launch that several solves
+     * share, of every one that it left unfinished); 1 makes any wait that is not
      * already satisfied time out at once. 0 restores the default. Applies to launches
      * issued (or captured into a batch's graph) after the call. */
     SVT_DEBUG_WAIT_LIMIT_NS = 3

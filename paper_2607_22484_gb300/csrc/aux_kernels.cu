@@ -422,6 +422,13 @@ __global__ void grouped_finalize_kernel(const AuxRec *recs, const CallRec *calls
     if (i >= count)
         return;
     const AuxRec &r = recs[i];
+    // A wait of the product launch gave up and left products of this solve unfinished (a product
+    // completes after all that it waits for, so the last of each chain speaks for the chain).
+    for (int d = 0; d < 2; ++d)
+        if (r.done[d] && *r.done[d] < r.done_target[d])
+            atomicCAS(r.status, 0, (int)SVT_ERR_TIMEOUT);
+    if (!r.last)
+        return;
     if (!isfinite(r.scal[SC_NRM_OUT]))
         atomicCAS(r.status, 0, (int)SVT_ERR_DIVERGED);
     if (calls[i].d_status)

@@ -31,9 +31,10 @@
 // to both CTAs, whose epilogues each drain their own 128 x 256 accumulator.
 //
 // Every wait on an mbarrier is bounded (kWaitTimeoutNs of global time); on
-// expiry the kernel records SVT_ERR_TIMEOUT in the problem's status word, the
-// other roles stop at their next wait, in-flight copies and MMAs are drained
-// (again with a bound) and tensor memory is released before the kernel returns.
+// expiry the kernel records SVT_ERR_TIMEOUT in the solve's status word (launches that
+// several solves share leave that to their finalize kernel, which finds the solves with
+// unfinished products), the other roles stop at their next wait, in-flight copies and MMAs
+// are drained (again with a bound) and tensor memory is released before the kernel returns.
 #pragma once
 
 #include <algorithm>
@@ -1071,7 +1072,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
 
     const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
-    int *status0 = prob_at(L, 0).ep.status;
+    int *status0 = L.shared ? nullptr : prob_at(L, 0).ep.status;  // of the solve (shared: of none)
     // CTA pairs: rank 0 (leader) issues the MMAs and hands out tile ids.
     const uint32_t rank = PAIR ? cluster_rank() : 0u;
     const bool leader = rank == 0;

@@ -20,13 +20,15 @@
 //     workspace fits in a free range of the context's workspace (first fit),
 //   * issues one window on its stream: grouped ingest of the newly admitted,
 //     ONE fused product launch that carries the next stages of every active
-//     request (both polar chains of each), about a millisecond of work, and
-//     grouped finalize of requests that reach their last op.
+//     request (both polar chains of each), about a millisecond of work, and a
+//     grouped finalize: requests whose products a time-out left unfinished are
+//     marked, those that reach their last op report their status.
 // A request therefore joins the very next window after memory frees up, and
 // its stages share launches with whatever else is running.
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <array>
 #include <chrono>
 #include <condition_variable>
 #include <cstdio>
@@ -172,6 +174,7 @@ struct BatchKey {
     std::vector<int64_t> shapes;     // m0, n0, m1, n1, ...
     Resolved r;
     int bn = 0;                      // product tile width of the grouped launch
+    uint64_t wait_ns = 0;            // its limit of dependency waits (recorded with it)
     bool operator<(const BatchKey &o) const
     {
         auto tie_r = [](const Resolved &x) {
@@ -180,8 +183,8 @@ struct BatchKey {
         };
         if (shapes != o.shapes)
             return shapes < o.shapes;
-        if (bn != o.bn)
-            return bn < o.bn;
+        if (bn != o.bn || wait_ns != o.wait_ns)
+            return std::tie(bn, wait_ns) < std::tie(o.bn, o.wait_ns);
         return tie_r(r) < tie_r(o.r);
     }
 };
@@ -189,8 +192,8 @@ struct BatchKey {
 // Upper bound on the device table bytes of a grouped batch.
 size_t batch_table_bytes(int count, const Resolved &r)
 {
-    const size_t n_tc = 1 + 3 * (size_t)std::max(0, r.iters) + 2 + 1;
-    const size_t nprob = n_tc * 2 * (size_t)count;
+    // Gram and combine: one product each; 3 launches a step and 2 of the polish: two each
+    const size_t nprob = (2 + 2 * (3 * (size_t)std::max(0, r.iters) + 2)) * (size_t)count;
     return align_up(sizeof(AuxRec) * count, kAlign) + align_up(sizeof(CallRec) * count, kAlign) +
            align_up(sizeof(TcProblem) * nprob, kAlign) + 2 * align_up(sizeof(int) * (nprob + 1), kAlign);
 }
@@ -432,7 +435,7 @@ svt_status follow_window_bn(svt_ctx *ctx, ServeState *s, Request *r)
 
 // One serving window: grouped ingest of newly admitted requests, one fused
 // product launch holding the next product stages of every active request,
-// grouped finalize of requests that reached their last op.
+// and a grouped finalize of all of them (see grouped_finalize_kernel).
 svt_status issue_window(svt_ctx *ctx, ServeState *s, int sms)
 {
     // Ring slot for this window's tables.
@@ -591,12 +594,24 @@ svt_status issue_window(svt_ctx *ctx, ServeState *s, int sms)
     }
     for (const auto &p : parts)
         set_chain_deps(probs, p.second.ps, p.second.pid);
-    // Finalize records.
+    // Finalize records: one for each request with products in this window. Its chains' last
+    // products here, entries of `probs`, become counters once the table's place is known.
     std::vector<AuxRec> faux;
     std::vector<CallRec> fcalls;
-    for (Request *r : fin) {
-        faux.push_back(aux_of(r, 0, 0));
-        fcalls.push_back(call_of(r));
+    std::vector<std::array<int, 2>> flast;
+    for (const auto &p : parts) {
+        AuxRec a = aux_of(p.first, 0, 0);
+        a.last = std::find(fin.begin(), fin.end(), p.first) != fin.end() ? 1 : 0;
+        std::array<int, 2> at = {-1, -1};
+        for (size_t i = 0; i < p.second.ps.size(); ++i)
+            for (int c = 0; c < 2; ++c)
+                if (p.second.ps[i].chain == c || p.second.ps[i].chain == 2) {
+                    at[c] = p.second.pid[i];
+                    a.done_target[c] = kEpiWarpsPublic * p.second.ps[i].valid;
+                }
+        faux.push_back(a);
+        fcalls.push_back(call_of(p.first));
+        flast.push_back(at);
     }
     // Stage the tables.
     size_t o_aux = take(sizeof(AuxRec) * aux.size()), o_calls = take(sizeof(CallRec) * calls.size());
@@ -606,6 +621,9 @@ svt_status issue_window(svt_ctx *ctx, ServeState *s, int sms)
     const size_t o_n = take(sizeof(int) * (probs.size() + 1));  // completion counters, tile counter
     if (used > kRingSlotBytes)
         return SVT_ERR_OOM;
+    for (size_t i = 0; i < faux.size(); ++i)
+        for (int c = 0; c < 2; ++c)
+            faux[i].done[c] = flast[i][c] >= 0 ? reinterpret_cast<const int *>(d + o_n) + flast[i][c] : nullptr;
     std::memcpy(h + o_aux, aux.data(), sizeof(AuxRec) * aux.size());
     std::memcpy(h + o_calls, calls.data(), sizeof(CallRec) * calls.size());
     std::memcpy(h + o_faux, faux.data(), sizeof(AuxRec) * faux.size());
@@ -636,6 +654,7 @@ svt_status issue_window(svt_ctx *ctx, ServeState *s, int sms)
         L.dep_wait_ns = ctx->dbg_wait_ns;
         L.done = reinterpret_cast<int *>(d + o_n);
         L.tile_counter = L.done + probs.size();
+        L.shared = 1;
         if (tc_gemm_launch_fused(L, s->win_bn, tiles, sms, st) != cudaSuccess)
             return SVT_ERR_CUDA;
         ++launched;
@@ -659,17 +678,17 @@ svt_status issue_window(svt_ctx *ctx, ServeState *s, int sms)
             r->state = 3;
         }
     }
-    if (!fin.empty()) {
-        if (grouped_finalize_launch(A(o_faux), C(o_fcalls), (int)fin.size(), st) != cudaSuccess)
+    if (!faux.empty()) {
+        if (grouped_finalize_launch(A(o_faux), C(o_fcalls), (int)faux.size(), st) != cudaSuccess)
             return SVT_ERR_CUDA;
         ++launched;
-        for (Request *r : fin) {
-            r->pc += 1;
-            if (plan_status_copy(ctx, *r->plan, &s->h_status[r->slot], st) != SVT_OK ||
-                cudaEventRecord(s->events[r->slot], st) != cudaSuccess)
-                return SVT_ERR_CUDA;
-            r->state = 3;
-        }
+    }
+    for (Request *r : fin) {
+        r->pc += 1;
+        if (plan_status_copy(ctx, *r->plan, &s->h_status[r->slot], st) != SVT_OK ||
+            cudaEventRecord(s->events[r->slot], st) != cudaSuccess)
+            return SVT_ERR_CUDA;
+        r->state = 3;
     }
     if (cudaEventRecord(s->ring_ev[k], st) != cudaSuccess)
         return SVT_ERR_CUDA;
@@ -1010,9 +1029,6 @@ svt_status build_batch(svt_ctx *ctx, ServeState *s, const svt_matrix *mats, int 
     bp->blocks_split = blk_s;
     bp->d_aux = reinterpret_cast<AuxRec *>(tbase + take(sizeof(AuxRec) * count));
     bp->d_calls = reinterpret_cast<CallRec *>(tbase + take(sizeof(CallRec) * count));
-    bp->tables.emplace_back(bp->d_aux, std::vector<uint8_t>(
-                                           reinterpret_cast<uint8_t *>(aux.data()),
-                                           reinterpret_cast<uint8_t *>(aux.data() + count)));
     // One persistent launch for every product of every matrix: stage-major order
     // (stage k of all matrices, then stage k + 1), with the dependencies between each
     // matrix's own products.
@@ -1063,6 +1079,14 @@ svt_status build_batch(svt_ctx *ctx, ServeState *s, const svt_matrix *mats, int 
     int *counters = reinterpret_cast<int *>(tbase + take(sizeof(int) * (probs.size() + 1)));
     if (toff > batch_table_bytes(count, r))
         return SVT_ERR_OOM;
+    for (int i = 0; i < count; ++i) {  // the combine waits for all other products of its matrix
+        aux[i].done[0] = counters + pids[i].back();
+        aux[i].done_target[0] = kEpiWarpsPublic * ps[i].back().valid;
+        aux[i].last = 1;
+    }
+    bp->tables.emplace_back(bp->d_aux, std::vector<uint8_t>(
+                                           reinterpret_cast<uint8_t *>(aux.data()),
+                                           reinterpret_cast<uint8_t *>(aux.data() + count)));
     bp->tables.emplace_back(dp, std::vector<uint8_t>(
                                     reinterpret_cast<uint8_t *>(probs.data()),
                                     reinterpret_cast<uint8_t *>(probs.data() + probs.size())));
@@ -1079,6 +1103,7 @@ svt_status build_batch(svt_ctx *ctx, ServeState *s, const svt_matrix *mats, int 
         L.dep_wait_ns = ctx->dbg_wait_ns;
         L.done = counters;
         L.tile_counter = counters + probs.size();
+        L.shared = 1;
         bp->launches.push_back(L);
         bp->tiles.push_back(total);
         bp->bns.push_back(bn);
@@ -1289,6 +1314,7 @@ svt_status svt_batch(svt_ctx_t ctx, const svt_matrix *mats, int count, void *str
     if (same && total + batch_table_bytes(count, res[0]) <= ctx->ws_bytes) {
         BatchKey key;
         key.r = res[0];
+        key.wait_ns = ctx->dbg_wait_ns;
         key.bn = (res[0].tile == 128 || res[0].tile == 256)
                      ? res[0].tile
                      : batch_bn(mats, count, res[0], ctx->num_sms);

@@ -171,6 +171,10 @@ struct TcLaunch {
     // Limit of the waits on other tiles' results (dependency counters), ns; 0: the
     // kernel's default. Set from the context's SVT_DEBUG_WAIT_LIMIT_NS.
     unsigned long long dep_wait_ns;
+    // Fused launches: the problems belong to several solves, each with its own status word. A
+    // wait that gives up then sets none of them; what it left unfinished is found from the
+    // completion counters (grouped_finalize_kernel).
+    int shared;
 };
 
 // One product of the FP64 SIMT path: D = L R^T, L M x K (ldl), R N x K (ldr).
@@ -244,6 +248,12 @@ struct AuxRec {
     void *xt_hi, *xt_lo;             // transposed copy
     int64_t ld_t;
     int blk_reduce, blk_split;       // first block of this matrix in the grouped grids
+    // Finalize: the completion counters of the last product of each of this solve's chains in
+    // the launch before it, and the counts that mean "complete" (null: nothing to check); last:
+    // the solve ends with that launch.
+    const int *done[2];
+    int done_target[2];
+    int last;
 };
 
 // Grouped memory-bound kernels over `count` matrices (records and call table in
