@@ -987,8 +987,8 @@ constexpr int kRingTiles = 4;  // fused launches: tiles in flight between the ro
 // epilogue's scales and what the producer and the MMA issuer would otherwise load from the
 // problem table between two tiles.
 struct RingTile {
-    int tile;  // index in the launch (-1: no more tiles)
-    int prob;  // -1: nothing to compute
+    int kblocks;  // of a segment (-1: no more tiles)
+    int prob;     // -1: nothing to compute
     int tm, tn;
     float alpha, beta, gamma;
     int geom;  // see pack_geom
@@ -996,25 +996,29 @@ struct RingTile {
 
 constexpr int kMaxMaps = 2;  // tensor maps of an operand: hi and lo part
 
-// k-blocks of a segment in bits 0..15 (K < 2^21), segments in 16..17, their L and R parts in
-// 18..20 and 21..23, e4m3 operands in 24, "the operands' dependencies are met" in 25.
-constexpr int kGeomReady = 1 << 25;
+// k-blocks of a segment: one is a 128-byte swizzle row, 64 BF16 or 128 e4m3 elements. (K up to
+// 2^30: no field of a packed word.)
+__device__ __forceinline__ int seg_kblocks(const TcProblem &P)
+{
+    const int kshift = P.fp8 ? 7 : 6;
+    return (P.K + (1 << kshift) - 1) >> kshift;
+}
+
+// Segments in bits 0..1, their L and R parts in 2..4 and 5..7, e4m3 operands in 8, "the operands'
+// dependencies are met" in 9.
+constexpr int kGeomReady = 1 << 9;
 __device__ __forceinline__ int pack_geom(const TcProblem &P)
 {
-    // A k-block is one 128-byte swizzle row: 64 BF16 or 128 e4m3 elements.
-    const int kshift = P.fp8 ? 7 : 6;
-    int g = (P.K + (1 << kshift) - 1) >> kshift;
-    g |= P.nseg << 16 | (P.fp8 ? 1 << 24 : 0);
+    int g = P.nseg | (P.fp8 ? 1 << 8 : 0);
 #pragma unroll
     for (int k = 0; k < 3; ++k)
-        g |= P.segL[k] << (18 + k) | P.segR[k] << (21 + k);
+        g |= P.segL[k] << (2 + k) | P.segR[k] << (5 + k);
     return g;
 }
-__device__ __forceinline__ int geom_kblocks(int g) { return g & 0xffff; }
-__device__ __forceinline__ int geom_segs(int g) { return (g >> 16) & 3; }
-__device__ __forceinline__ int geom_l(int g, int sg) { return (g >> (18 + sg)) & 1; }
-__device__ __forceinline__ int geom_r(int g, int sg) { return (g >> (21 + sg)) & 1; }
-__device__ __forceinline__ bool geom_fp8(int g) { return (g >> 24) & 1; }
+__device__ __forceinline__ int geom_segs(int g) { return g & 3; }
+__device__ __forceinline__ int geom_l(int g, int sg) { return (g >> (2 + sg)) & 1; }
+__device__ __forceinline__ int geom_r(int g, int sg) { return (g >> (5 + sg)) & 1; }
+__device__ __forceinline__ bool geom_fp8(int g) { return (g >> 8) & 1; }
 
 // k-blocks per pipeline slot (one pair of barriers). With 128 x 64 tiles a k-block's four MMAs take
 // 134 cycles, while the waits, the vote and the branches of one round of the producer's and of the
@@ -1161,7 +1165,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
                     tc = tile_coord<BN, TILE_ROWS, STRIPS>(L.gtab[prob], prob, t - start);
                 }
                 EpiScales sc{1.f, 0.f, 0.f};
-                int geom = 0;
+                int geom = 0, kblocks = 0;
                 bool ok = true;
                 if (tc.valid) {
                     const TcProblem &P = L.gtab[tc.prob];
@@ -1178,6 +1182,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
                         prefetch_tensormap(&P.mapR[lane]);
                     }
                     geom = pack_geom(P);
+                    kblocks = seg_kblocks(P);
                     // Operands are results of earlier problems. Strip launches wait here until
                     // the strips this tile reads are complete (L: the strip of this tile's row,
                     // R: of its column), and so do tiles whose scales come from a norm. Other
@@ -1228,8 +1233,9 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
                     t = -1;
                     tc.valid = false;
                 }
-                const int ent[8] = {t, tc.valid ? tc.prob : -1, tc.tm, tc.tn, __float_as_int(sc.alpha),
-                                    __float_as_int(sc.beta), __float_as_int(sc.gamma), geom};
+                const int ent[8] = {t < 0 ? -1 : kblocks, tc.valid ? tc.prob : -1, tc.tm, tc.tn,
+                                    __float_as_int(sc.alpha), __float_as_int(sc.beta),
+                                    __float_as_int(sc.gamma), geom};
                 int word = ent[0];  // lane k < 8 writes word k
 #pragma unroll
                 for (int q = 1; q < 8; ++q)
@@ -1266,7 +1272,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
             for (;;) {
                 if (!wait_bar<PAIR>(&rfull[ri], rphase, abort_flag, status0, kWaitTimeoutNs))
                     break;
-                const int t = ring[ri].tile, prob = ring[ri].prob, tm = ring[ri].tm, tn = ring[ri].tn;
+                const int kblocks = ring[ri].kblocks, prob = ring[ri].prob, tm = ring[ri].tm, tn = ring[ri].tn;
                 if (prob >= 0) {
                     const TcProblem &P = prob_at(L, prob);
                     const int pid = P.pid;
@@ -1291,7 +1297,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
                     ri = 0;
                     rphase ^= 1u;
                 }
-                if (t < 0)
+                if (kblocks < 0)
                     break;
             }
         }
@@ -1305,11 +1311,11 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
         uint32_t rphase = 0;
         for (int t = t_first; ok; t += t_step) {
             TileCoord tc;
-            int geom = 0;
+            int geom = 0, kblocks = 0;
             if (CHAIN) {
                 if (!wait_warp<PAIR>(&rfull[ri], rphase, abort_flag, status0, kWaitTimeoutNs))
                     break;
-                t = warp_uniform(ring[ri].tile);
+                kblocks = warp_uniform(ring[ri].kblocks);
                 tc.prob = warp_uniform(ring[ri].prob);
                 tc.tm = warp_uniform(ring[ri].tm);
                 tc.tn = warp_uniform(ring[ri].tn);
@@ -1324,7 +1330,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
                 }
                 // The scheduler takes the next tile once this one can start: a CTA holding two
                 // tiles that wait would keep work from CTAs that are idle.
-                if (t < 0)
+                if (kblocks < 0)
                     break;
                 if (!tc.valid && (!PAIR || leader) && elect_one())
                     mbar_arrive(ptaken);
@@ -1336,9 +1342,11 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
             if (!tc.valid)
                 continue;
             const TcProblem &P = prob_at(L, tc.prob);
-            if (!CHAIN)
+            if (!CHAIN) {
                 geom = pack_geom(P);
-            const int kshift = geom_fp8(geom) ? 7 : 6, kblocks = geom_kblocks(geom);
+                kblocks = seg_kblocks(P);
+            }
+            const int kshift = geom_fp8(geom) ? 7 : 6;
             const int row0 = (PAIR ? 2 * tc.tm + (int)rank : tc.tm) * kBM;
             const int col0 = tc.tn * BN + (int)rank * B_ROWS;
             if (CHAIN) {
@@ -1424,11 +1432,11 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
         uint32_t rphase = 0;
         for (int t = t_first; ok; t += t_step) {
             TileCoord tc;
-            int geom = 0;
+            int geom = 0, kblocks = 0;
             if (CHAIN) {
                 if (!wait_warp<false>(&rfull[ri], rphase, abort_flag, status0, kWaitTimeoutNs))
                     break;
-                t = warp_uniform(ring[ri].tile);
+                kblocks = warp_uniform(ring[ri].kblocks);
                 tc.prob = warp_uniform(ring[ri].prob);
                 tc.tm = warp_uniform(ring[ri].tm);
                 tc.tn = warp_uniform(ring[ri].tn);
@@ -1441,14 +1449,16 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
                     ri = 0;
                     rphase ^= 1u;
                 }
-                if (t < 0)
+                if (kblocks < 0)
                     break;
             } else {
                 if (t >= total)
                     break;
                 tc = decode_tile<BN, TILE_ROWS, STRIPS>(L, t);
-                if (tc.valid)
+                if (tc.valid) {
                     geom = pack_geom(prob_at(L, tc.prob));
+                    kblocks = seg_kblocks(prob_at(L, tc.prob));
+                }
             }
             if (!tc.valid)
                 continue;
@@ -1463,7 +1473,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
             auto k_loop = [&](auto f8_tag) -> bool {
                 constexpr bool F8 = decltype(f8_tag)::value;
                 constexpr uint32_t id = F8 ? idesc_e4m3(TILE_ROWS, BN) : idesc_bf16(TILE_ROWS, BN);
-                const int kblocks = geom_kblocks(geom), segs = geom_segs(geom);
+                const int segs = geom_segs(geom);
                 uint32_t acc = 0;
                 for (int sg = 0; sg < segs; ++sg) {
                     for (int left = kblocks, count; left > 0; left -= count) {
@@ -1555,7 +1565,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
             if (CHAIN) {
                 if (!wait_bar<PAIR>(&rfull[ri], rphase, abort_flag, status0, kWaitTimeoutNs))
                     break;
-                t = ring[ri].tile;
+                const bool end = ring[ri].kblocks < 0;
                 tc.prob = ring[ri].prob;
                 tc.tm = ring[ri].tm;
                 tc.tn = ring[ri].tn;
@@ -1569,7 +1579,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
                     ri = 0;
                     rphase ^= 1u;
                 }
-                if (t < 0)
+                if (end)
                     break;
             } else {
                 if (t >= total)
