@@ -1,5 +1,6 @@
 // Launches of the product kernel (gemm_tc_kernel.cuh) by tile-width code.
 #include <algorithm>
+#include <cstring>
 
 #include "svt_internal.h"
 
@@ -34,6 +35,13 @@ cudaError_t tc_gemm_launch_fused(const TcLaunch &l, int bn, int total_tiles, int
         return bn == kBnPair ? tc_launch_pair(g, true, true, total_tiles, num_sms, s)
                              : cudaErrorInvalidValue;
     return launch_width(g, true, bn, total_tiles, num_sms, s);
+}
+
+cudaError_t tc_gemm_load_fused(int bn, int num_sms)
+{
+    TcLaunch none;
+    std::memset(&none, 0, sizeof(none));
+    return launch_width(none, true, bn, 0, num_sms, nullptr);
 }
 
 int tc_num_tiles(const TcProblem &p, int bn)

@@ -237,6 +237,7 @@ struct ServeState {
     bool ring_busy[kRing] = {};
     int ring_next = 0;
     int win_bn = 0;  // tile-width code of the windows' products
+    bool widths_loaded = false;       // the windows' kernels, before the first large request
     uint64_t windows = 0;
     FILE *metrics = nullptr;          // per-request JSON lines (svt_serve_metrics)
 };
@@ -745,6 +746,15 @@ bool tick(svt_ctx *ctx, ServeState *s)
             break;
         }
         s->bigq.erase(pick);
+        // Windows change their tile width with the requests. The first launch of a width would load
+        // its kernel, which waits for the large lane's launches in flight and held the scheduler for
+        // 4.4 to 7.0 ms beside an 8192 x 4096 FP32 request. Before the first of them it takes 0.35 ms
+        // a width, once a process. (A failure shows at the launch.)
+        if (!s->widths_loaded)
+            for (const BatchCost &b : kBatchCosts)
+                if (tc_gemm_load_fused(b.bn, ctx->num_sms) != cudaSuccess)
+                    cudaGetLastError();
+        s->widths_loaded = true;
         const double t0 = trace_file() ? now_ms() : 0.0;
         int slot = 0;
         while (s->slot_used[slot])

@@ -202,6 +202,9 @@ cudaError_t tc_gemm_launch(const TcLaunch &l, int bn, int num_sms, cudaStream_t 
 // strips: the table carries per-strip dependencies (bn kBnPair only).
 cudaError_t tc_gemm_launch_fused(const TcLaunch &l, int bn, int total_tiles, int num_sms,
                                  cudaStream_t s, bool strips = false);
+// Loads the kernel of one tile-width code's fused launches without a launch. A kernel is otherwise
+// loaded by its first launch, which then may wait for all work on the device.
+cudaError_t tc_gemm_load_fused(int bn, int num_sms);
 // One launch of the product kernel in one tile configuration (each in its own translation unit).
 cudaError_t tc_launch_64(const TcLaunch &l, bool chain, int total_tiles, int num_sms, cudaStream_t s);
 cudaError_t tc_launch_128(const TcLaunch &l, bool chain, int total_tiles, int num_sms, cudaStream_t s);
