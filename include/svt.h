@@ -550,7 +550,9 @@ svt_status svt_ctx_profile_read_ex(svt_ctx_t ctx, double *tc_ms, double *tc_flop
  * three (128 x 64, or pairs on 256 x 128), that tile stands for 128 x 128, here and
  * wherever a stored or imported 128 is used. The choice is stored in the context; later svt_polar /
  * svt_polar_ex calls with the same shape and options and tile = 0 use it. Y
- * receives A_tau. Synchronises `stream`.
+ * receives A_tau. Synchronises `stream`. Shapes that run as one launch in shared memory (both
+ * sides at most 128, the default pipeline) have no mode to choose: Y receives A_tau, nothing is
+ * timed or stored, and an imported choice for such a shape has no effect.
  * Errors: as svt_polar_ex; SVT_ERR_BUSY while serving requests are in flight.
  * The FP64 tier has no tile choice (returns SVT_OK without work).
  */

@@ -1703,6 +1703,16 @@ svt_status svt_autotune(svt_ctx_t ctx, const float *A, int64_t m, int64_t n, int
         return SVT_ERR_CUDA;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     CallArgs a{A, lda, tau, Y, ldy, nullptr};
+    r.tile = 0;  // the later calls that a choice serves have tile = 0
+    if (use_small(ctx, m, n, r)) {  // they run as one launch, whatever is stored: nothing to choose
+        Plan *plan = nullptr;
+        st = get_plan(ctx, m, n, r, 0, ctx->ws_bytes, &plan, kSmallPlan);
+        if (st == SVT_OK)
+            st = run_plan(ctx, *plan, a, s);
+        if (st == SVT_OK && cudaStreamSynchronize(s) != cudaSuccess)
+            st = SVT_ERR_CUDA;
+        return st;
+    }
     const int widths[3] = {128, 256, kBnPair};
     std::vector<int> choice;
     if (r.fuse) {
