@@ -465,6 +465,15 @@ svt_status svt_debug_gemm_e4m3(svt_ctx_t ctx, const void *L, const void *R, int6
                                int64_t K, int64_t ldl, int64_t ldr, float *D, int64_t ldd, int tile,
                                void *stream);
 
+/* Diagnostic (used by the tests): the tiles that a call would run its products on, in *mode,
+ * for these shapes and options and the context's tuning. count = 1: svt_polar_ex; more: one
+ * svt_batch. Pointers, strides and tau of `mats` are not looked at.
+ *   64, 128, 256: one CTA per 128 x 64, 128 x 128 or 128 x 256 tile; 384, 512: a pair of CTAs
+ *   per 256 x 128 or 256 x 256 tile; 1: one launch in shared memory; 0: no common tile (the
+ *   FP64 tier, opt.fuse = 0, batches that run matrix by matrix).
+ * Errors: SVT_ERR_INVALID, SVT_ERR_UNSUPPORTED (options). */
+svt_status svt_debug_tile_mode(svt_ctx_t ctx, const svt_matrix *mats, int count, int *mode);
+
 /* Failure-path check of the device-side bounded waits: launches the product kernel
  * (fused form) on a one-tile table whose tile waits for its own completion, so the
  * wait runs out (about 2 s); the kernel records SVT_ERR_TIMEOUT in *d_status (device

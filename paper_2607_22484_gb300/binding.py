@@ -46,6 +46,7 @@ EXPORTS = [
     "svt_ctx_profile_read_ex", "svt_debug_wait_timeout", "svt_polar_f64", "svt_serve_cancel",
     "svt_serve_metrics", "svt_ctx_debug", "svt_tuning_export", "svt_tuning_import",
     "svt_polar_fp8", "svt_workspace_bytes_fp8", "svt_debug_gemm_e4m3",
+    "svt_debug_tile_mode",
 ]
 NOALLOC_SCRATCH_BYTES = 32 << 20
 
@@ -167,6 +168,7 @@ def lib():
                                          ctypes.POINTER(ctypes.c_int),
                                          ctypes.POINTER(ctypes.c_double)]
         L.svt_debug_wait_timeout.argtypes = [vp, vp, vp]
+        L.svt_debug_tile_mode.argtypes = [vp, ctypes.POINTER(Matrix), i32, ctypes.POINTER(ctypes.c_int)]
         L.svt_ctx_launch_count.argtypes = [vp]
         L.svt_ctx_launch_count.restype = ctypes.c_uint64
         L.svt_ctx_profile.argtypes = [vp, i32]
@@ -627,6 +629,17 @@ class Context:
                                             int(tile), ctypes.c_void_p(_stream_ptr(stream))),
                "svt_debug_gemm_bf16_ex")
         return D
+
+    def tile_mode(self, shapes, **opts) -> int:
+        """The tiles that polar() (one shape) or one batch() call (several) would run on
+        (svt_debug_tile_mode)."""
+        arr = (Matrix * len(shapes))()
+        for x, (m, n) in zip(arr, shapes):
+            x.m, x.n, x.opt = m, n, make_options(**opts)
+        mode = ctypes.c_int(-1)
+        _check(lib().svt_debug_tile_mode(self.handle, arr, len(shapes), ctypes.byref(mode)),
+               "svt_debug_tile_mode")
+        return mode.value
 
     def _matrix(self, A, tau, out, status, opts):
         import torch

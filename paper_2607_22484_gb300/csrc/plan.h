@@ -310,6 +310,9 @@ svt_status plan_status_copy(svt_ctx *ctx, const Plan &P, int *host_dst, cudaStre
 // tile width), as svt_polar_ex looks it up (under ctx->mu).
 svt_status plan_for_solve(svt_ctx *ctx, int64_t m, int64_t n, const Resolved &r, Plan **out,
                           std::shared_ptr<Plan> *keep = nullptr);
+// Tile-width code of the products of such a solve (kSmallPlan: one launch in shared memory; 0: the
+// FP64 tier, or launch by launch).
+int solve_tile_code(const svt_ctx *ctx, int64_t m, int64_t n, const Resolved &r);
 // Refresh the plan's fused-launch table in the workspace from its host image (async on s).
 svt_status upload_fused_table(svt_ctx *ctx, Plan &P, cudaStream_t s);
 // A solve split into consecutive parts of about `target` tensor flops each (at most

@@ -1229,9 +1229,11 @@ bool serve_busy(svt_ctx *ctx)
 
 namespace {
 
-// Tile width of a grouped batch whose options leave it open.
-int batch_bn(const svt_matrix *mats, int count, const Resolved &r, int sms)
+// Tile width of a grouped batch: its options', or from the cost model.
+int batch_tile(const svt_matrix *mats, int count, const Resolved &r, int sms)
 {
+    if (r.tile == 128 || r.tile == 256)
+        return r.tile;
     int best = 0;
     double least = 0.0;
     for (const BatchCost &b : kBatchCosts) {
@@ -1325,9 +1327,7 @@ svt_status svt_batch(svt_ctx_t ctx, const svt_matrix *mats, int count, void *str
         BatchKey key;
         key.r = res[0];
         key.wait_ns = ctx->dbg_wait_ns;
-        key.bn = (res[0].tile == 128 || res[0].tile == 256)
-                     ? res[0].tile
-                     : batch_bn(mats, count, res[0], ctx->num_sms);
+        key.bn = batch_tile(mats, count, res[0], ctx->num_sms);
         for (int i = 0; i < count; ++i) {
             key.shapes.push_back(mats[i].m);
             key.shapes.push_back(mats[i].n);
@@ -1400,6 +1400,25 @@ svt_status svt_batch(svt_ctx_t ctx, const svt_matrix *mats, int count, void *str
             cudaStreamWaitEvent(cs, s->events[1 + i], 0) != cudaSuccess)
             return SVT_ERR_CUDA;
     }
+    return SVT_OK;
+}
+
+svt_status svt_debug_tile_mode(svt_ctx_t ctx, const svt_matrix *mats, int count, int *mode)
+{
+    if (!ctx || !mats || count <= 0 || !mode)
+        return SVT_ERR_INVALID;
+    for (int i = 0; i < count; ++i)
+        if (mats[i].m <= 0 || mats[i].n <= 0)
+            return SVT_ERR_INVALID;
+    std::vector<Resolved> res;
+    bool same = false;
+    if (svt_status rs = resolve_all(mats, count, res, &same))
+        return rs;
+    std::lock_guard<std::mutex> g(ctx->mu);
+    if (count == 1)
+        *mode = solve_tile_code(ctx, mats[0].m, mats[0].n, res[0]);
+    else
+        *mode = same ? batch_tile(mats, count, res[0], ctx->num_sms) : 0;
     return SVT_OK;
 }
 

@@ -1410,22 +1410,37 @@ static int narrow_mode(const svt_ctx *ctx, int64_t m, int64_t n, const Resolved 
     return a == kBn64 || a == kBnPair128 ? a : 128;
 }
 
+// force_bn of the plan that a solve runs with.
+static int solve_mode(const svt_ctx *ctx, int64_t m, int64_t n, const Resolved &r)
+{
+    if (r.tile)
+        return r.tile;
+    if (use_small(ctx, m, n, r))
+        return kSmallPlan;
+    const auto t = ctx->tuning.find(tune_key(m, n, r));
+    if (t == ctx->tuning.end())
+        return 0;
+    const bool all128 = std::all_of(t->second.begin(), t->second.end(), [](int w) { return w == 128; });
+    return r.fuse && all128 ? narrow_mode(ctx, m, n, r) : -1;
+}
+
 svt_status plan_for_solve(svt_ctx *ctx, int64_t m, int64_t n, const Resolved &r, Plan **out,
                           std::shared_ptr<Plan> *keep)
 {
-    int fbn = 0;
-    if (r.tile) {
-        fbn = r.tile;
-    } else if (use_small(ctx, m, n, r)) {
-        fbn = kSmallPlan;
-    } else {
-        const auto t = ctx->tuning.find(tune_key(m, n, r));
-        if (t != ctx->tuning.end()) {
-            const bool all128 = std::all_of(t->second.begin(), t->second.end(), [](int w) { return w == 128; });
-            fbn = r.fuse && all128 ? narrow_mode(ctx, m, n, r) : -1;
-        }
-    }
-    return get_plan(ctx, m, n, r, 0, ctx->ws_bytes, out, fbn, keep);
+    return get_plan(ctx, m, n, r, 0, ctx->ws_bytes, out, solve_mode(ctx, m, n, r), keep);
+}
+
+int solve_tile_code(const svt_ctx *ctx, int64_t m, int64_t n, const Resolved &r)
+{
+    if (r.prec == SVT_FP64 || !r.fuse)
+        return 0;
+    const int mode = solve_mode(ctx, m, n, r);
+    if (mode > 0)
+        return mode;
+    if (mode == 0)
+        return fused_auto_width(m, n, r, ctx->num_sms);
+    const std::vector<int> &w = ctx->tuning.at(tune_key(m, n, r));  // one width, unless imported
+    return std::equal(w.begin() + 1, w.end(), w.begin()) ? w.front() : 0;
 }
 
 svt_status plan_status_copy(svt_ctx *ctx, const Plan &P, int *host_dst, cudaStream_t s)
