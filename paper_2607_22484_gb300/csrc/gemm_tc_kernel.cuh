@@ -220,7 +220,7 @@ __device__ __forceinline__ bool aligned16(const void *p)
 struct EpiHot {
     const void *c0, *c1;
     void *o0, *o1, *t0, *t1;
-    const CUtensorMap *maps;  // mapO[0..1], mapT[0..1], mapU[0..1] of the problem
+    const CUtensorMap *maps;  // mapO[0..1], mapT[0..1] of the problem
     double *norm_acc;
     const double *diag, *dss;
     int64_t ldc, ldo, ldt;
@@ -1718,8 +1718,8 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
                                 const CUtensorMap *m = h.maps;
                                 const bool both = Spec::mirror && !diag;
                                 if (unit) {
-                                    tma_store_2d(&m[4], x, y, stage_buf);
-                                    tma_store_2d(&m[5], y, x, stage_buf + kStgMirror64);
+                                    tma_store_2d(&m[1], x, y, stage_buf);  // (u_tma's maps)
+                                    tma_store_2d(&m[3], y, x, stage_buf + kStgMirror64);
                                 } else {
                                     const CUtensorMap *mm = Spec::sym ? m : m + 2;
                                     tma_store_2d(&m[0], x, y, stage_buf);
@@ -1807,9 +1807,8 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
     }
 }
 
-static_assert(offsetof(TcProblem, mapT) == offsetof(TcProblem, mapO) + 2 * sizeof(CUtensorMap) &&
-                  offsetof(TcProblem, mapU) == offsetof(TcProblem, mapT) + 2 * sizeof(CUtensorMap),
-              "the epilogue addresses mapO, mapT and mapU as one array");
+static_assert(offsetof(TcProblem, mapT) == offsetof(TcProblem, mapO) + 2 * sizeof(CUtensorMap),
+              "the epilogue addresses mapO and mapT as one array");
 
 template <int BN, int STAGES, bool PAIR>
 constexpr int smem_bytes()

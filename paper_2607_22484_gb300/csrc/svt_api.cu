@@ -142,10 +142,10 @@ void attach_store_maps(TcProblem &p)
     // 64-column units of a BF16 output: the mirror goes to the output itself (symmetric) or to
     // the transposed copy.
     p.u_tma = e.o_kind == O_PAIR ? 1 : 0;
-    if (e.o_kind == O_BF16 && p.o_tma && !e.o_trans && (p.sym || p.t_tma))
-        p.u_tma = encode_store_map(&p.mapU[0], e.o0, p.M, p.N, e.ldo, false, 64, 32) &&
-                  (p.sym ? encode_store_map(&p.mapU[1], e.o0, p.M, p.N, e.ldo, false, 32, 64)
-                         : encode_store_map(&p.mapU[1], e.t0, p.N, p.M, e.ldt, false, 32, 64));
+    if (e.o_kind == O_BF16 && p.o_tma && !e.o_trans && e.t_kind != O_PAIR && (p.sym || p.t_tma))
+        p.u_tma = encode_store_map(&p.mapO[1], e.o0, p.M, p.N, e.ldo, false, 64, 32) &&
+                  (p.sym ? encode_store_map(&p.mapT[1], e.o0, p.M, p.N, e.ldo, false, 32, 64)
+                         : encode_store_map(&p.mapT[1], e.t0, p.N, p.M, e.ldt, false, 32, 64));
 }
 
 

@@ -116,10 +116,11 @@ struct TcProblem {
     CUtensorMap mapR[2];             // R operands, box 64 x BN
     CUtensorMap mapO[2];             // output hi/lo (or FP32), box 32 x 32, for TMA stores
     CUtensorMap mapT[2];             // transposed copy hi/lo, box 32 x 32
-    CUtensorMap mapU[2];             // BF16 output's 64-column units: in place (box 64 x 32), and
-                                     // mirrored or as the transposed copy (box 32 x 64)
+    // A BF16 output has no lo parts: with u_tma, mapO[1] and mapT[1] are those of its 64-column
+    // units, in place (box 64 x 32) and mirrored or as the transposed copy (box 32 x 64). (Maps
+    // of their own would make the table, which counts as workspace, 32 KiB longer at 20 steps.)
     int o_tma, t_tma;                // 1: store through mapO / mapT
-    int u_tma;                       // 1: mapU holds what a BF16 output's units need (or pairs,
+    int u_tma;                       // 1: the maps have what a BF16 output's units need (or pairs,
                                      // which have no units)
     int patch, call_idx;             // grouped launches: fields taken from calls[call_idx]
     // Fused (chained) launches: completion counter index of this problem, and the
