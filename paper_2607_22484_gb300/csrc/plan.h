@@ -150,8 +150,9 @@ struct Plan {
     }
     int tc_launches_per_solve = 0;
     int kernel_launches = 0;
-    int force_bn = 0;               // 0: tile width per launch; 128 / 256: fixed (grouped batches);
-                                    // -1: per-launch widths from bn_choice (autotuned)
+    int force_bn = 0;               // 0: tile width per launch; a tile-width code: fixed;
+                                    // -1: per-launch widths from bn_choice (autotuned);
+                                    // kSmallPlan: one launch in shared memory
     std::vector<int> bn_choice;     // tile width of each product launch (autotuned plans)
     // One-launch solve of a one-tile matrix (kSmallPlan): no product table, no workspace.
     bool small = false;

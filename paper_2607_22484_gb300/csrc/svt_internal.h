@@ -29,7 +29,8 @@ constexpr int kBK = 64;           // K per pipeline stage: one 128-byte swizzle 
 // output tile. kBnPair: a cluster of two CTAs per 256 x 256 tile
 // (tcgen05 cta_group::2), each CTA holding 128 x 256 of it and staging half of
 // the tile's R rows. kBnPair128: such a cluster per 256 x 128 tile; kBn64: one CTA per
-// 128 x 64 tile (these two are chosen by fused_auto_width, they are no option values).
+// 128 x 64 tile (these two are chosen by fused_auto_width and the batches' cost model, they are no
+// option values).
 constexpr int kBnPair = 512;
 constexpr int kBnPair128 = 384;
 constexpr int kBn64 = 64;
@@ -124,7 +125,8 @@ struct TcProblem {
                                      // which have no units)
     int patch, call_idx;             // grouped launches: fields taken from calls[call_idx]
     // Fused (chained) launches: completion counter index of this problem, and the
-    // problems whose results it reads with the counts that mean "complete".
+    // problems that it waits for (whose results it reads, or which read what it
+    // overwrites) with the counts that mean "complete".
     int pid;
     int dep[2];
     int dep_target[2];
